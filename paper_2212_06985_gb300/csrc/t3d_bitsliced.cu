@@ -22,27 +22,12 @@ namespace {
 
 constexpr int kThreads = 256;
 
-struct SiteWordGrid {
-    dim3 grid, block;
-};
-
 // Words per block row: 32, or the next power of two >= words for tiny batches.
 int row_words(int64_t words)
 {
     int tx = 32;
     while (tx > 1 && tx / 2 >= words) tx /= 2;
     return tx;
-}
-
-// x = words (coalesced), y = sites (layout conversion kernels).
-SiteWordGrid site_word_grid(int64_t n_sites, int64_t words)
-{
-    int tx = row_words(words);
-    int ty = kThreads / tx;
-    SiteWordGrid g;
-    g.block = dim3(tx, ty, 1);
-    g.grid = dim3((unsigned)((n_sites + ty - 1) / ty), (unsigned)((words + tx - 1) / tx), 1);
-    return g;
 }
 
 // Blocks an item needs for a (sites x words) tiling with rows of tx words.
@@ -681,29 +666,153 @@ __global__ void k_flip_finish(const __grid_constant__ ItemDesc d, int n_apply, i
         d.s[i] = 0;
 }
 
-__global__ void k_pack(int64_t n_bits, int64_t n_samples, int64_t W, const uint8_t* __restrict__ bits,
-                       uint64_t* __restrict__ words)
+// Layout conversion, bits [sample][n_bits] bytes <-> words [n_bits][W].  HBM-bound: a byte
+// per bit crosses once, so the tile is shaped for both sides' runs.  A block takes
+// kLayoutCols bit columns of tw (up to 16) words; a warp takes the 64 samples of one word,
+// each lane four columns, so a sample's row is read (written) in 128-byte runs (four bytes a
+// lane; rows that are not 4-byte aligned go byte by byte in 32-byte runs) and the word
+// rows in runs of 8 tw bytes through a shared-memory transposition.  Eight samples' bits of a
+// lane's four columns share one register (byte k holds column k), so a sample costs a mask, a
+// shift and an OR.  (The earlier one thread per (bit, word) read a byte every n_bits bytes:
+// L = 12, 20,000 samples, 104 MB of bytes, 351 us packing and 335 us unpacking.)
+constexpr int kLayoutCols = 128;
+constexpr int kLayoutWords = 16;
+constexpr int kLayoutPitch = kLayoutCols + 2;
+
+// Column of a lane's k-th byte within the tile.
+template <bool kVec>
+__device__ __forceinline__ int layout_col(int lane, int k) { return kVec ? 4 * lane + k : lane + 32 * k; }
+
+template <bool kVec>
+__global__ void __launch_bounds__(32 * kLayoutWords)
+k_pack(int64_t n_bits, int64_t n_samples, int64_t W, const uint8_t* __restrict__ bits, uint64_t* __restrict__ words,
+       int64_t col_tiles, int64_t tiles)
 {
-    int64_t w = (int64_t)blockIdx.y * blockDim.x + threadIdx.x;
-    int64_t i = (int64_t)blockIdx.x * blockDim.y + threadIdx.y;
-    if (w >= W || i >= n_bits) return;
-    uint64_t acc = 0;
-    for (int j = 0; j < 64; ++j) {
-        int64_t sample = w * 64 + j;
-        if (sample >= n_samples) break;
-        acc |= (uint64_t)(bits[sample * n_bits + i] & 1) << j;
+    __shared__ __align__(16) uint64_t tile[kLayoutWords * kLayoutPitch];
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, tw = blockDim.x >> 5;
+    for (int64_t b = blockIdx.x; b < tiles; b += gridDim.x) {
+        const int64_t wt = b / col_tiles, c0 = (b - wt * col_tiles) * kLayoutCols;
+        const int64_t w = wt * tw + wi;
+        const int64_t s0 = w * 64;
+        const int count = w < W ? (int)min((int64_t)64, n_samples - s0) : 0;
+        bool in[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) in[k] = c0 + layout_col<kVec>(lane, k) < n_bits;
+        const uint8_t* __restrict__ p = bits + s0 * n_bits + c0 + layout_col<kVec>(lane, 0);
+        // the four columns' bytes of sample j (kVec: n_bits is a multiple of 4, all or none)
+        auto row = [&](int j) -> uint32_t {
+            const uint8_t* q = p + j * n_bits;
+            if (kVec) return in[0] ? __ldcs(reinterpret_cast<const unsigned int*>(q)) : 0u;
+            uint32_t v = 0;
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (in[k]) v |= (uint32_t)__ldcs(q + 32 * k) << (8 * k);
+            return v;
+        };
+        uint32_t acc[8];
+        if (count == 64) {
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                acc[g] = 0;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) acc[g] |= (row(8 * g + j) & 0x01010101u) << j;
+            }
+        } else {
+#pragma unroll
+            for (int g = 0; g < 8; ++g) {
+                acc[g] = 0;
+                for (int j = 0; j < 8; ++j)
+                    if (8 * g + j < count) acc[g] |= (row(8 * g + j) & 0x01010101u) << j;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            // byte k of the eight registers, samples 0..7 lowest
+            const uint32_t pair = (uint32_t)(k | ((4 + k) << 4));
+            const uint32_t lo = __byte_perm(__byte_perm(acc[0], acc[1], pair), __byte_perm(acc[2], acc[3], pair), 0x5410);
+            const uint32_t hi = __byte_perm(__byte_perm(acc[4], acc[5], pair), __byte_perm(acc[6], acc[7], pair), 0x5410);
+            tile[wi * kLayoutPitch + layout_col<kVec>(lane, k)] = (uint64_t)lo | ((uint64_t)hi << 32);
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < kLayoutCols * tw; i += blockDim.x) {
+            const int c = i / tw, k = i - c * tw;
+            if (c0 + c < n_bits && wt * tw + k < W) words[(c0 + c) * W + wt * tw + k] = tile[k * kLayoutPitch + c];
+        }
+        __syncthreads();
     }
-    words[i * W + w] = acc;
 }
 
-__global__ void k_unpack(int64_t n_bits, int64_t n_samples, int64_t W, const uint64_t* __restrict__ words,
-                         uint8_t* __restrict__ bits)
+template <bool kVec>
+__global__ void __launch_bounds__(32 * kLayoutWords)
+k_unpack(int64_t n_bits, int64_t n_samples, int64_t W, const uint64_t* __restrict__ words, uint8_t* __restrict__ bits,
+         int64_t col_tiles, int64_t tiles)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t sample = blockIdx.y + (int64_t)gridDim.y * blockIdx.z;
-    if (i >= n_bits || sample >= n_samples) return;
-    bits[sample * n_bits + i] = (uint8_t)((words[i * W + sample / 64] >> (sample % 64)) & 1ULL);
+    __shared__ __align__(16) uint64_t tile[kLayoutWords * kLayoutPitch];
+    const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, tw = blockDim.x >> 5;
+    for (int64_t b = blockIdx.x; b < tiles; b += gridDim.x) {
+        const int64_t wt = b / col_tiles, c0 = (b - wt * col_tiles) * kLayoutCols;
+        for (int i = threadIdx.x; i < kLayoutCols * tw; i += blockDim.x) {
+            const int c = i / tw, k = i - c * tw;
+            if (c0 + c < n_bits && wt * tw + k < W) tile[k * kLayoutPitch + c] = words[(c0 + c) * W + wt * tw + k];
+        }
+        __syncthreads();
+        const int64_t w = wt * tw + wi, s0 = w * 64;
+        const int count = w < W ? (int)min((int64_t)64, n_samples - s0) : 0;
+        bool in[4];
+        uint64_t v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            in[k] = c0 + layout_col<kVec>(lane, k) < n_bits;
+            v[k] = count > 0 && in[k] ? tile[wi * kLayoutPitch + layout_col<kVec>(lane, k)] : 0;
+        }
+        uint8_t* __restrict__ p = bits + s0 * n_bits + c0 + layout_col<kVec>(lane, 0);
+#pragma unroll
+        for (int g = 0; g < 8; ++g) {
+            // byte g of the four columns' words side by side: bit j of each byte is sample 8 g + j
+            const uint32_t pair = (uint32_t)((g & 3) | ((4 + (g & 3)) << 4));
+            uint32_t h[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) h[k] = (uint32_t)(v[k] >> (g < 4 ? 0 : 32));
+            const uint32_t x = __byte_perm(__byte_perm(h[0], h[1], pair), __byte_perm(h[2], h[3], pair), 0x5410);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                if (8 * g + j >= count) break;
+                const uint32_t o = (x >> j) & 0x01010101u;
+                uint8_t* q = p + (8 * g + j) * n_bits;
+                if (kVec) {
+                    if (in[0]) *reinterpret_cast<uint32_t*>(q) = o;
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (in[k]) q[32 * k] = (uint8_t)(o >> (8 * k));
+                }
+            }
+        }
+        __syncthreads();
+    }
 }
+
+// Grid of the layout kernels: words per block (a warp each), column tiles, tiles in all.
+struct LayoutGrid {
+    int threads;
+    unsigned blocks;
+    int64_t col_tiles, tiles;
+};
+
+LayoutGrid layout_grid(int64_t n_bits, int64_t W)
+{
+    int tw = kLayoutWords;
+    while (tw > 1 && tw / 2 >= W) tw /= 2;
+    LayoutGrid g;
+    g.threads = 32 * tw;
+    g.col_tiles = (n_bits + kLayoutCols - 1) / kLayoutCols;
+    g.tiles = g.col_tiles * ((W + tw - 1) / tw);
+    g.blocks = (unsigned)std::min<int64_t>(g.tiles, 0x7fffffffLL);
+    return g;
+}
+
+// Four bytes of a row at a time: every sample's row starts 4-byte aligned.
+bool layout_vec(const void* bits, int64_t n_bits) { return n_bits % 4 == 0 && aligned(bits, 4); }
 
 }  // namespace
 
@@ -1149,9 +1258,13 @@ extern "C" t3d_status toric3d_pack(int64_t n_bits, int64_t n_samples, const uint
     T3D_TRY(check_words(words, "words"));
     int64_t W = words_for(n_samples);
     T3D_REQUIRE(W <= 65535LL * 32, "n_samples out of range");
-    auto g = site_word_grid(n_bits, W);
-    ProfScope prof(T3D_K_LAYOUT, as_stream(stream));
-    k_pack<<<g.grid, g.block, 0, as_stream(stream)>>>(n_bits, n_samples, W, bits, words);
+    const LayoutGrid g = layout_grid(n_bits, W);
+    cudaStream_t st = as_stream(stream);
+    ProfScope prof(T3D_K_LAYOUT, st);
+    if (layout_vec(bits, n_bits))
+        k_pack<true><<<g.blocks, g.threads, 0, st>>>(n_bits, n_samples, W, bits, words, g.col_tiles, g.tiles);
+    else
+        k_pack<false><<<g.blocks, g.threads, 0, st>>>(n_bits, n_samples, W, bits, words, g.col_tiles, g.tiles);
     T3D_LAUNCH_CHECK("pack");
     return T3D_OK;
 }
@@ -1164,12 +1277,13 @@ extern "C" t3d_status toric3d_unpack(int64_t n_bits, int64_t n_samples, const ui
     T3D_REQUIRE(bits != nullptr, "bits is NULL");
     T3D_TRY(check_words(words, "words"));
     int64_t W = words_for(n_samples);
-    dim3 block(256);
-    unsigned gy = (unsigned)std::min<int64_t>(n_samples, 65535);
-    unsigned gz = (unsigned)((n_samples + gy - 1) / gy);
-    dim3 grid((unsigned)((n_bits + 255) / 256), gy, gz);
-    ProfScope prof(T3D_K_LAYOUT, as_stream(stream));
-    k_unpack<<<grid, block, 0, as_stream(stream)>>>(n_bits, n_samples, W, words, bits);
+    const LayoutGrid g = layout_grid(n_bits, W);
+    cudaStream_t st = as_stream(stream);
+    ProfScope prof(T3D_K_LAYOUT, st);
+    if (layout_vec(bits, n_bits))
+        k_unpack<true><<<g.blocks, g.threads, 0, st>>>(n_bits, n_samples, W, words, bits, g.col_tiles, g.tiles);
+    else
+        k_unpack<false><<<g.blocks, g.threads, 0, st>>>(n_bits, n_samples, W, words, bits, g.col_tiles, g.tiles);
     T3D_LAUNCH_CHECK("unpack");
     return T3D_OK;
 }
