@@ -14,7 +14,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libtoric3d.so")
-SOURCES = ["t3d_api.cu", "t3d_bitsliced.cu", "t3d_bp.cu", "t3d_run.cu", "t3d_noalloc.cu", "t3d_cnn.cu",
+SOURCES = ["t3d_api.cu", "t3d_bitsliced.cu", "t3d_column.cu", "t3d_bp.cu", "t3d_run.cu", "t3d_noalloc.cu", "t3d_cnn.cu",
            "t3d_cnn_tc.cu", "t3d_bp_meta.cu",
            "t3d_tanner.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -850,10 +850,16 @@ t3d_status launch_syndrome(ItemTable& tab, uint64_t thr, uint64_t seed, uint32_t
     return T3D_OK;
 }
 
-t3d_status launch_sweeps(ItemTable& tab, const char* schedule, int slen, int n_apply, uint32_t sweep0,
+t3d_status launch_sweeps(ItemTable& all, const char* schedule, int slen, int n_apply, uint32_t sweep0,
                          uint64_t seed, uint32_t cycle, cudaStream_t st)
 {
     if (n_apply <= 0) return T3D_OK;
+    // lattices that fit one SM run the whole schedule in one launch
+    for (int i = 0; i < all.n; ++i)
+        if (column_fits(all.it[i].lat.L) && !all.it[i].stop)
+            T3D_TRY(launch_column_sweeps(all.it[i], schedule, slen, n_apply, sweep0, seed, cycle, st));
+    ItemTable tab = select_items(all, [](const ItemDesc& d) { return !column_fits(d.lat.L) || d.stop; });
+    if (tab.n == 0) return T3D_OK;
     for (int i = 0; i < tab.n; ++i) {
         ItemDesc& d = tab.it[i];
         const int64_t nw = d.nw ? d.nw : d.W;
@@ -927,12 +933,18 @@ t3d_status launch_sweeps(ItemTable& tab, const char* schedule, int slen, int n_a
     return T3D_OK;
 }
 
-t3d_status launch_flip_until_clear(ItemTable& tab, int max_sweeps, int32_t* sweeps_done, cudaStream_t st)
+t3d_status launch_flip_until_clear(ItemTable& all, int max_sweeps, int32_t* sweeps_done, cudaStream_t st)
 {
     if (max_sweeps <= 0) {
         if (sweeps_done) T3D_CUDA_CHECK(cudaMemsetAsync(sweeps_done, 0, sizeof(int32_t), st));
         return T3D_OK;
     }
+    for (int i = 0; i < all.n; ++i)
+        if (column_fits(all.it[i].lat.L))
+            T3D_TRY(launch_column_until_clear(all.it[i], max_sweeps, i == 0 ? sweeps_done : nullptr, st));
+    if (all.n > 0 && column_fits(all.it[0].lat.L)) sweeps_done = nullptr;
+    ItemTable tab = select_items(all, [](const ItemDesc& d) { return !column_fits(d.lat.L); });
+    if (tab.n == 0) return T3D_OK;
     for (int i = 0; i < tab.n; ++i) {
         T3D_REQUIRE(tab.it[i].stop != nullptr, "flip until clear: item %d has no flag words", i);
         T3D_CUDA_CHECK(cudaMemsetAsync(tab.it[i].stop, 0, kStopWords * sizeof(uint32_t), st));

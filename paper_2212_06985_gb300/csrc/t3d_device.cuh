@@ -161,6 +161,85 @@ __device__ __forceinline__ Words2 stream_words(uint64_t seed, uint32_t stream, u
     return r;
 }
 
+// The same generator for a thread that draws many sites of one word (group) and cycle.  The
+// first three rounds separate: with the counter (group, site, cycle, tag | block), the round
+// function never mixes the site with the block before round 4, so a site costs two products
+// and a block two products once each, and a (site, block) pair only rounds 4 to 10: seven
+// instead of ten (noise at L = 32, 8192 samples: see k_noise).
+struct PhiloxColumn {
+    uint32_t hg, lg;   // M0 * group
+    uint32_t hc, lc;   // M1 * cycle
+    uint32_t k0, k1;
+    uint32_t tag;      // stream << 30 | sweep << 8
+};
+
+struct PhiloxBlock {   // the block's share of the state after three rounds
+    uint32_t x, y, z;
+};
+
+struct PhiloxSite {    // the site's share
+    uint32_t a, b, c;
+};
+
+constexpr uint32_t kPhiloxM0 = 0xD2511F53u, kPhiloxM1 = 0xCD9E8D57u;
+constexpr uint32_t kPhiloxW0 = 0x9E3779B9u, kPhiloxW1 = 0xBB67AE85u;
+
+__device__ __forceinline__ PhiloxColumn philox_column(uint64_t seed, uint32_t stream, uint32_t cycle, uint32_t sweep,
+                                                      uint64_t group)
+{
+    PhiloxColumn c;
+    c.hg = __umulhi(kPhiloxM0, (uint32_t)group);
+    c.lg = kPhiloxM0 * (uint32_t)group;
+    c.hc = __umulhi(kPhiloxM1, cycle);
+    c.lc = kPhiloxM1 * cycle;
+    c.k0 = (uint32_t)seed;
+    c.k1 = (uint32_t)(seed >> 32);
+    c.tag = (stream << 30) | (sweep << 8);
+    return c;
+}
+
+__device__ __forceinline__ PhiloxBlock philox_block(const PhiloxColumn& c, uint32_t block)
+{
+    const uint32_t n2 = c.hg ^ (c.tag | block) ^ c.k1;                               // round 1
+    const uint32_t n0 = __umulhi(kPhiloxM1, n2) ^ c.lc ^ (c.k0 + kPhiloxW0);         // round 2
+    PhiloxBlock b;                                                                   // round 3
+    b.x = (kPhiloxM1 * n2) ^ (c.k0 + 2 * kPhiloxW0);
+    b.y = __umulhi(kPhiloxM0, n0) ^ (c.k1 + 2 * kPhiloxW1);
+    b.z = kPhiloxM0 * n0;
+    return b;
+}
+
+__device__ __forceinline__ PhiloxSite philox_site(const PhiloxColumn& c, uint32_t site)
+{
+    const uint32_t n0 = c.hc ^ site ^ c.k0;                                          // round 1
+    const uint32_t n2 = __umulhi(kPhiloxM0, n0) ^ c.lg ^ (c.k1 + kPhiloxW1);         // round 2
+    PhiloxSite s;                                                                    // round 3
+    s.a = __umulhi(kPhiloxM1, n2);
+    s.b = kPhiloxM1 * n2;
+    s.c = kPhiloxM0 * n0;
+    return s;
+}
+
+__device__ __forceinline__ U32x4 philox_finish(const PhiloxColumn& col, const PhiloxSite& s, const PhiloxBlock& b)
+{
+    uint32_t c0 = s.a ^ b.x, c1 = s.b, c2 = s.c ^ b.y, c3 = b.z;
+    uint32_t k0 = col.k0 + 2 * kPhiloxW0, k1 = col.k1 + 2 * kPhiloxW1;
+#pragma unroll
+    for (int round = 3; round < 10; ++round) {
+        k0 += kPhiloxW0;
+        k1 += kPhiloxW1;
+        const uint32_t h0 = __umulhi(kPhiloxM0, c0), l0 = kPhiloxM0 * c0;
+        const uint32_t h1 = __umulhi(kPhiloxM1, c2), l1 = kPhiloxM1 * c2;
+        c0 = h1 ^ c1 ^ k0;
+        c1 = l1;
+        c2 = h0 ^ c3 ^ k1;
+        c3 = l0;
+    }
+    U32x4 r;
+    r.v[0] = c0; r.v[1] = c1; r.v[2] = c2; r.v[3] = c3;
+    return r;
+}
+
 // 64 Bernoulli(P / 2^32) bits, one per sample of word `group` (P = thr): lane j is set iff
 // U_j < P for a 32-bit uniform U_j.  The six high bits of every lane (bit 31-i of U_j = bit j
 // of stream word i, i = 0..5, blocks 0..2) are compared with P's, most significant first and
@@ -200,6 +279,55 @@ __device__ __forceinline__ uint64_t bernoulli_word(uint64_t thr, uint64_t seed, 
             const uint64_t b = eq & (0 - eq);   // the lowest tied lane left (0 once none is)
             if ((o.v[i] >> 6) < low) lt |= b;
             eq ^= b;
+        }
+    }
+    return lt;
+}
+
+// bernoulli_word for a thread that draws many sites of one column: the same words, the blocks'
+// shares (0..2, and 3 for the tails) computed once.
+struct BernoulliColumn {
+    PhiloxColumn col;
+    PhiloxBlock blk[4];
+};
+
+__device__ __forceinline__ BernoulliColumn bernoulli_column(uint64_t seed, uint32_t stream, uint32_t cycle,
+                                                            uint64_t group)
+{
+    BernoulliColumn b;
+    b.col = philox_column(seed, stream, cycle, 0, group);
+#pragma unroll
+    for (uint32_t i = 0; i < 4; ++i) b.blk[i] = philox_block(b.col, i);
+    return b;
+}
+
+// thr in 1 .. 2^32 - 1 (the callers take the constant cases before their loops).
+__device__ __forceinline__ uint64_t bernoulli_site(const BernoulliColumn& bc, uint32_t thr, uint32_t site)
+{
+    const PhiloxSite ps = philox_site(bc.col, site);
+    uint64_t lt = 0, eq = ~0ULL;
+#pragma unroll
+    for (int blk = 0; blk < 3; ++blk) {
+        const U32x4 o = philox_finish(bc.col, ps, bc.blk[blk]);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const uint64_t w = (uint64_t)o.v[2 * i] | ((uint64_t)o.v[2 * i + 1] << 32);
+            if ((thr >> (31 - (2 * blk + i))) & 1u) {
+                lt |= eq & ~w;
+                eq &= w;
+            } else {
+                eq &= ~w;
+            }
+        }
+    }
+    const uint32_t low = thr << 6;   // o >> 6 < low 26 bits of P  <=>  o < those bits << 6
+    for (uint32_t blk = 3; eq != 0; ++blk) {
+        const U32x4 o = philox_finish(bc.col, ps, blk == 3 ? bc.blk[3] : philox_block(bc.col, blk));
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const uint64_t rest = eq & (eq - 1);   // without the lowest tied lane left
+            if (o.v[i] < low) lt |= eq ^ rest;
+            eq = rest;
         }
     }
     return lt;

@@ -120,6 +120,17 @@ t3d_status launch_flip_until_clear(ItemTable& tab, int max_sweeps, int32_t* swee
 t3d_status launch_sweeps(ItemTable& tab, const char* schedule, int slen, int n_apply,
                          uint32_t sweep0, uint64_t seed, uint32_t cycle, cudaStream_t st);
 t3d_status launch_logical(ItemTable& tab, cudaStream_t st);
+// Lattices whose syndrome and flip words fit one SM (t3d_column.cu, L <= 16): a schedule, a flip
+// until clear, or whole runs in one launch per item.  No scratch (ItemDesc::tmp, stop) is used.
+struct ItemDesc;
+bool column_fits(int L);
+t3d_status launch_column_sweeps(const ItemDesc& d, const char* schedule, int slen, int n_apply, uint32_t sweep0,
+                                uint64_t seed, uint32_t cycle, cudaStream_t st);
+t3d_status launch_column_until_clear(const ItemDesc& d, int max_sweeps, int32_t* sweeps_done, cudaStream_t st);
+// cycles cycle0 + 1 .. cycle0 + cycles of noise, measurement and the schedule, then, with perfect
+// >= 0, a noiseless measurement decoded by up to that many flip applications; e in, e out.
+t3d_status launch_column_run(const ItemDesc& d, int cycles, uint32_t cycle0, uint64_t thr_p, uint64_t thr_q,
+                             uint64_t seed, const char* schedule, int slen, int n_apply, int perfect, cudaStream_t st);
 // e ^= d, s ^= H d from decision words dec[word][site][4] (32-bit halves).
 t3d_status launch_dec_apply(const Lattice& lat, int64_t W, int64_t words, const uint64_t* dec, uint64_t* e,
                             uint64_t* s, cudaStream_t st);

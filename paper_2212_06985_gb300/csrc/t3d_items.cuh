@@ -109,6 +109,17 @@ inline bool has_live(const ItemTable& tab)
     return false;
 }
 
+// The items of `tab` for which keep(item) holds, in order.
+template <class F>
+inline ItemTable select_items(const ItemTable& tab, F&& keep)
+{
+    ItemTable out = tab;
+    out.n = 0;
+    for (int i = 0; i < tab.n; ++i)
+        if (keep(tab.it[i])) out.it[out.n++] = tab.it[i];
+    return out;
+}
+
 inline void finish_table(ItemTable& tab)
 {
     tab.prefix[0] = 0;

@@ -343,15 +343,27 @@ t3d_status enqueue_run(const t3d_run_cfg& c, const Plan& pl, cudaStream_t st)
     const uint64_t thr_p = prob_threshold(c.p), thr_q = prob_threshold(c.q);
     const int slen = (int)strnlen(c.schedule, sizeof(c.schedule));
     ItemTable tab;
-    for (int t = 1; t <= c.T; ++t) {
+    // flip / p-flip runs of lattices that fit one SM: all cycles and the noiseless round in one
+    // launch per item; the other items (`items`) go step by step
+    const bool columns = !learned(c) && !c.use_bp;
+    auto stepwise = [&](const ItemDesc& d) { return !columns || !column_fits(d.lat.L); };
+    if (columns) {
+        if (c.T > 0 || c.perfect_round)
+            for (int i = 0; i < pl.items.n; ++i)
+                if (column_fits(pl.items.it[i].lat.L))
+                    T3D_TRY(launch_column_run(pl.items.it[i], c.T, c.cycle0, thr_p, thr_q, c.seed, c.schedule, slen,
+                                              c.n_apply, c.perfect_round ? c.perfect_max_sweeps : -1, st));
+    }
+    const ItemTable items = select_items(pl.items, stepwise);
+    for (int t = 1; t <= c.T && items.n > 0; ++t) {
         const uint32_t cycle = c.cycle0 + (uint32_t)t;
         if (learned(c)) {
             T3D_TRY(enqueue_learned_cycle(c, pl, cycle, thr_p, thr_q, slen, st));
             continue;
         }
-        tab = pl.items;
+        tab = items;
         T3D_TRY(launch_noise(tab, thr_p, c.seed, cycle, st));
-        tab = pl.items;
+        tab = items;
         T3D_TRY(launch_syndrome(tab, thr_q, c.seed, cycle, st));
         if (meta_checks(c)) {
             for (int i = 0; i < pl.items.n; ++i) {
@@ -364,20 +376,21 @@ t3d_status enqueue_run(const t3d_run_cfg& c, const Plan& pl, cudaStream_t st)
                               nullptr, st));
         }
         if (c.n_apply > 0) {
-            tab = pl.items;
+            tab = items;
             T3D_TRY(launch_sweeps(tab, c.schedule, slen, c.n_apply, 0, c.seed, cycle, st));
         }
     }
-    if (c.perfect_round) {
+    if (c.perfect_round && items.n > 0) {
         const uint32_t cycle = c.cycle0 + (uint32_t)c.T + 1;
-        tab = pl.items;
+        tab = items;
         T3D_TRY(launch_syndrome(tab, 0, c.seed, cycle, st));
         if (c.perfect_max_sweeps > 0) {
             // flip until every item's syndrome clears, at most perfect_max_sweeps applications
             // (the applications after an item clears do no work; the results are those of
             // perfect_max_sweeps applications)
-            tab = pl.items;
-            for (int i = 0; i < tab.n; ++i) tab.it[i].stop = pl.stop[i];
+            ItemTable flagged = pl.items;
+            for (int i = 0; i < flagged.n; ++i) flagged.it[i].stop = pl.stop[i];
+            tab = select_items(flagged, stepwise);
             T3D_TRY(launch_flip_until_clear(tab, c.perfect_max_sweeps, nullptr, st));
         }
     }
