@@ -30,19 +30,39 @@ int row_words(int64_t words)
     return tx;
 }
 
-// Blocks an item needs for a (sites x words) tiling with rows of tx words.
-int64_t tile_blocks(int64_t n_sites, int64_t W, int tx)
+// Blocks an item needs for a (sites x words) tiling with rows of tx words and `per` sites a thread.
+int64_t tile_blocks(int64_t n_sites, int64_t W, int tx, int per = 1)
 {
-    const int ty = kThreads / tx;
+    const int ty = kThreads / tx * per;
     return ((n_sites + ty - 1) / ty) * ((W + tx - 1) / tx);
+}
+
+// Sites per thread of the noise and measurement kernels: a thread that draws several sites of
+// one word computes the word's share of the generator once (about 45 instructions).  Up to
+// kMaxPer, a power of two, as long as the launch keeps about eight blocks per SM.  (The p-flip
+// decisions wait for their syndrome words as well: several sites a thread measured 1.80 against
+// 1.68 ms at L = 32, 10^5 samples, so they take one.)
+constexpr int kMaxPer = 16;
+
+int sites_per_thread(const ItemTable& tab, int dirs)
+{
+    int64_t blocks = 0;
+    for (int i = 0; i < tab.n; ++i) {
+        const ItemDesc& d = tab.it[i];
+        const int64_t nw = d.nw ? d.nw : d.W;
+        blocks += tile_blocks((int64_t)dirs * d.lat.L3, nw, row_words(nw));
+    }
+    int per = 1;
+    while (per < kMaxPer && blocks / (2 * per) >= 152 * 8) per *= 2;
+    return per;
 }
 
 // The same for the kernels that split a block index with 32-bit arithmetic
 // (tile_site_word): T3D_EINVAL if the item needs 2^32 blocks or more (a state
 // array of at least 2^32 x 256 words, far beyond device memory).
-t3d_status tile_blocks_checked(const ItemDesc& d, int64_t n_sites, int64_t W, int tx, int64_t* blocks)
+t3d_status tile_blocks_checked(const ItemDesc& d, int64_t n_sites, int64_t W, int tx, int64_t* blocks, int per = 1)
 {
-    *blocks = tile_blocks(n_sites, W, tx);
+    *blocks = tile_blocks(n_sites, W, tx, per);
     T3D_REQUIRE(n_sites < (1LL << 31) && *blocks < (1LL << 32),
                 "lattice L = %d with %lld words needs too many thread blocks", d.lat.L, (long long)W);
     return T3D_OK;
@@ -68,44 +88,81 @@ __device__ __forceinline__ bool tile_site_word(const ItemDesc& d, int64_t lb, in
 }
 
 
-// e ^= Bernoulli(p) for every edge (Sec. 3.1 phenomenological qubit noise).
+// The same for a thread that takes `per` (a power of two) sites of one word: its first site and
+// the step to the next (the block's rows); a block covers per * ty consecutive sites.
+__device__ __forceinline__ bool tile_sites(const ItemDesc& d, int64_t lb, int n_sites, int per, int& site, int& step,
+                                           int64_t& w)
+{
+    const int tx = d.tx, lx = __ffs(tx) - 1, ly = __ffs(kThreads) - 1 - lx, lp = __ffs(per) - 1 + ly;
+    const uint32_t site_tiles = ((uint32_t)n_sites + (1u << lp) - 1) >> lp;
+    const uint32_t word_tile = (uint32_t)lb / site_tiles;
+    const uint32_t site_tile = (uint32_t)lb - word_tile * site_tiles;
+    const int t = threadIdx.x;
+    w = (int64_t)word_tile * tx + (t & (tx - 1));
+    site = (int)(site_tile << lp) + (t >> lx);
+    step = 1 << ly;
+    return w < (d.nw ? d.nw : d.W) && site < n_sites;
+}
+
+// e ^= Bernoulli(p) for every edge (Sec. 3.1 phenomenological qubit noise).  Bound by the
+// generator's integer instructions (the ALU pipe at 68%, ncu, 8192 samples at L = 32); a thread
+// draws up to 16 edges of one word, so that the first rounds' products of the word and of its
+// blocks are shared (PhiloxColumn): 157 -> 105 M warp instructions there, and 2.28 -> 1.82 ms at
+// L = 32, 10^5 samples (one edge a thread before; 4 edges a thread 2.04 ms).
 __global__ void __launch_bounds__(kThreads)
-k_noise(const __grid_constant__ ItemTable tab, uint64_t thr, uint64_t seed, uint32_t cycle)
+k_noise(const __grid_constant__ ItemTable tab, uint64_t thr, uint64_t seed, uint32_t cycle, int per)
 {
     for_each_item_block(tab, [&](const ItemDesc& d, int64_t lb) {
-        int v;
+        const int n = 3 * d.lat.L3;
+        int v, step;
         int64_t w;
-        if (!tile_site_word(d, lb, 3 * d.lat.L3, v, w)) return;
-        const uint64_t flips =
-            bernoulli_word(thr, seed, kStreamQubit, (uint64_t)v, cycle, 0, d.group0 + w);
-        if (flips) d.e[(int64_t)v * d.W + w] ^= flips;
+        if (!tile_sites(d, lb, n, per, v, step, w)) return;
+        const BernoulliColumn bc = bernoulli_column(seed, kStreamQubit, cycle, d.group0 + w);
+        uint64_t* __restrict__ e = d.e + (int64_t)v * d.W + w;
+        const int64_t stepW = (int64_t)step * d.W;
+        for (int k = 0; k < per && v < n; ++k, v += step, e += stepW) {
+            const uint64_t was = *e;   // requested before the draw, which hides its latency
+            *e = was ^ (thr >> 32 ? ~0ULL : bernoulli_site(bc, (uint32_t)thr, (uint32_t)v));
+        }
     });
 }
 
-// s_f = XOR of the face's four edges, then ^= Bernoulli(q) (Sec. 2, Sec. 3.1).
+// s_f = XOR of the face's four edges, then ^= Bernoulli(q) (Sec. 2, Sec. 3.1).  A thread takes the
+// three faces of up to 16 sites of one word: nine edge words per site instead of twelve, and the
+// generator's share of the word once (as k_noise): 190 -> 119 M warp instructions at L = 32, 8192
+// samples, and 2.61 -> 2.02 ms at 10^5 samples (one face a thread before).
 __global__ void __launch_bounds__(kThreads)
-k_syndrome(const __grid_constant__ ItemTable tab, uint64_t thr, uint64_t seed, uint32_t cycle)
+k_syndrome(const __grid_constant__ ItemTable tab, uint64_t thr, uint64_t seed, uint32_t cycle, int per)
 {
     for_each_item_block(tab, [&](const ItemDesc& d, int64_t lb) {
         const Lattice lat = d.lat;
-        int f;
+        int site, step;
         int64_t w;
-        if (!tile_site_word(d, lb, 3 * lat.L3, f, w)) return;
-        const int n = (f >= lat.L3) + (f >= 2 * lat.L3), site = f - n * lat.L3;
-        // face (n, r) spans the axes a < b other than n; its edges are the a-edges at r and
-        // r + e_b and the b-edges at r and r + e_a (periodic site deltas by selects, no
-        // per-thread arrays)
-        const Coord r = site_coord(lat, site);
+        if (!tile_sites(d, lb, lat.L3, per, site, step, w)) return;
+        const int64_t W = d.W, L3W = (int64_t)lat.L3 * W;
         const int L = lat.L;
-        const int dx = r.x[0] + 1 == L ? 1 - L : 1, dy = r.x[1] + 1 == L ? L - lat.L2 : L,
-                  dz = r.x[2] + 1 == L ? lat.L2 - lat.L3 : lat.L2;
-        const int a = n == 0 ? 1 : 0, b = n == 2 ? 1 : 2;
-        const int da = a == 0 ? dx : dy, db = b == 1 ? dy : dz;
-        const uint64_t* __restrict__ pa = d.e + ((int64_t)a * lat.L3 + site) * d.W + w;
-        const uint64_t* __restrict__ pb = d.e + ((int64_t)b * lat.L3 + site) * d.W + w;
-        uint64_t acc = pa[0] ^ pa[(int64_t)db * d.W] ^ pb[0] ^ pb[(int64_t)da * d.W];
-        acc ^= bernoulli_word(thr, seed, kStreamMeas, (uint64_t)f, cycle, 0, d.group0 + w);
-        d.s[(int64_t)f * d.W + w] = acc;
+        const BernoulliColumn bc = bernoulli_column(seed, kStreamMeas, cycle, d.group0 + w);
+        for (int k = 0; k < per && site < lat.L3; ++k, site += step) {
+            // face (n, r) spans the axes a < b other than n; its edges are the a-edges at r and
+            // r + e_b and the b-edges at r and r + e_a
+            const Coord r = site_coord(lat, site);
+            const int64_t dx = (int64_t)(r.x[0] + 1 == L ? 1 - L : 1) * W,
+                          dy = (int64_t)(r.x[1] + 1 == L ? L - lat.L2 : L) * W,
+                          dz = (int64_t)(r.x[2] + 1 == L ? lat.L2 - lat.L3 : lat.L2) * W;
+            const uint64_t* __restrict__ px = d.e + (int64_t)site * W + w;
+            const uint64_t* __restrict__ py = px + L3W;
+            const uint64_t* __restrict__ pz = py + L3W;
+            const uint64_t ex = px[0], ey = py[0], ez = pz[0];
+            uint64_t s[3] = {ey ^ py[dz] ^ ez ^ pz[dy], ex ^ px[dz] ^ ez ^ pz[dx], ex ^ px[dy] ^ ey ^ py[dx]};
+            uint64_t* __restrict__ out = d.s + (int64_t)site * W + w;
+            if (thr != 0) {
+#pragma unroll
+                for (int n = 0; n < 3; ++n)
+                    s[n] ^= thr >> 32 ? ~0ULL : bernoulli_site(bc, (uint32_t)thr, (uint32_t)(n * lat.L3 + site));
+            }
+#pragma unroll
+            for (int n = 0; n < 3; ++n) out[n * L3W] = s[n];
+        }
     });
 }
 
@@ -820,32 +877,34 @@ bool layout_vec(const void* bits, int64_t n_bits) { return n_bits % 4 == 0 && al
 t3d_status launch_noise(ItemTable& tab, uint64_t thr, uint64_t seed, uint32_t cycle, cudaStream_t st)
 {
     if (thr == 0) return T3D_OK;
+    const int per = sites_per_thread(tab, 3);
     for (int i = 0; i < tab.n; ++i) {
         ItemDesc& d = tab.it[i];
         const int64_t nw = d.nw ? d.nw : d.W;
         d.tx = row_words(nw);
-        T3D_TRY(tile_blocks_checked(d, 3LL * d.lat.L3, nw, d.tx, &d.blocks));
+        T3D_TRY(tile_blocks_checked(d, 3LL * d.lat.L3, nw, d.tx, &d.blocks, per));
     }
     finish_table(tab);
     ProfScope prof(T3D_K_NOISE, st);
     k_noise<<<persistent_grid((const void*)k_noise, kThreads, T3D_K_NOISE, tab.prefix[tab.n], has_live(tab)), kThreads,
-              0, st>>>(tab, thr, seed, cycle);
+              0, st>>>(tab, thr, seed, cycle, per);
     T3D_LAUNCH_CHECK("noise");
     return T3D_OK;
 }
 
 t3d_status launch_syndrome(ItemTable& tab, uint64_t thr, uint64_t seed, uint32_t cycle, cudaStream_t st)
 {
+    const int per = sites_per_thread(tab, 1);
     for (int i = 0; i < tab.n; ++i) {
         ItemDesc& d = tab.it[i];
         const int64_t nw = d.nw ? d.nw : d.W;
         d.tx = row_words(nw);
-        T3D_TRY(tile_blocks_checked(d, 3LL * d.lat.L3, nw, d.tx, &d.blocks));
+        T3D_TRY(tile_blocks_checked(d, d.lat.L3, nw, d.tx, &d.blocks, per));
     }
     finish_table(tab);
     ProfScope prof(T3D_K_SYNDROME, st);
     k_syndrome<<<persistent_grid((const void*)k_syndrome, kThreads, T3D_K_SYNDROME, tab.prefix[tab.n], has_live(tab)),
-                 kThreads, 0, st>>>(tab, thr, seed, cycle);
+                 kThreads, 0, st>>>(tab, thr, seed, cycle, per);
     T3D_LAUNCH_CHECK("syndrome");
     return T3D_OK;
 }

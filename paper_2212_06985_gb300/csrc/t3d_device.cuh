@@ -165,7 +165,7 @@ __device__ __forceinline__ Words2 stream_words(uint64_t seed, uint32_t stream, u
 // first three rounds separate: with the counter (group, site, cycle, tag | block), the round
 // function never mixes the site with the block before round 4, so a site costs two products
 // and a block two products once each, and a (site, block) pair only rounds 4 to 10: seven
-// instead of ten (noise at L = 32, 8192 samples: see k_noise).
+// instead of ten (measured at k_noise).
 struct PhiloxColumn {
     uint32_t hg, lg;   // M0 * group
     uint32_t hc, lc;   // M1 * cycle
