@@ -913,11 +913,12 @@ t3d_status launch_sweeps(ItemTable& all, const char* schedule, int slen, int n_a
                          uint64_t seed, uint32_t cycle, cudaStream_t st)
 {
     if (n_apply <= 0) return T3D_OK;
-    // lattices that fit one SM run the whole schedule in one launch
+    // lattices that fit one SM or a cluster run the whole schedule in one launch
+    auto on_chip = [&](const ItemDesc& d) { return !d.stop && sweeps_fit(d.lat.L, d.nw ? d.nw : d.W, n_apply); };
     for (int i = 0; i < all.n; ++i)
-        if (column_fits(all.it[i].lat.L) && !all.it[i].stop)
+        if (on_chip(all.it[i]))
             T3D_TRY(launch_column_sweeps(all.it[i], schedule, slen, n_apply, sweep0, seed, cycle, st));
-    ItemTable tab = select_items(all, [](const ItemDesc& d) { return !column_fits(d.lat.L) || d.stop; });
+    ItemTable tab = select_items(all, [&](const ItemDesc& d) { return !on_chip(d); });
     if (tab.n == 0) return T3D_OK;
     for (int i = 0; i < tab.n; ++i) {
         ItemDesc& d = tab.it[i];
@@ -998,11 +999,12 @@ t3d_status launch_flip_until_clear(ItemTable& all, int max_sweeps, int32_t* swee
         if (sweeps_done) T3D_CUDA_CHECK(cudaMemsetAsync(sweeps_done, 0, sizeof(int32_t), st));
         return T3D_OK;
     }
+    auto on_chip = [&](const ItemDesc& d) { return sweeps_fit(d.lat.L, d.nw ? d.nw : d.W, max_sweeps); };
     for (int i = 0; i < all.n; ++i)
-        if (column_fits(all.it[i].lat.L))
+        if (on_chip(all.it[i]))
             T3D_TRY(launch_column_until_clear(all.it[i], max_sweeps, i == 0 ? sweeps_done : nullptr, st));
-    if (all.n > 0 && column_fits(all.it[0].lat.L)) sweeps_done = nullptr;
-    ItemTable tab = select_items(all, [](const ItemDesc& d) { return !column_fits(d.lat.L); });
+    if (all.n > 0 && on_chip(all.it[0])) sweeps_done = nullptr;
+    ItemTable tab = select_items(all, [&](const ItemDesc& d) { return !on_chip(d); });
     if (tab.n == 0) return T3D_OK;
     for (int i = 0; i < tab.n; ++i) {
         T3D_REQUIRE(tab.it[i].stop != nullptr, "flip until clear: item %d has no flag words", i);

@@ -22,6 +22,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
 #include "t3d_device.cuh"
 #include "t3d_host.hpp"
@@ -273,6 +274,397 @@ k_column(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgr
     }
 }
 
+// ------------------------------------------------------------------ slabs of a cluster
+// Larger lattices (L = 15 .. 32): the lattice of one word is split into z-slabs over the blocks
+// of a thread-block cluster, each keeping its slab's syndrome and flip words in shared memory.
+// The two phases of an application read one word per (x, y) column from the neighbouring block
+// (distributed shared memory): the syndrome below the slab, the flips above it; a cluster barrier
+// separates them.  The flips that reach e are gathered in registers, kK sites a thread, and XORed
+// into e once at the end.
+__device__ __forceinline__ void cluster_barrier()
+{
+    asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The word at this block's shared-memory address `p` in block `rank` of the cluster.
+__device__ __forceinline__ uint64_t cluster_load(const uint64_t* p, uint32_t rank)
+{
+    uint64_t v;
+    asm volatile(
+        "{\n"
+        ".reg .u32 a;\n"
+        "mapa.shared::cluster.u32 a, %1, %2;\n"
+        "ld.shared::cluster.u64 %0, [a];\n"
+        "}\n"
+        : "=l"(v)
+        : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank)
+        : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void cluster_store(uint32_t* p, uint32_t rank, uint32_t v)
+{
+    asm volatile(
+        "{\n"
+        ".reg .u32 a;\n"
+        "mapa.shared::cluster.u32 a, %0, %1;\n"
+        "st.shared::cluster.u32 [a], %2;\n"
+        "}\n" ::"r"((uint32_t)__cvta_generic_to_shared(p)),
+        "r"(rank), "r"(v)
+        : "memory");
+}
+
+constexpr int kMaxCluster = 8;
+
+// Where a word's column lies: row r of word w at p[r * row + w * word].
+struct ColumnView {
+    uint64_t* p;
+    int64_t row, word;
+    __device__ __forceinline__ uint64_t& at(int64_t r, int64_t w) const { return p[r * row + w * word]; }
+};
+
+// Thread (x, j) of z-part zp owns the sites of rows j and j + ceil(L / 2), z0 <= z < z1 (at most
+// kZ planes); the z-neighbours are words it has just read.  Bound by the shared-memory pipe (23
+// words read or written per site and application) and, in p-flip, the ALU (the coins).  Measured
+// at L = 32, 10^5 samples, one application of a longer schedule: flip 0.43 ms against 0.83 as a
+// kernel of its own, p-flip 0.83 against 1.46; the columns' way in and out costs 2.2 ms once (see
+// sweeps_fit).  Keeping the syndrome in registers too (17 words, but 96 registers of state that
+// spill) measured the same, row pairs with shared y-neighbours and prefetched planes slower.
+// Keeps the compiler from computing what follows from v outside the loop over applications: the
+// unrolled sites' shared-memory addresses, kept in registers across it, would push the state
+// itself into local memory.
+__device__ __forceinline__ int here(int v)
+{
+    asm volatile("" : "+r"(v));
+    return v;
+}
+
+template <int kZ, int kT>
+__global__ void __launch_bounds__(kT, 1)
+k_slab(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgram pr, int C, const ColumnView sv,
+       const ColumnView ev, int e_store)
+{
+    extern __shared__ uint64_t sm[];
+    __shared__ uint32_t left[2][kMaxCluster];   // flip until clear: the blocks' unsatisfied checks
+    const int L = d.lat.L, P = d.lat.L2, L3 = d.lat.L3;
+    const int rank = (int)(blockIdx.x % (unsigned)C);
+    const int zbase = rank * L / C, nz = (rank + 1) * L / C - zbase, most = (L + C - 1) / C;
+    const int down = rank == 0 ? C - 1 : rank - 1, up = rank + 1 == C ? 0 : rank + 1;
+    const int nz_down = (down + 1) * L / C - down * L / C;
+    const int N = most * P;
+    uint64_t* const S0 = sm;
+    uint64_t* const S1 = sm + N;
+    uint64_t* const S2 = sm + 2 * N;
+    uint64_t* const Fx = sm + 3 * N;
+    uint64_t* const Fy = sm + 4 * N;
+    uint64_t* const Fz = sm + 5 * N;
+
+    const int t = threadIdx.x;
+    const int half = (L + 1) / 2, H = half * L;    // rows j and j + half of a plane
+    const int zp = t / H, u = t - zp * H;
+    const int j = u / L, x = u - j * L;
+    const bool mine = zp < pr.zt;
+    const int rows = !mine ? 0 : j + half < L ? 2 : 1;
+    const int z0 = mine ? zp * nz / pr.zt : 0, z1 = mine ? (zp + 1) * nz / pr.zt : 0;
+    // offsets of the y-neighbours of the two rows (periodic)
+    const int ym0 = j == 0 ? (L - 1) * L : -L, ym1 = -L;
+    const int yp0 = j + 1 == L ? -j * L : L, yp1 = j + half + 1 == L ? -(j + half) * L : L;
+    const int xm = x == 0 ? L - 1 : -1, xp = x + 1 == L ? 1 - L : 1;
+
+    const int64_t words = d.nw ? d.nw : d.W;
+    const int64_t have = d.live ? min(words, *d.live - d.w0) : words;
+    for (int64_t w = blockIdx.x / (unsigned)C; w < have; w += gridDim.x / (unsigned)C) {
+        const uint64_t group = word_group(d, w);
+        const int o0 = here(z0 * P + u), r0 = here((zbase + z0) * P + u);
+        uint64_t acc[kZ][2][3];
+#pragma unroll
+        for (int k = 0; k < kZ; ++k)
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+#pragma unroll
+                for (int n = 0; n < 3; ++n) {
+                    acc[k][c][n] = 0;
+                    if (z0 + k < z1 && c < rows)
+                        sm[n * N + o0 + k * P + c * H] = sv.at(n * L3 + r0 + k * P + c * H, w);
+                }
+        cluster_barrier();
+
+        // the coin words of the thread's edges into F (p-flip; each thread reads its own back)
+        auto coins = [&](uint32_t sweep) {
+            const PhiloxColumn pc = philox_column(pr.seed, kStreamCoin, pr.cycle0, sweep, group);
+            const PhiloxBlock b0 = philox_block(pc, 0), b1 = philox_block(pc, 1);
+            for (int c = 0; c < rows; ++c)
+                for (int z = z0; z < z1; ++z) {
+                    const int i = z * P + u + c * H;
+                    const PhiloxSite ps = philox_site(pc, (uint32_t)(zbase * P + i));
+                    const U32x4 a = philox_finish(pc, ps, b0);
+                    Fx[i] = (uint64_t)a.v[0] | ((uint64_t)a.v[1] << 32);
+                    Fy[i] = (uint64_t)a.v[2] | ((uint64_t)a.v[3] << 32);
+                    const U32x4 b = philox_finish(pc, ps, b1);
+                    Fz[i] = (uint64_t)b.v[0] | ((uint64_t)b.v[1] << 32);
+                }
+        };
+        // decide: flips of the thread's edges into F and acc
+        auto decide = [&](auto prob) {
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                if (c >= rows) break;
+                int i = here(z0 * P + u + c * H);
+                uint64_t m0, m1;   // faces 0 and 1 of the plane below
+                if (z0 == 0) {
+                    m0 = cluster_load(S0 + (nz_down - 1) * P + i, (uint32_t)down);
+                    m1 = cluster_load(S1 + (nz_down - 1) * P + i, (uint32_t)down);
+                } else {
+                    m0 = S0[i - P];
+                    m1 = S1[i - P];
+                }
+                const int im = c ? ym1 : ym0;
+#pragma unroll
+                for (int k = 0; k < kZ; ++k, i += P) {
+                    if (z0 + k >= z1) break;
+                    const uint64_t s0 = S0[i], s1 = S1[i], s2 = S2[i];
+                    const uint64_t s2y = S2[i + im], s2x = S2[i + xm], s1x = S1[i + xm], s0y = S0[i + im];
+                    uint64_t fx = at_least_three(s2, s2y, s1, m1), fy = at_least_three(s2, s2x, s0, m0),
+                             fz = at_least_three(s1, s1x, s0, s0y);
+                    if (decltype(prob)::value) {
+                        fx |= exactly_two(s2, s2y, s1, m1) & Fx[i];
+                        fy |= exactly_two(s2, s2x, s0, m0) & Fy[i];
+                        fz |= exactly_two(s1, s1x, s0, s0y) & Fz[i];
+                    }
+                    Fx[i] = fx;
+                    Fy[i] = fy;
+                    Fz[i] = fz;
+                    acc[k][c][0] ^= fx;
+                    acc[k][c][1] ^= fy;
+                    acc[k][c][2] ^= fz;
+                    m0 = s0;
+                    m1 = s1;
+                }
+            }
+        };
+        // update: the faces take their edges' flips; whether any keeps an unsatisfied check
+        auto update = [&]() -> uint64_t {
+            uint64_t nz_left = 0;
+#pragma unroll
+            for (int c = 0; c < 2; ++c) {
+                if (c >= rows) break;
+                const int top = here(u + c * H);
+                uint64_t fxa, fya;   // x- and y-edge flips of the plane above
+                if (z1 == nz) {
+                    fxa = cluster_load(Fx + top, (uint32_t)up);
+                    fya = cluster_load(Fy + top, (uint32_t)up);
+                } else {
+                    fxa = Fx[z1 * P + top];
+                    fya = Fy[z1 * P + top];
+                }
+                const int ip = c ? yp1 : yp0;
+                int i = top + (z0 + kZ - 1) * P;
+#pragma unroll
+                for (int k = kZ - 1; k >= 0; --k, i -= P) {
+                    if (z0 + k >= z1) continue;
+                    const uint64_t fx = Fx[i], fy = Fy[i], fz = Fz[i];
+                    const uint64_t n0 = S0[i] ^ fy ^ fya ^ fz ^ Fz[i + ip],
+                                   n1 = S1[i] ^ fx ^ fxa ^ fz ^ Fz[i + xp],
+                                   n2 = S2[i] ^ fx ^ Fx[i + ip] ^ fy ^ Fy[i + xp];
+                    S0[i] = n0;
+                    S1[i] = n1;
+                    S2[i] = n2;
+                    nz_left |= n0 | n1 | n2;
+                    fxa = fx;
+                    fya = fy;
+                }
+            }
+            return nz_left;
+        };
+
+        if (pr.until_clear) {
+            uint64_t nz_left = 0;
+            for (int c = 0; c < rows; ++c)
+                for (int z = z0; z < z1; ++z) {
+                    const int i = z * P + u + c * H;
+                    nz_left |= S0[i] | S1[i] | S2[i];
+                }
+            int ran = 0;
+            for (;;) {
+                // every block tells every block; the slots alternate, so a slot is written again
+                // only after the barrier that follows its reads
+                const uint32_t any = __syncthreads_or(nz_left != 0) ? 1u : 0u;
+                if (t < C) cluster_store(&left[ran & 1][rank], (uint32_t)t, any);
+                cluster_barrier();
+                uint32_t all = 0;
+                for (int r = 0; r < C; ++r) all |= left[ran & 1][r];
+                if (!all || ran == pr.n_apply) break;
+                decide(std::false_type());
+                cluster_barrier();
+                nz_left = update();
+                ++ran;
+            }
+            if (pr.sweeps_done && rank == 0 && t == 0) atomicMax(pr.sweeps_done, ran);
+        } else {
+            for (int k = 0, letter = 0; k < pr.n_apply; ++k) {
+                if ((pr.sched >> letter) & 1) {
+                    coins(pr.sweep0 + (uint32_t)k);
+                    decide(std::true_type());
+                } else {
+                    decide(std::false_type());
+                }
+                if (++letter == pr.slen) letter = 0;
+                cluster_barrier();
+                update();
+                cluster_barrier();
+            }
+        }
+        const int r1 = here((zbase + z0) * P + u);
+#pragma unroll
+        for (int k = 0; k < kZ; ++k)
+#pragma unroll
+            for (int c = 0; c < 2; ++c)
+                if (z0 + k < z1 && c < rows) {
+#pragma unroll
+                    for (int n = 0; n < 3; ++n) {
+                        const int64_t r = n * L3 + r1 + k * P + c * H;
+                        sv.at(r, w) = sm[n * N + o0 + k * P + c * H];
+                        if (e_store)
+                            ev.at(r, w) = acc[k][c][n];
+                        else
+                            xor_into(&ev.at(r, w), acc[k][c][n]);
+                    }
+                }
+    }
+}
+
+// Word rows <-> contiguous columns: in [R][W] -> out [W][R] and back (kXor: XORed into the
+// rows), in 32 x 32 tiles through shared memory, 256-byte runs on both sides.
+constexpr int kTurn = 32;
+
+__global__ void __launch_bounds__(256) k_to_columns(int64_t R, int64_t W, const uint64_t* __restrict__ in,
+                                                    uint64_t* __restrict__ out)
+{
+    __shared__ uint64_t tile[kTurn][kTurn + 1];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t r0 = (int64_t)blockIdx.x * kTurn, w0 = (int64_t)blockIdx.y * kTurn;
+#pragma unroll
+    for (int i = 0; i < kTurn; i += 8)
+        if (r0 + ty + i < R && w0 + tx < W) tile[ty + i][tx] = in[(r0 + ty + i) * W + w0 + tx];
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kTurn; i += 8)
+        if (w0 + ty + i < W && r0 + tx < R) out[(w0 + ty + i) * R + r0 + tx] = tile[tx][ty + i];
+}
+
+template <bool kXor>
+__global__ void __launch_bounds__(256) k_from_columns(int64_t R, int64_t W, const uint64_t* __restrict__ in,
+                                                      uint64_t* __restrict__ out)
+{
+    __shared__ uint64_t tile[kTurn][kTurn + 1];
+    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+    const int64_t r0 = (int64_t)blockIdx.x * kTurn, w0 = (int64_t)blockIdx.y * kTurn;
+    uint64_t was[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int i = 0; i < kTurn; i += 8) {
+        if (w0 + ty + i < W && r0 + tx < R) tile[ty + i][tx] = __ldcs(&in[(w0 + ty + i) * R + r0 + tx]);
+        if (kXor && r0 + ty + i < R && w0 + tx < W) was[i / 8] = out[(r0 + ty + i) * W + w0 + tx];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kTurn; i += 8)
+        if (r0 + ty + i < R && w0 + tx < W) out[(r0 + ty + i) * W + w0 + tx] = was[i / 8] ^ tile[tx][ty + i];
+}
+
+// Blocks of a cluster for lattice size L: the choice with the most busy SMs, counting the blocks
+// that can be resident with about 200 KB each (cudaOccupancyMaxActiveClusters on GB300) and the
+// share of them that a split of L planes into unequal slabs leaves waiting.  A thread takes at
+// most four planes of its row pair (96 registers of state).  cluster 0: none fits.
+struct SlabShape {
+    int cluster, zt, z, threads;
+    size_t smem;
+};
+
+SlabShape slab_shape(int L)
+{
+    constexpr int resident[kMaxCluster + 1] = {0, 152, 152, 138, 144, 140, 138, 105, 120};
+    SlabShape best{0, 0, 0, 0, 0};
+    double busy = 0.0;
+    const int per = (L + 1) / 2 * L;
+    for (int c = 1; c <= kMaxCluster && c <= L; ++c) {
+        const int most = (L + c - 1) / c;
+        const size_t smem = (size_t)48 * L * L * most;
+        if (smem + 1024 > kColumnSmem) continue;
+        const double b = resident[c] * (double)L / (c * most);
+        if (b <= busy) continue;
+        // planes per thread: 4 with up to 512 threads, 3 with up to 640, 2 with up to 896
+        for (int z = std::min(4, most); z >= 1; --z) {
+            const int zt = (most + z - 1) / z, threads = (per * zt + 31) / 32 * 32;
+            if (threads > (z == 4 ? 512 : z == 3 ? 640 : 896)) continue;
+            busy = b;
+            best = SlabShape{c, zt, z, threads, smem};
+            break;
+        }
+    }
+    return best;
+}
+
+template <int kZ, int kT>
+t3d_status launch_slab_k(const ItemDesc& d, const ColumnProgram& pr, const SlabShape& c, int kind,
+                         const ColumnView& sv, const ColumnView& ev, int e_store, cudaStream_t st)
+{
+    auto kernel = k_slab<kZ, kT>;
+    T3D_TRY(allow_dynamic_smem((const void*)kernel, c.smem));
+    const int64_t words = d.nw ? d.nw : d.W;
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof(cfg));
+    cfg.gridDim = dim3((unsigned)(c.cluster * std::min<int64_t>(words, 0x7fffffffLL / c.cluster)));
+    cfg.blockDim = dim3((unsigned)c.threads);
+    cfg.dynamicSmemBytes = c.smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)c.cluster;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    ProfScope prof(kind, st);
+    T3D_CUDA_CHECK(cudaLaunchKernelEx(&cfg, kernel, d, pr, c.cluster, sv, ev, e_store));
+    return T3D_OK;
+}
+
+// A word's column is strided by the row length, so a block reads 32-byte sectors for 8-byte words.
+// From kTurnWords words on the syndrome is turned into contiguous columns first (in the item's
+// scratch array), the gathered flips are written as columns into the syndrome's own array, and both
+// are turned back.
+constexpr int64_t kTurnWords = 64;
+
+t3d_status launch_slab(const ItemDesc& d, ColumnProgram pr, int kind, cudaStream_t st)
+{
+    const SlabShape c = slab_shape(d.lat.L);
+    pr.zt = c.zt;
+    const int64_t R = 3LL * d.lat.L3;
+    const bool turn = d.tmp && !d.live && !d.nw && d.W >= kTurnWords && (d.W + kTurn - 1) / kTurn <= 65535;
+    ColumnView sv{d.s, d.W, 1}, ev{d.e, d.W, 1};
+    const dim3 grid((unsigned)((R + kTurn - 1) / kTurn), (unsigned)((d.W + kTurn - 1) / kTurn));
+    if (turn) {
+        sv = ColumnView{d.tmp, 1, R};
+        ev = ColumnView{d.s, 1, R};
+        ProfScope prof(kind, st);
+        k_to_columns<<<grid, 256, 0, st>>>(R, d.W, d.s, d.tmp);
+        T3D_LAUNCH_CHECK("syndrome columns");
+    }
+    if (c.z == 4)
+        T3D_TRY((launch_slab_k<4, 512>(d, pr, c, kind, sv, ev, turn, st)));
+    else if (c.z == 3)
+        T3D_TRY((launch_slab_k<3, 640>(d, pr, c, kind, sv, ev, turn, st)));
+    else
+        T3D_TRY((launch_slab_k<2, 896>(d, pr, c, kind, sv, ev, turn, st)));
+    if (turn) {
+        ProfScope prof(kind, st);
+        k_from_columns<true><<<grid, 256, 0, st>>>(R, d.W, d.s, d.e);
+        T3D_LAUNCH_CHECK("flips into the error state");
+        k_from_columns<false><<<grid, 256, 0, st>>>(R, d.W, d.tmp, d.s);
+        T3D_LAUNCH_CHECK("syndrome rows");
+    }
+    return T3D_OK;
+}
+
 size_t column_bytes(int L, bool e_smem) { return (size_t)L * L * L * (e_smem ? 72 : 48); }
 
 bool e_fits(int L) { return column_bytes(L, true) <= kColumnSmem; }
@@ -336,6 +728,15 @@ uint64_t schedule_bits(const char* schedule, int slen)
 
 bool column_fits(int L) { return column_bytes(L, false) <= kColumnSmem; }
 
+// Whether a schedule of n_apply applications runs on chip.  Above L = 16 the columns are turned
+// first and back afterwards from kTurnWords words on (about 2.2 ms at L = 32, 10^5 samples, five
+// applications' gain: FFPFF 5.6 -> 4.8 ms, PFFPFF x 32 in 33 -> 20 ms); below that a step by
+// step schedule is bound by its launches.
+bool sweeps_fit(int L, int64_t words, int n_apply)
+{
+    return column_fits(L) || (slab_shape(L).cluster > 0 && (words < kTurnWords || n_apply >= 5));
+}
+
 t3d_status launch_column_sweeps(const ItemDesc& d, const char* schedule, int slen, int n_apply, uint32_t sweep0,
                                 uint64_t seed, uint32_t cycle, cudaStream_t st)
 {
@@ -347,7 +748,8 @@ t3d_status launch_column_sweeps(const ItemDesc& d, const char* schedule, int sle
     pr.n_apply = n_apply;
     pr.sweep0 = sweep0;
     pr.cycle0 = cycle;
-    return launch_column<false>(d, pr, pr.sched ? T3D_K_PFLIP : T3D_K_FLIP, st);
+    const int kind = pr.sched ? T3D_K_PFLIP : T3D_K_FLIP;
+    return e_fits(d.lat.L) ? launch_column<false>(d, pr, kind, st) : launch_slab(d, pr, kind, st);
 }
 
 t3d_status launch_column_until_clear(const ItemDesc& d, int max_sweeps, int32_t* sweeps_done, cudaStream_t st)
@@ -359,7 +761,7 @@ t3d_status launch_column_until_clear(const ItemDesc& d, int max_sweeps, int32_t*
     pr.n_apply = max_sweeps;
     pr.until_clear = 1;
     pr.sweeps_done = sweeps_done;
-    return launch_column<false>(d, pr, T3D_K_FLIP, st);
+    return e_fits(d.lat.L) ? launch_column<false>(d, pr, T3D_K_FLIP, st) : launch_slab(d, pr, T3D_K_FLIP, st);
 }
 
 t3d_status launch_column_run(const ItemDesc& d, int cycles, uint32_t cycle0, uint64_t thr_p, uint64_t thr_q,

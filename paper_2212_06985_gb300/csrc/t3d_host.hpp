@@ -120,10 +120,11 @@ t3d_status launch_flip_until_clear(ItemTable& tab, int max_sweeps, int32_t* swee
 t3d_status launch_sweeps(ItemTable& tab, const char* schedule, int slen, int n_apply,
                          uint32_t sweep0, uint64_t seed, uint32_t cycle, cudaStream_t st);
 t3d_status launch_logical(ItemTable& tab, cudaStream_t st);
-// Lattices whose syndrome and flip words fit one SM (t3d_column.cu, L <= 16): a schedule, a flip
-// until clear, or whole runs in one launch per item.  No scratch (ItemDesc::tmp, stop) is used.
+// Lattices whose syndrome and flip words fit one SM or a cluster of them (t3d_column.cu): a
+// schedule, a flip until clear, or a whole run in one launch per item.  No scratch (ItemDesc::tmp, stop) is used.
 struct ItemDesc;
-bool column_fits(int L);
+bool column_fits(int L);   // whole runs (L <= 16)
+bool sweeps_fit(int L, int64_t words, int n_apply);   // schedules and flip until clear (L <= 32)
 t3d_status launch_column_sweeps(const ItemDesc& d, const char* schedule, int slen, int n_apply, uint32_t sweep0,
                                 uint64_t seed, uint32_t cycle, cudaStream_t st);
 t3d_status launch_column_until_clear(const ItemDesc& d, int max_sweeps, int32_t* sweeps_done, cudaStream_t st);

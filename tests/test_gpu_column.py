@@ -1,6 +1,7 @@
-"""Lattices kept on one SM (t3d_column.cu) against the oracle, bit for bit: the smallest (several
-words per block), odd ones, the largest with the error words in shared memory (L = 14) and beside
-it (15, 16), the first larger one that goes step by step (17); ragged batches, a starting error,
+"""Lattices kept on one SM or a cluster (t3d_column.cu) against the oracle, bit for bit: the smallest
+(several words per block), odd ones, the largest with the error words in shared memory (L = 14) and
+beside it (15, 16), every cluster size the larger ones take (17 .. 32, equal and unequal slabs), the
+first that goes step by step (33); ragged batches, a starting error,
 schedules that do and do not cycle, more than one cycle, sample0, and the noise extremes 0 and 1."""
 import numpy as np
 import pytest
@@ -40,7 +41,7 @@ def test_runs_match_oracle(L, S, T, p, schedule, n_apply, perfect, graph):
     assert np.array_equal(mask.cpu().numpy()[:k], ora_mask)
 
 
-@pytest.mark.parametrize("L", [2, 3, 4, 9, 14, 15, 16])
+@pytest.mark.parametrize("L", [2, 3, 4, 9, 14, 15, 16, 17, 20, 23, 26, 27, 30, 31, 32, 33])
 @pytest.mark.parametrize("S", [40, 200])
 def test_sweeps_and_until_clear_match_oracle(L, S):
     n, W = 3 * L ** 3, inp.words_for(S)
