@@ -33,7 +33,10 @@ namespace {
 
 using namespace bpm;
 
-constexpr int kBpThreads = 256;
+// Four sites per block: blocks retire, and their messages' rows are requested again, in finer
+// steps than with 256 threads (16 iterations of 12,480 samples at L = 32: 106.2 -> 104.1 ms; 64
+// threads 103.3, slower at L = 16 and 24; 512 threads 111.0).
+constexpr int kBpThreads = 128;
 constexpr int kWord = 64;  // samples per message row (one bit-sliced word)
 constexpr float kMsgClamp = 30.0f;
 // Message offsets within one word-row block, 3 L^3 * 256 floats, stay below 2^31.
@@ -149,11 +152,13 @@ __device__ __forceinline__ bool site_warp(const Lattice& lat, int64_t lb, SiteWa
 // Offset of edge (d, site)'s 4x64 message block within a word-row block.
 __device__ __forceinline__ int msg_off(int site, int d) { return (site * 3 + d) * (4 * kWord); }
 
-// Where an iteration takes the syndrome from: the caller's bit-sliced words
-// (kSynWords), the same and also a per-word copy for later iterations
-// (kSynWordsSave: the three faces' words of a site side by side), or that
-// copy (kSynSaved), which brings a site's syndrome in one 32-byte load.
-enum SynMode { kSynWords = 0, kSynWordsSave = 1, kSynSaved = 2 };
+// Where an iteration takes the syndrome from: the caller's bit-sliced words (kSynWords) or a
+// per-word copy with the three faces' words of a site side by side (kSynSaved), which brings a
+// site's syndrome in one 32-byte load.  kSynFirstTwo computes the first two iterations at once
+// from that copy: the first one's messages are +-m1 by the syndrome bit of the face that sends
+// them, so nothing is read but 24 syndrome words a site, and nothing of the first iteration is
+// written (16 iterations of 12,480 samples at L = 32: 109.5 -> 106.2 ms).
+enum SynMode { kSynWords = 0, kSynSaved = 1, kSynFirstTwo = 2 };
 
 struct __align__(32) Syn3 {
     uint64_t f[4];  // faces 0..2, padding
@@ -169,7 +174,7 @@ __device__ __forceinline__ bool sbit(uint64_t word, int lane, int j) { return (w
 // every output is (-1)^{s_f} m1 with m1 = 2 atanh(tq tanh(l0/2)^3) computed
 // once on the host, and the launch only writes.
 template <int kSyn>
-__global__ void __launch_bounds__(kBpThreads, 4)
+__global__ void __launch_bounds__(kBpThreads, 8)
 k_bp_step(const __grid_constant__ ItemTable tab, float l0, TD q, float m1)
 {
     for_each_item_block(tab, [&](const ItemDesc& d, int64_t lb) {
@@ -181,7 +186,7 @@ k_bp_step(const __grid_constant__ ItemTable tab, float l0, TD q, float m1)
     const int lane = threadIdx.x & 31;
     Syn3* __restrict__ syn = reinterpret_cast<Syn3*>(d.syn);
     uint64_t s0, s1, s2;
-    if (kSyn == kSynSaved) {
+    if (kSyn != kSynWords) {
         const Syn3 v = syn[sw.w * lat.L3 + sw.site];
         s0 = v.f[0];
         s1 = v.f[1];
@@ -190,14 +195,6 @@ k_bp_step(const __grid_constant__ ItemTable tab, float l0, TD q, float m1)
         s0 = d.s[((int64_t)0 * lat.L3 + sw.site) * W + sw.w];
         s1 = d.s[((int64_t)1 * lat.L3 + sw.site) * W + sw.w];
         s2 = d.s[((int64_t)2 * lat.L3 + sw.site) * W + sw.w];
-        if (kSyn == kSynWordsSave && lane == 0) {
-            Syn3 v;
-            v.f[0] = s0;
-            v.f[1] = s1;
-            v.f[2] = s2;
-            v.f[3] = 0;
-            syn[sw.w * lat.L3 + sw.site] = v;
-        }
     }
     const int64_t wbase = sw.w * (int64_t)lat.L3 * (3 * 4 * kWord) + 2 * lane;
     const int r = sw.site, rx = sw.nb[0], ry = sw.nb[1], rz = sw.nb[2];
@@ -206,7 +203,7 @@ k_bp_step(const __grid_constant__ ItemTable tab, float l0, TD q, float m1)
     const int oXy = msg_off(ry, 0), oXz = msg_off(rz, 0);
     const int oYx = msg_off(rx, 1), oYz = msg_off(rz, 1);
     const int oZx = msg_off(rx, 2), oZy = msg_off(ry, 2);
-    if (!d.msg_in) {
+    if (kSyn != kSynFirstTwo && !d.msg_in) {
         float* o = d.msg_out + wbase;
         auto PUT1 = [&](int off, uint64_t sw) {
             const float a = sbit(sw, lane, 0) ? -m1 : m1, b = sbit(sw, lane, 1) ? -m1 : m1;
@@ -229,17 +226,36 @@ k_bp_step(const __grid_constant__ ItemTable tab, float l0, TD q, float m1)
     // inputs [face][edge] for the lane's two samples, edges in face_edges order
     float2 in[3][4];
     {
+        // slot k of an edge comes from the face listed k-th for it: x-edge at q faces 2 at q,
+        // 2 at q - e_y, 1 at q, 1 at q - e_z; y-edge 2 at q, 2 at q - e_x, 0 at q, 0 at q - e_z;
+        // z-edge 1 at q, 1 at q - e_x, 0 at q, 0 at q - e_y.  M(o, k, n, q): slot k of the edge whose
+        // block is at o, which face (n, q) sends.
         const float* m = d.msg_in + wbase;
-        auto M = [&](int o, int k) { return *reinterpret_cast<const float2*>(m + o + k * kWord); };
-        const float2 xr0 = M(oXr, 0), xr1 = M(oXr, 1), xr2 = M(oXr, 2), xr3 = M(oXr, 3);
-        const float2 yr0 = M(oYr, 0), yr1 = M(oYr, 1), yr2 = M(oYr, 2), yr3 = M(oYr, 3);
-        const float2 zr0 = M(oZr, 0), zr1 = M(oZr, 1), zr2 = M(oZr, 2), zr3 = M(oZr, 3);
-        const float2 yz0 = M(oYz, 0), yz1 = M(oYz, 1), yz2 = M(oYz, 2);
-        const float2 zy0 = M(oZy, 0), zy1 = M(oZy, 1), zy2 = M(oZy, 2);
-        const float2 xz0 = M(oXz, 0), xz1 = M(oXz, 1), xz2 = M(oXz, 2);
-        const float2 zx0 = M(oZx, 0), zx2 = M(oZx, 2), zx3 = M(oZx, 3);
-        const float2 xy0 = M(oXy, 0), xy2 = M(oXy, 2), xy3 = M(oXy, 3);
-        const float2 yx0 = M(oYx, 0), yx2 = M(oYx, 2), yx3 = M(oYx, 3);
+        const uint32_t* __restrict__ D =
+            reinterpret_cast<const uint32_t*>(syn + sw.w * lat.L3) + (lane >> 4);   // the lane's half of a word
+        const int sh = 2 * (lane & 15);
+        int bx = 0, by = 0, bz = 0;   // r - e_x, r - e_y, r - e_z as site deltas
+        if (kSyn == kSynFirstTwo) {
+            const Coord c = site_coord(lat, r);
+            bx = c.x[0] == 0 ? lat.L - 1 : -1;
+            by = c.x[1] == 0 ? lat.L2 - lat.L : -lat.L;
+            bz = c.x[2] == 0 ? lat.L3 - lat.L2 : -lat.L2;
+        }
+        auto M = [&](int o, int k, int n, int q) {
+            if (kSyn != kSynFirstTwo) return *reinterpret_cast<const float2*>(m + o + k * kWord);
+            // the two syndrome bits as sign bits of m1
+            const uint32_t v = D[q * 8 + 2 * n] >> sh, mb = __float_as_uint(m1);
+            return make_float2(__uint_as_float(mb ^ (v << 31)), __uint_as_float(mb ^ ((v << 30) & 0x80000000u)));
+        };
+        const float2 xr0 = M(oXr, 0, 2, r), xr1 = M(oXr, 1, 2, r + by), xr2 = M(oXr, 2, 1, r), xr3 = M(oXr, 3, 1, r + bz);
+        const float2 yr0 = M(oYr, 0, 2, r), yr1 = M(oYr, 1, 2, r + bx), yr2 = M(oYr, 2, 0, r), yr3 = M(oYr, 3, 0, r + bz);
+        const float2 zr0 = M(oZr, 0, 1, r), zr1 = M(oZr, 1, 1, r + bx), zr2 = M(oZr, 2, 0, r), zr3 = M(oZr, 3, 0, r + by);
+        const float2 yz0 = M(oYz, 0, 2, rz), yz1 = M(oYz, 1, 2, rz + bx), yz2 = M(oYz, 2, 0, rz);
+        const float2 zy0 = M(oZy, 0, 1, ry), zy1 = M(oZy, 1, 1, ry + bx), zy2 = M(oZy, 2, 0, ry);
+        const float2 xz0 = M(oXz, 0, 2, rz), xz1 = M(oXz, 1, 2, rz + by), xz2 = M(oXz, 2, 1, rz);
+        const float2 zx0 = M(oZx, 0, 1, rx), zx2 = M(oZx, 2, 0, rx), zx3 = M(oZx, 3, 0, rx + by);
+        const float2 xy0 = M(oXy, 0, 2, ry), xy2 = M(oXy, 2, 1, ry), xy3 = M(oXy, 3, 1, ry + bz);
+        const float2 yx0 = M(oYx, 0, 2, rx), yx2 = M(oYx, 2, 0, rx), yx3 = M(oYx, 3, 0, rx + bz);
         const float2 L0 = f2(l0);
         auto A = [](float2 a, float2 b) { return __fadd2_rn(a, b); };
         const float2 xs = A(A(L0, xr1), xr3), ys = A(A(L0, yr1), yr3), zs = A(A(L0, zr1), zr3);
@@ -279,6 +295,43 @@ k_bp_step(const __grid_constant__ ItemTable tab, float l0, TD q, float m1)
     PUT(oXy + 1 * kWord, y[1]);
     PUT(oYr + 0 * kWord, y[2]);
     PUT(oYx + 1 * kWord, y[3]);
+    });
+}
+
+// The chunk's syndrome words copied to [word][site], a site's three faces side by side.  One thread
+// per (site, word), words fastest, so the rows are read coalesced and each thread writes one
+// 32-byte sector.
+constexpr int kSynWordsPerRow = 32;
+constexpr int kSynSitesPerBlock = kBpThreads / kSynWordsPerRow;
+
+__host__ __device__ __forceinline__ int64_t syn_blocks(int L3, int64_t words)
+{
+    return ((L3 + kSynSitesPerBlock - 1) / kSynSitesPerBlock) *
+           ((words + kSynWordsPerRow - 1) / kSynWordsPerRow);
+}
+
+// (site, word) of a thread of such a launch.
+__device__ __forceinline__ bool syn_thread(const ItemDesc& d, int64_t lb, int& r, int64_t& w)
+{
+    const int64_t site_tiles = (d.lat.L3 + kSynSitesPerBlock - 1) / kSynSitesPerBlock;
+    const int64_t word_tile = lb / site_tiles;
+    r = (int)((lb - word_tile * site_tiles) * kSynSitesPerBlock + (threadIdx.x / kSynWordsPerRow));
+    w = word_tile * kSynWordsPerRow + (threadIdx.x % kSynWordsPerRow);
+    return r < d.lat.L3 && w < d.words && word_live(d, w);
+}
+
+__global__ void __launch_bounds__(kBpThreads)
+k_bp_copy_syndrome(const __grid_constant__ ItemTable tab)
+{
+    for_each_item_block(tab, [&](const ItemDesc& d, int64_t lb) {
+    int r;
+    int64_t w;
+    if (!syn_thread(d, lb, r, w)) return;
+    Syn3 v;
+#pragma unroll
+    for (int n = 0; n < 3; ++n) v.f[n] = d.s[((int64_t)n * d.lat.L3 + r) * d.W + w];
+    v.f[3] = 0;
+    reinterpret_cast<Syn3*>(d.syn)[w * d.lat.L3 + r] = v;
     });
 }
 
@@ -370,26 +423,14 @@ k_bp_decide(const __grid_constant__ ItemTable tab, float l0)
 //   n=0: d(y,r) ^ d(y,r+e_z) ^ d(z,r) ^ d(z,r+e_y)
 //   n=1: d(x,r) ^ d(x,r+e_z) ^ d(z,r) ^ d(z,r+e_x)
 //   n=2: d(x,r) ^ d(x,r+e_y) ^ d(y,r) ^ d(y,r+e_x).
-constexpr int kSynWordsPerRow = 32;
-constexpr int kSynSitesPerBlock = kBpThreads / kSynWordsPerRow;
-
-__host__ __device__ __forceinline__ int64_t syn_blocks(int L3, int64_t words)
-{
-    return ((L3 + kSynSitesPerBlock - 1) / kSynSitesPerBlock) *
-           ((words + kSynWordsPerRow - 1) / kSynWordsPerRow);
-}
-
 __global__ void __launch_bounds__(kBpThreads)
 k_bp_syndrome(const __grid_constant__ ItemTable tab)
 {
     for_each_item_block(tab, [&](const ItemDesc& d, int64_t lb) {
     const Lattice lat = d.lat;
-    const int64_t site_tiles = (lat.L3 + kSynSitesPerBlock - 1) / kSynSitesPerBlock;
-    const int64_t word_tile = lb / site_tiles;
-    const int r = (int)((lb - word_tile * site_tiles) * kSynSitesPerBlock + (threadIdx.x / kSynWordsPerRow));
-    const int64_t w = word_tile * kSynWordsPerRow + (threadIdx.x % kSynWordsPerRow);
-    if (r >= lat.L3 || w >= d.words) return;
-    if (!word_live(d, w)) return;
+    int r;
+    int64_t w;
+    if (!syn_thread(d, lb, r, w)) return;
     const Coord rc = site_coord(lat, r);
     const int step[3] = {1, lat.L, lat.L2};
     int nb[3];
@@ -444,24 +485,38 @@ void set_blocks(ItemTable& tab)
     finish_table(tab);
 }
 
+void set_syn_blocks(ItemTable& tab)
+{
+    for (int i = 0; i < tab.n; ++i) {
+        ItemDesc& d = tab.it[i];
+        d.blocks = syn_blocks(d.lat.L3, d.words);
+        d.live_wpu = kSynWordsPerRow;
+        d.live_bpu = (d.lat.L3 + kSynSitesPerBlock - 1) / kSynSitesPerBlock;
+    }
+    finish_table(tab);
+}
+
+t3d_status launch_copy_syndrome(ItemTable& tab, cudaStream_t st)
+{
+    set_syn_blocks(tab);
+    ProfScope prof(T3D_K_BP_STEP, st);
+    k_bp_copy_syndrome<<<persistent_grid((const void*)k_bp_copy_syndrome, kBpThreads, T3D_K_BP_DECIDE, tab.prefix[tab.n],
+                                         has_live(tab)),
+                         kBpThreads, 0, st>>>(tab);
+    T3D_LAUNCH_CHECK("bp syndrome copy");
+    return T3D_OK;
+}
+
 t3d_status launch_step(ItemTable& tab, int mode, double p, double q_meas, cudaStream_t st)
 {
     set_blocks(tab);
     const int64_t blocks = tab.prefix[tab.n];
     const bool live = has_live(tab);
     ProfScope prof(T3D_K_BP_STEP, st);
-    if (mode == kSynWordsSave)
-        k_bp_step<kSynWordsSave><<<persistent_grid((const void*)k_bp_step<kSynWordsSave>, kBpThreads,
-                                                   T3D_K_BP_STEP, blocks, live),
-                                   kBpThreads, 0, st>>>(tab, prior(p), meas_pair(q_meas), first_message(p, q_meas));
-    else if (mode == kSynSaved)
-        k_bp_step<kSynSaved><<<persistent_grid((const void*)k_bp_step<kSynSaved>, kBpThreads, T3D_K_BP_STEP,
-                                               blocks, live),
-                               kBpThreads, 0, st>>>(tab, prior(p), meas_pair(q_meas), first_message(p, q_meas));
-    else
-        k_bp_step<kSynWords><<<persistent_grid((const void*)k_bp_step<kSynWords>, kBpThreads, T3D_K_BP_STEP,
-                                               blocks, live),
-                               kBpThreads, 0, st>>>(tab, prior(p), meas_pair(q_meas), first_message(p, q_meas));
+    auto kernel = mode == kSynFirstTwo ? k_bp_step<kSynFirstTwo>
+                                       : (mode == kSynSaved ? k_bp_step<kSynSaved> : k_bp_step<kSynWords>);
+    kernel<<<persistent_grid((const void*)kernel, kBpThreads, T3D_K_BP_STEP, blocks, live), kBpThreads, 0, st>>>(
+        tab, prior(p), meas_pair(q_meas), first_message(p, q_meas));
     T3D_LAUNCH_CHECK("bp step");
     return T3D_OK;
 }
@@ -475,13 +530,7 @@ t3d_status launch_decide(ItemTable& tab, double p, cudaStream_t st)
                       kBpThreads, 0, st>>>(tab, prior(p));
         T3D_LAUNCH_CHECK("bp decide");
     }
-    for (int i = 0; i < tab.n; ++i) {
-        ItemDesc& d = tab.it[i];
-        d.blocks = syn_blocks(d.lat.L3, d.words);
-        d.live_wpu = kSynWordsPerRow;
-        d.live_bpu = (d.lat.L3 + kSynSitesPerBlock - 1) / kSynSitesPerBlock;
-    }
-    finish_table(tab);
+    set_syn_blocks(tab);
     ProfScope prof(T3D_K_BP_DECIDE, st);
     k_bp_syndrome<<<persistent_grid((const void*)k_bp_syndrome, kBpThreads, T3D_K_BP_DECIDE, tab.prefix[tab.n], has_live(tab)),
                     kBpThreads, 0, st>>>(tab);
@@ -552,12 +601,14 @@ t3d_status launch_bp(const ItemTable& items, double p, double q_meas, int iters,
         float* A[kMaxItems];
         float* B[kMaxItems];
         ItemTable tab = chunk_table(items, bufs, chunk_words, r, llr_out, A, B);
-        for (int it = 0; it < iters; ++it) {
+        // the first two iterations in one launch (a single one reads the bit-sliced words)
+        if (iters >= 2) T3D_TRY(launch_copy_syndrome(tab, st));
+        for (int it = iters >= 2 ? 1 : 0; it < iters; ++it) {
             for (int k = 0; k < tab.n; ++k) {
-                tab.it[k].msg_in = it == 0 ? nullptr : B[k];
+                tab.it[k].msg_in = it <= 1 ? nullptr : B[k];
                 tab.it[k].msg_out = A[k];
             }
-            T3D_TRY(launch_step(tab, it == 0 ? kSynWordsSave : kSynSaved, p, q_meas, st));
+            T3D_TRY(launch_step(tab, it == 0 ? kSynWords : (it == 1 ? kSynFirstTwo : kSynSaved), p, q_meas, st));
             for (int k = 0; k < tab.n; ++k) std::swap(A[k], B[k]);
         }
         for (int k = 0; k < tab.n; ++k) tab.it[k].msg_in = iters > 0 ? B[k] : nullptr;
@@ -576,7 +627,8 @@ t3d_status autotune_bp(const ItemTable& items, double p, double q_meas, float* c
         tab.it[k].msg_in = nullptr;
         tab.it[k].msg_out = A[k];
     }
-    T3D_TRY(launch_step(tab, kSynWordsSave, p, q_meas, st));  // realistic messages in A
+    T3D_TRY(launch_copy_syndrome(tab, st));
+    T3D_TRY(launch_step(tab, kSynFirstTwo, p, q_meas, st));  // realistic messages in A
     for (int k = 0; k < tab.n; ++k) {
         tab.it[k].msg_in = A[k];
         tab.it[k].msg_out = B[k];
