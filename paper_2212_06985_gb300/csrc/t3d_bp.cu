@@ -42,48 +42,6 @@ constexpr float kMsgClamp = 30.0f;
 // Message offsets within one word-row block, 3 L^3 * 256 floats, stay below 2^31.
 constexpr int kMaxBpL = 128;
 
-// The check node on a lane's two samples at once with the packed two-wide FP32
-// instructions (__fadd2_rn, __fmul2_rn, __ffma2_rn): every operation is the scalar
-// one of td_of / td_mul / two_atanh (t3d_bp_math.cuh) in the same order and
-// rounding, applied to both samples, so the messages are bit for bit those of the
-// scalar code; the MUFU approximations and the selects stay per sample.
-struct TD2 {
-    float2 t, d;
-};
-
-__device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
-
-__device__ __forceinline__ TD2 td2_mul(const TD2& A, const TD2& B)
-{
-    return TD2{__fmul2_rn(A.t, B.t), __ffma2_rn(A.t, B.d, A.d)};
-}
-
-__device__ __forceinline__ TD2 td2_of(float2 x)
-{
-    const float2 a = make_float2(fabsf(x.x), fabsf(x.y));
-    const float2 m = __fmul2_rn(make_float2(-a.x, -a.y), f2(kLog2e));
-    const float2 E = make_float2(ex2_approx(m.x), ex2_approx(m.y));
-    const float2 e1 = __fadd2_rn(f2(1.0f), E);
-    const float2 r = make_float2(rcp_approx(e1.x), rcp_approx(e1.y));
-    float2 h = __ffma2_rn(a, f2(-1.0f / 24.0f), f2(1.0f / 6.0f));
-    h = __ffma2_rn(a, h, f2(-0.5f));
-    h = __ffma2_rn(a, h, f2(1.0f));
-    const float2 ah = __fmul2_rn(a, h);
-    const float2 ome = __fadd2_rn(f2(1.0f), make_float2(-E.x, -E.y));
-    const float2 om = make_float2(a.x < 0.1f ? ah.x : ome.x, a.y < 0.1f ? ah.y : ome.y);
-    return TD2{__fmul2_rn(om, r), __fmul2_rn(__fadd2_rn(E, E), r)};
-}
-
-__device__ __forceinline__ float2 two_atanh2(float2 P, float2 D)
-{
-    const float2 u = __fmul2_rn(P, P);
-    const float2 poly = __ffma2_rn(u, __ffma2_rn(u, f2(1.0f / 5.0f), f2(1.0f / 3.0f)), f2(1.0f));
-    const float2 series = __fmul2_rn(__fmul2_rn(f2(2.0f), P), poly);
-    const float2 arg = __fmul2_rn(__fadd2_rn(f2(1.0f), P), make_float2(rcp_approx(D.x), rcp_approx(D.y)));
-    const float2 logv = __fmul2_rn(f2(kLn2), make_float2(lg2_approx(arg.x), lg2_approx(arg.y)));
-    return make_float2(P.x < 0.05f ? series.x : logv.x, P.y < 0.05f ? series.y : logv.y);
-}
-
 // Eq. 2 for the four edges of one face on both samples of a lane: y[j] from the other three
 // inputs and the measurement-variable pair q; the sign of y[j] is (-1)^{s_f} times the product
 // of the other inputs' signs, the XOR of their IEEE sign bits.  Bit for bit the scalar check

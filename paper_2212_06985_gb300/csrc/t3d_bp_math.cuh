@@ -111,6 +111,79 @@ __device__ __forceinline__ void check_node(const float (&x)[K], bool syn, float 
     }
 }
 
+// The check node on a lane's two samples at once with the packed two-wide FP32
+// instructions (__fadd2_rn, __fmul2_rn, __ffma2_rn): every operation is the scalar
+// one of td_of / td_mul / two_atanh (t3d_bp_math.cuh) in the same order and
+// rounding, applied to both samples, so the messages are bit for bit those of the
+// scalar code; the MUFU approximations and the selects stay per sample.
+struct TD2 {
+    float2 t, d;
+};
+
+__device__ __forceinline__ float2 f2(float v) { return make_float2(v, v); }
+
+__device__ __forceinline__ TD2 td2_mul(const TD2& A, const TD2& B)
+{
+    return TD2{__fmul2_rn(A.t, B.t), __ffma2_rn(A.t, B.d, A.d)};
+}
+
+__device__ __forceinline__ TD2 td2_of(float2 x)
+{
+    const float2 a = make_float2(fabsf(x.x), fabsf(x.y));
+    const float2 m = __fmul2_rn(make_float2(-a.x, -a.y), f2(kLog2e));
+    const float2 E = make_float2(ex2_approx(m.x), ex2_approx(m.y));
+    const float2 e1 = __fadd2_rn(f2(1.0f), E);
+    const float2 r = make_float2(rcp_approx(e1.x), rcp_approx(e1.y));
+    float2 h = __ffma2_rn(a, f2(-1.0f / 24.0f), f2(1.0f / 6.0f));
+    h = __ffma2_rn(a, h, f2(-0.5f));
+    h = __ffma2_rn(a, h, f2(1.0f));
+    const float2 ah = __fmul2_rn(a, h);
+    const float2 ome = __fadd2_rn(f2(1.0f), make_float2(-E.x, -E.y));
+    const float2 om = make_float2(a.x < 0.1f ? ah.x : ome.x, a.y < 0.1f ? ah.y : ome.y);
+    return TD2{__fmul2_rn(om, r), __fmul2_rn(__fadd2_rn(E, E), r)};
+}
+
+__device__ __forceinline__ float2 two_atanh2(float2 P, float2 D)
+{
+    const float2 u = __fmul2_rn(P, P);
+    const float2 poly = __ffma2_rn(u, __ffma2_rn(u, f2(1.0f / 5.0f), f2(1.0f / 3.0f)), f2(1.0f));
+    const float2 series = __fmul2_rn(__fmul2_rn(f2(2.0f), P), poly);
+    const float2 arg = __fmul2_rn(__fadd2_rn(f2(1.0f), P), make_float2(rcp_approx(D.x), rcp_approx(D.y)));
+    const float2 logv = __fmul2_rn(f2(kLn2), make_float2(lg2_approx(arg.x), lg2_approx(arg.y)));
+    return make_float2(P.x < 0.05f ? series.x : logv.x, P.y < 0.05f ? series.y : logv.y);
+}
+
+// check_node on a lane's two samples: the same products in the same order (a product with the
+// neutral pair (1, 0) is exact, so the ends of the prefix and suffix chains are the inputs
+// themselves), bit for bit.
+template <int K>
+__device__ __forceinline__ void check_node2(const float2 (&x)[K], bool syn0, bool syn1, float2 (&out)[K])
+{
+    static_assert(K >= 3, "at least three inputs");
+    TD2 v[K], suf[K];
+    uint32_t sa0 = syn0 ? 0x80000000u : 0u, sa1 = syn1 ? 0x80000000u : 0u;
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        v[i] = td2_of(x[i]);
+        sa0 ^= __float_as_uint(x[i].x);
+        sa1 ^= __float_as_uint(x[i].y);
+    }
+    suf[K - 2] = v[K - 1];
+#pragma unroll
+    for (int i = K - 3; i >= 0; --i) suf[i] = td2_mul(v[i + 1], suf[i + 1]);
+    TD2 pre = v[0];
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+        const TD2 o = i == 0 ? suf[0] : (i == K - 1 ? pre : td2_mul(pre, suf[i]));
+        if (i > 0 && i < K - 1) pre = td2_mul(pre, v[i]);
+        const float2 a = two_atanh2(o.t, o.d);
+        const float m0 = fminf(a.x, kCheckClamp), m1 = fminf(a.y, kCheckClamp);
+        const uint32_t g0 = (sa0 ^ __float_as_uint(x[i].x)) & 0x80000000u;
+        const uint32_t g1 = (sa1 ^ __float_as_uint(x[i].y)) & 0x80000000u;
+        out[i] = make_float2(__uint_as_float(__float_as_uint(m0) | g0), __uint_as_float(__float_as_uint(m1) | g1));
+    }
+}
+
 // Sample-innermost message rows (samples of a chunk padded to 64): a thread
 // takes four consecutive samples of one row with 16-byte loads and stores.
 __device__ __forceinline__ float4 ld4(const float* base, int64_t row, int64_t S, int64_t smp)

@@ -16,10 +16,10 @@
 //   Fm[face]      face -> its measurement variable
 //   Cl[face]      cube at the face's site (the face is its lower face) -> the face's variable
 //   Ch[face]      cube one step down along the face's normal (upper face) -> the variable
-// One iteration is three kernels: the total of every edge (prior + its four
-// face messages), the faces (inputs: edge total minus the face's own message,
-// and the measurement variable's prior + both cube messages), the cubes
-// (inputs: prior + face message + the other cube's message).  Check nodes use
+// One iteration is one kernel over the sites: the faces (inputs: the edge's total -- prior +
+// its four face messages -- minus the face's own message, and the measurement variable's
+// prior + both cube messages) and the cube (inputs: prior + face message + the other cube's
+// message).  Check nodes use
 // the plain BP's cancellation-free (t, d = 1 - t) arithmetic (t3d_bp_math.cuh),
 // so magnitudes keep FP32 accuracy up to the +-30 clamp.
 #include <cuda_runtime.h>
@@ -36,14 +36,13 @@ namespace t3d {
 namespace meta {
 namespace {
 
-using bpm::add4;
-using bpm::check_node;
-using bpm::comp;
-using bpm::ld4;
-using bpm::st4;
-using bpm::sub4;
+using bpm::check_node2;
 
-constexpr int kThreads = 256;   // threads per block, each on consecutive samples of one index
+constexpr int kThreads = 128;
+constexpr int kWordsPer = kThreads / 32;   // words per block of the iteration kernel
+constexpr int kDecideThreads = 256;        // samples per block of the decision kernel
+constexpr int64_t kMaxWords = 65535LL * kWordsPer;   // grid y of both kernels
+static_assert(kMaxWords * 64 <= 65535LL * kDecideThreads, "the decision kernel's grid");
 
 struct Bufs {
     float* F;     // [3L^3][4][S]
@@ -58,20 +57,129 @@ struct Args {
     int64_t W;              // row stride of the bit-sliced arrays (words)
     const uint64_t* s;      // measured syndrome, chunk's first word at column 0
     float l0, lq;
-    const float* T;         // edge totals [3L^3][S]
     Bufs in, out;
 };
 
-
-// Syndrome bits of samples smp .. smp + 3 (smp a multiple of 4) in bits 0..3.
-__device__ __forceinline__ uint32_t syn_bits4(const Args& a, int64_t row, int64_t smp)
+// One flooding iteration in one kernel.  A warp takes the three faces and the cube at one site for
+// the 64 samples of a word, two samples a lane, so every message row is one 256-byte access: the
+// totals of the nine edges its faces touch are summed from their messages on the spot (36 rows,
+// of which 12 are the faces' own), and the cube messages a face needs are the ones its cube reads.
+// Each message is read from HBM once and written once, 56 bytes per edge and sample; the earlier
+// three kernels (edge totals, faces, cubes) wrote and read the totals as well and read the face
+// and cube messages twice, 104 bytes.  kFirst: every message in is zero and nothing is read.
+// A block takes four words of one site (1 KB runs of a row).  Bound by the latency of those loads at
+// 20 warps per SM (96 registers; DRAM at 61% of its peak, issue 55%).  At L = 18, 1,536 samples
+// one iteration takes 0.29 ms against 0.37 for the three kernels, 12 iterations with the decision
+// 4.88 -> 3.49 ms (four sites and one word per block 3.70, 256 threads 3.81, six blocks per SM 4.00).
+template <bool kFirst>
+__global__ void __launch_bounds__(kThreads, 5) k_iteration(const __grid_constant__ Args a)
 {
-    return (uint32_t)(a.s[row * a.W + (smp >> 6)] >> (smp & 63)) & 0xFu;
-}
+    const Lattice lat = a.lat;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int r = (int)blockIdx.x;
+    const int64_t w = (int64_t)blockIdx.y * kWordsPer + warp;
+    if (w * 64 >= a.S) return;
+    const int64_t col = w * 64 + 2 * lane;
+    const int L3 = lat.L3;
+    const Coord c = site_coord(lat, r);
+    const int L = lat.L;
+    // steps to the neighbours (periodic); site + plus[] or + minus[]
+    const int px = c.x[0] + 1 == L ? 1 - L : 1, mx = c.x[0] == 0 ? L - 1 : -1;
+    const int py = c.x[1] + 1 == L ? L - lat.L2 : L, my = c.x[1] == 0 ? lat.L2 - L : -L;
+    const int pz = c.x[2] + 1 == L ? lat.L2 - lat.L3 : lat.L2, mz = c.x[2] == 0 ? lat.L3 - lat.L2 : -lat.L2;
+    const int rx = r + px, ry = r + py, rz = r + pz;
 
-__device__ __forceinline__ int64_t step_site(const Lattice& lat, const Coord& c, int ax, int delta)
-{
-    return site_index(lat, shifted(lat, c, ax, delta));
+    // row indices stay below 2^28 and a row below 2^32 bytes: one 32 x 32 -> 64-bit product each
+    const uint32_t stride = (uint32_t)a.S * 4u;
+    auto row = [&](const float* base, int i) {
+        return __ldg(reinterpret_cast<const float2*>(reinterpret_cast<const char*>(base + col) + (uint64_t)(uint32_t)i * stride));
+    };
+    auto put = [&](float* base, int i, float2 v) {
+        __stcs(reinterpret_cast<float2*>(reinterpret_cast<char*>(base + col) + (uint64_t)(uint32_t)i * stride), v);
+    };
+    // message of face (n, q) to its edge j
+    auto F = [&](int n, int q, int j) { return row(a.in.F, (n * L3 + q) * 4 + j); };
+    auto add = [](float2 u, float2 v) { return __fadd2_rn(u, v); };
+    auto sub = [](float2 u, float2 v) { return __fadd2_rn(u, make_float2(-v.x, -v.y)); };
+    const float2 l0 = make_float2(a.l0, a.l0), lq = make_float2(a.lq, a.lq);
+    auto sum4 = [&](float2 m0, float2 m1, float2 m2, float2 m3) { return add(add(add(add(l0, m0), m1), m2), m3); };
+    auto word = [&](int f) { return a.s[(int64_t)f * a.W + w]; };
+    auto bit = [&](uint64_t v, int j) { return (bool)((v >> (2 * lane + j)) & 1ULL); };
+
+    // the faces' own messages, requested before the cube's arithmetic
+    float2 f[3][4];
+#pragma unroll
+    for (int n = 0; n < 3; ++n)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) f[n][j] = kFirst ? make_float2(0.0f, 0.0f) : F(n, r, j);
+
+    // the cube: its lower faces (n, r), whose variable it reaches through Cl, and its upper faces
+    // (n, r + e_n), through Ch
+    const int up[3] = {rx, ry, rz};
+    uint64_t syn[3], par = 0;
+    float2 xm[3];   // the faces' measurement-variable inputs
+    {
+        float2 x[6], o[6];
+#pragma unroll
+        for (int n = 0; n < 3; ++n) {
+            const int fl = n * L3 + r, fu = n * L3 + up[n];
+            syn[n] = word(fl);
+            par ^= syn[n] ^ word(fu);
+            if (kFirst) {
+                x[2 * n] = x[2 * n + 1] = xm[n] = lq;
+            } else {
+                const float2 ch = row(a.in.Ch, fl);
+                x[2 * n] = add(add(lq, row(a.in.Fm, fl)), ch);
+                x[2 * n + 1] = add(add(lq, row(a.in.Fm, fu)), row(a.in.Cl, fu));
+                xm[n] = add(add(lq, row(a.in.Cl, fl)), ch);
+            }
+        }
+        check_node2<6>(x, bit(par, 0), bit(par, 1), o);
+#pragma unroll
+        for (int n = 0; n < 3; ++n) {
+            put(a.out.Cl, n * L3 + r, o[2 * n]);
+            put(a.out.Ch, n * L3 + up[n], o[2 * n + 1]);
+        }
+    }
+    // an edge's four faces in the order of edge_slots: x-edge at q (1, q) 0, (1, q - e_z) 1, (2, q) 0,
+    // (2, q - e_y) 1; y-edge (0, q) 0, (0, q - e_z) 1, (2, q) 2, (2, q - e_x) 3; z-edge (0, q) 2,
+    // (0, q - e_y) 3, (1, q) 2, (1, q - e_x) 3
+    auto face = [&](int n, const float2 (&x)[5]) {
+        float2 o[5];
+        check_node2<5>(x, bit(syn[n], 0), bit(syn[n], 1), o);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) put(a.out.F, (n * L3 + r) * 4 + j, o[j]);
+        put(a.out.Fm, n * L3 + r, o[4]);
+    };
+    if (kFirst) {
+#pragma unroll
+        for (int n = 0; n < 3; ++n) {
+            const float2 x[5] = {l0, l0, l0, l0, xm[n]};
+            face(n, x);
+        }
+        return;
+    }
+    const float2 Ty = sum4(f[0][0], F(0, r + mz, 1), f[2][2], F(2, r + mx, 3));
+    const float2 Tz = sum4(f[0][2], F(0, r + my, 3), f[1][2], F(1, r + mx, 3));
+    {
+        const float2 Tyz = sum4(F(0, rz, 0), f[0][1], F(2, rz, 2), F(2, rz + mx, 3));
+        const float2 Tzy = sum4(F(0, ry, 2), f[0][3], F(1, ry, 2), F(1, ry + mx, 3));
+        const float2 x[5] = {sub(Ty, f[0][0]), sub(Tyz, f[0][1]), sub(Tz, f[0][2]), sub(Tzy, f[0][3]), xm[0]};
+        face(0, x);
+    }
+    const float2 Tx = sum4(f[1][0], F(1, r + mz, 1), f[2][0], F(2, r + my, 1));
+    {
+        const float2 Txz = sum4(F(1, rz, 0), f[1][1], F(2, rz, 0), F(2, rz + my, 1));
+        const float2 Tzx = sum4(F(0, rx, 2), F(0, rx + my, 3), F(1, rx, 2), f[1][3]);
+        const float2 x[5] = {sub(Tx, f[1][0]), sub(Txz, f[1][1]), sub(Tz, f[1][2]), sub(Tzx, f[1][3]), xm[1]};
+        face(1, x);
+    }
+    {
+        const float2 Txy = sum4(F(1, ry, 0), F(1, ry + mz, 1), F(2, ry, 0), f[2][1]);
+        const float2 Tyx = sum4(F(0, rx, 0), F(0, rx + mz, 1), F(2, rx, 2), f[2][3]);
+        const float2 x[5] = {sub(Tx, f[2][0]), sub(Txy, f[2][1]), sub(Ty, f[2][2]), sub(Tyx, f[2][3]), xm[2]};
+        face(2, x);
+    }
 }
 
 // The four (face, slot) pairs of edge (d, r): for each normal n != d with third axis
@@ -86,120 +194,36 @@ __device__ __forceinline__ void edge_slots(const Lattice& lat, int d, int r, int
         const int lo = d < ax ? 0 : 2;
         f[2 * i] = (int64_t)n * lat.L3 + r;
         slot[2 * i] = lo;
-        f[2 * i + 1] = (int64_t)n * lat.L3 + step_site(lat, c, ax, -1);
+        f[2 * i + 1] = (int64_t)n * lat.L3 + site_index(lat, shifted(lat, c, ax, -1));
         slot[2 * i + 1] = lo + 1;
     }
 }
 
-// The iteration kernels give each thread four consecutive samples of one index:
-// blockIdx.x is the index, blockIdx.y * blockDim.x + threadIdx.x the sample quad.
-__device__ __forceinline__ int64_t quad_sample(const Args& a)
-{
-    return ((int64_t)blockIdx.y * blockDim.x + threadIdx.x) * 4;
-}
-
-__global__ void __launch_bounds__(kThreads) k_edge_totals(const Args a, float* __restrict__ T)
-{
-    const int64_t smp = quad_sample(a);
-    const int64_t v = blockIdx.x;
-    if (smp >= a.S) return;
-    const int d = (int)(v / a.lat.L3), r = (int)(v % a.lat.L3);
-    int64_t f[4];
-    int slot[4];
-    edge_slots(a.lat, d, r, f, slot);
-    float4 t = make_float4(a.l0, a.l0, a.l0, a.l0);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) t = add4(t, ld4(a.in.F, f[k] * 4 + slot[k], a.S, smp));
-    st4(T, v, a.S, smp, t);
-}
-
-__global__ void __launch_bounds__(kThreads) k_faces(const Args a)
-{
-    const int64_t smp = quad_sample(a);
-    const int64_t fc = blockIdx.x;
-    if (smp >= a.S) return;
-    const int n = (int)(fc / a.lat.L3), r = (int)(fc % a.lat.L3);
-    const Coord c = site_coord(a.lat, r);
-    const int ax = n == 0 ? 1 : 0, bx = n == 2 ? 1 : 2;   // in-plane axes a < b
-    const int64_t L3 = a.lat.L3;
-    const int64_t ed[4] = {ax * L3 + r, ax * L3 + step_site(a.lat, c, bx, 1), bx * L3 + r,
-                           bx * L3 + step_site(a.lat, c, ax, 1)};
-    float4 x4[5];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) x4[j] = sub4(ld4(a.T, ed[j], a.S, smp), ld4(a.in.F, fc * 4 + j, a.S, smp));
-    const float4 lq = make_float4(a.lq, a.lq, a.lq, a.lq);
-    x4[4] = add4(add4(lq, ld4(a.in.Cl, fc, a.S, smp)), ld4(a.in.Ch, fc, a.S, smp));
-    const uint32_t syn = syn_bits4(a, fc, smp);
-    float o4[5][4];
-#pragma unroll
-    for (int cpt = 0; cpt < 4; ++cpt) {
-        float x[5], o[5];
-#pragma unroll
-        for (int j = 0; j < 5; ++j) x[j] = comp(x4[j], cpt);
-        check_node<5>(x, (syn >> cpt) & 1u, o);
-#pragma unroll
-        for (int j = 0; j < 5; ++j) o4[j][cpt] = o[j];
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) st4(a.out.F, fc * 4 + j, a.S, smp, make_float4(o4[j][0], o4[j][1], o4[j][2], o4[j][3]));
-    st4(a.out.Fm, fc, a.S, smp, make_float4(o4[4][0], o4[4][1], o4[4][2], o4[4][3]));
-}
-
-__global__ void __launch_bounds__(kThreads) k_cubes(const Args a)
-{
-    const int64_t smp = quad_sample(a);
-    const int r = blockIdx.x;
-    if (smp >= a.S) return;
-    const Coord c = site_coord(a.lat, r);
-    const int64_t L3 = a.lat.L3;
-    int64_t fl[3], fu[3];   // lower faces (n, r), upper faces (n, r + e_n)
-    uint32_t par = 0;
-    float4 x4[6];
-    const float4 lq = make_float4(a.lq, a.lq, a.lq, a.lq);
-#pragma unroll
-    for (int nn = 0; nn < 3; ++nn) {
-        fl[nn] = nn * L3 + r;
-        fu[nn] = nn * L3 + step_site(a.lat, c, nn, 1);
-        par ^= syn_bits4(a, fl[nn], smp) ^ syn_bits4(a, fu[nn], smp);
-        // this cube is the lower-face cube of fl (its message is Cl) and the upper-face cube of fu (Ch)
-        x4[2 * nn] = add4(add4(lq, ld4(a.in.Fm, fl[nn], a.S, smp)), ld4(a.in.Ch, fl[nn], a.S, smp));
-        x4[2 * nn + 1] = add4(add4(lq, ld4(a.in.Fm, fu[nn], a.S, smp)), ld4(a.in.Cl, fu[nn], a.S, smp));
-    }
-    float o4[6][4];
-#pragma unroll
-    for (int cpt = 0; cpt < 4; ++cpt) {
-        float x[6], o[6];
-#pragma unroll
-        for (int j = 0; j < 6; ++j) x[j] = comp(x4[j], cpt);
-        check_node<6>(x, (par >> cpt) & 1u, o);
-#pragma unroll
-        for (int j = 0; j < 6; ++j) o4[j][cpt] = o[j];
-    }
-#pragma unroll
-    for (int nn = 0; nn < 3; ++nn) {
-        st4(a.out.Cl, fl[nn], a.S, smp, make_float4(o4[2 * nn][0], o4[2 * nn][1], o4[2 * nn][2], o4[2 * nn][3]));
-        st4(a.out.Ch, fu[nn], a.S, smp,
-            make_float4(o4[2 * nn + 1][0], o4[2 * nn + 1][1], o4[2 * nn + 1][2], o4[2 * nn + 1][3]));
-    }
-}
-
-// Posteriors and decisions: qubit v: l = T_v; decision words (one ballot per 32
-// samples) into dec[word][site][4] as 32-bit halves; optional posteriors.
-__global__ void __launch_bounds__(kThreads) k_decide(const Args a, int64_t n_samples, uint32_t* __restrict__ dec32,
+// Posteriors and decisions: qubit v: l = prior + its four face messages (a.in.F nullptr: no
+// iteration ran, every message is zero); decision words (one ballot per 32 samples) into
+// dec[word][site][4] as 32-bit halves; optional posteriors.
+__global__ void __launch_bounds__(kDecideThreads) k_decide(const Args a, int64_t n_samples, uint32_t* __restrict__ dec32,
                                                       float* __restrict__ llr, int64_t llr_stride)
 {
-    const int64_t smp = (int64_t)blockIdx.y * kThreads + threadIdx.x;
+    const int64_t smp = (int64_t)blockIdx.y * kDecideThreads + threadIdx.x;
     const int64_t v = blockIdx.x;
     const int64_t L3 = a.lat.L3, n = 3 * L3;
     if (smp >= a.S) return;   // S is a multiple of 64: whole warps
-    const float l = a.T[v * a.S + smp];
+    const int d = (int)(v / L3), r = (int)(v % L3);
+    float l = a.l0, m = a.lq;
+    if (a.in.F) {
+        int64_t f[4];
+        int slot[4];
+        edge_slots(a.lat, d, r, f, slot);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) l += __ldcs(&a.in.F[(f[k] * 4 + slot[k]) * a.S + smp]);
+        if (llr) m = m + __ldcs(&a.in.Fm[v * a.S + smp]) + __ldcs(&a.in.Cl[v * a.S + smp]) + __ldcs(&a.in.Ch[v * a.S + smp]);
+    }
     const bool valid = smp < n_samples;
     const uint32_t bits = __ballot_sync(0xffffffffu, valid && l < 0.0f);
-    const int d = (int)(v / L3), r = (int)(v % L3);
     if ((threadIdx.x & 31) == 0) dec32[((smp >> 6) * L3 + r) * 8 + 2 * d + ((smp >> 5) & 1)] = bits;
     if (llr && valid) {
         llr[v * llr_stride + smp] = l;
-        const float m = a.lq + a.in.Fm[v * a.S + smp] + a.in.Cl[v * a.S + smp] + a.in.Ch[v * a.S + smp];
         llr[(n + v) * llr_stride + smp] = m;
     }
 }
@@ -210,29 +234,24 @@ Bufs split_messages(float* m, int64_t n, int64_t S)
     return Bufs{m, m + 4 * n * S, m + 5 * n * S, m + 6 * n * S};
 }
 
-// Quad-kernel block: S / 4 sample quads, at most kThreads a block, whole warps.
-unsigned quad_threads(int64_t S) { return (unsigned)std::min<int64_t>(kThreads, (S / 4 + 31) / 32 * 32); }
-
-unsigned quad_blocks(int64_t S) { return (unsigned)((S / 4 + quad_threads(S) - 1) / quad_threads(S)); }
-
-// One flooding iteration: every check -> variable message of `out` from those of `in`.
-t3d_status launch_iteration(Args& a, float* T, const Bufs& in, const Bufs& out, cudaStream_t st)
+// One flooding iteration: every check -> variable message of `out` from those of `in`
+// (in.F nullptr: the first iteration, all zero).
+t3d_status launch_iteration(Args& a, const Bufs& in, const Bufs& out, cudaStream_t st)
 {
-    const int64_t n = 3LL * a.lat.L3;
-    const unsigned tx = quad_threads(a.S), gy = quad_blocks(a.S);
     a.in = in;
     a.out = out;
     ProfScope prof(T3D_K_BP_STEP, st);
-    k_edge_totals<<<dim3((unsigned)n, gy), tx, 0, st>>>(a, T);
-    T3D_LAUNCH_CHECK("meta-check BP edge totals");
-    k_faces<<<dim3((unsigned)n, gy), tx, 0, st>>>(a);
-    T3D_LAUNCH_CHECK("meta-check BP faces");
-    k_cubes<<<dim3((unsigned)a.lat.L3, gy), tx, 0, st>>>(a);
-    T3D_LAUNCH_CHECK("meta-check BP cubes");
+    const int64_t words = a.S / 64;
+    const dim3 grid((unsigned)a.lat.L3, (unsigned)((words + kWordsPer - 1) / kWordsPer));
+    if (in.F)
+        k_iteration<false><<<grid, kThreads, 0, st>>>(a);
+    else
+        k_iteration<true><<<grid, kThreads, 0, st>>>(a);
+    T3D_LAUNCH_CHECK("meta-check BP iteration");
     return T3D_OK;
 }
 
-Args make_args(const Lattice& lat, int64_t S, int64_t W, const uint64_t* s, double p, double q, float* T)
+Args make_args(const Lattice& lat, int64_t S, int64_t W, const uint64_t* s, double p, double q)
 {
     Args a;
     std::memset(&a, 0, sizeof(a));
@@ -242,7 +261,6 @@ Args make_args(const Lattice& lat, int64_t S, int64_t W, const uint64_t* s, doub
     a.s = s;
     a.l0 = (float)std::log((1.0 - p) / p);
     a.lq = (float)std::log((1.0 - q) / q);
-    a.T = T;
     return a;
 }
 
@@ -265,9 +283,8 @@ t3d_status launch_bp_meta(const Lattice& lat, int64_t n_samples, int64_t W, uint
                           double q, int iters, void* work, size_t work_bytes, float* llr_out, cudaStream_t st)
 {
     const int64_t words = words_for(n_samples);
-    // at most 65535 sample blocks of kThreads per launch (grid y)
     const int64_t chunk = std::min<int64_t>({words, (int64_t)(work_bytes / bytes_per_word(lat.L)),
-                                             65535LL * kThreads / 64});
+                                             kMaxWords});
     T3D_REQUIRE(chunk >= 1, "workspace too small: %zu bytes < %zu per 64-sample word", work_bytes,
                 bytes_per_word(lat.L));
     T3D_REQUIRE(llr_out == nullptr || chunk == words, "llr_out needs a workspace for all samples at once");
@@ -281,19 +298,15 @@ t3d_status launch_bp_meta(const Lattice& lat, int64_t n_samples, int64_t W, uint
             base += (floats * sizeof(float) + 255) / 256 * 256;
             return ptr;
         };
-        float* T = take(n * S);
         const Bufs b[2] = {split_messages(take(7 * n * S), n, S), split_messages(take(7 * n * S), n, S)};
         uint64_t* dec = reinterpret_cast<uint64_t*>(base);
-        // every message starts at zero: the first iteration sees the priors alone
-        T3D_CUDA_CHECK(cudaMemsetAsync(b[0].F, 0, 7 * n * S * sizeof(float), st));
-        Args a = make_args(lat, S, W, s + w0, p, q, T);
-        for (int it = 0; it < iters; ++it) T3D_TRY(launch_iteration(a, T, b[it & 1], b[(it + 1) & 1], st));
-        a.in = b[iters & 1];
+        Args a = make_args(lat, S, W, s + w0, p, q);
+        for (int it = 0; it < iters; ++it)
+            T3D_TRY(launch_iteration(a, it ? b[it & 1] : Bufs{nullptr, nullptr, nullptr, nullptr}, b[(it + 1) & 1], st));
+        a.in = iters ? b[iters & 1] : Bufs{nullptr, nullptr, nullptr, nullptr};
         ProfScope prof(T3D_K_BP_DECIDE, st);
-        k_edge_totals<<<dim3((unsigned)n, quad_blocks(S)), quad_threads(S), 0, st>>>(a, T);
-        T3D_LAUNCH_CHECK("meta-check BP posteriors");
-        k_decide<<<dim3((unsigned)n, (unsigned)((S + kThreads - 1) / kThreads)), kThreads, 0, st>>>(a, ns, reinterpret_cast<uint32_t*>(dec), llr_out,
-                                                             n_samples);
+        k_decide<<<dim3((unsigned)n, (unsigned)((S + kDecideThreads - 1) / kDecideThreads)), kDecideThreads, 0, st>>>(
+            a, ns, reinterpret_cast<uint32_t*>(dec), llr_out, n_samples);
         T3D_LAUNCH_CHECK("meta-check BP decisions");
         T3D_TRY(launch_dec_apply(lat, W, cw, dec, e + w0, s + w0, st));
     }
@@ -323,7 +336,7 @@ extern "C" t3d_status toric3d_bp_meta_step(int L, int64_t n_samples, const uint6
 {
     clear_error();
     T3D_TRY(check_lattice(L));
-    T3D_REQUIRE(n_samples >= 1 && words_for(n_samples) <= 65535LL * meta::kThreads / 64, "n_samples out of range");
+    T3D_REQUIRE(n_samples >= 1 && words_for(n_samples) <= meta::kMaxWords, "n_samples out of range");
     T3D_TRY(check_words(s, "s"));
     T3D_REQUIRE(p > 0.0 && p < 1.0, "BP needs 0 < p < 1");
     T3D_REQUIRE(q > 0.0 && q < 1.0, "meta-checks need measurement errors: 0 < q < 1");
@@ -336,9 +349,8 @@ extern "C" t3d_status toric3d_bp_meta_step(int L, int64_t n_samples, const uint6
                 mb / 7);
     const Lattice lat = make_lattice_host(L);
     const int64_t n = 3LL * lat.L3, S = 64 * words_for(n_samples);
-    float* T = static_cast<float*>(work);
-    meta::Args a = meta::make_args(lat, S, words_for(n_samples), s, p, q, T);
-    return meta::launch_iteration(a, T, meta::split_messages(const_cast<float*>(msg_in), n, S),
+    meta::Args a = meta::make_args(lat, S, words_for(n_samples), s, p, q);
+    return meta::launch_iteration(a, meta::split_messages(const_cast<float*>(msg_in), n, S),
                                   meta::split_messages(msg_out, n, S), as_stream(stream));
 }
 

@@ -33,3 +33,38 @@ def test_decode_equals_single_iterations(L, S, iters, q):
     ge, gs = e.clone(), s.clone()
     t3d.toric3d_bp(L, S, ge, gs, 0.04, q, iters, workspace(t3d.toric3d_bp_workspace_bytes(L, 64)))
     assert torch.equal(ge, we) and torch.equal(gs, ws)
+
+
+@pytest.mark.parametrize("L,S", [(2, 70), (3, 64), (4, 300), (6, 1)])
+@pytest.mark.parametrize("iters", [0, 1, 2, 3])
+def test_meta_decode_equals_single_iterations(L, S, iters):
+    """The meta-check decode (whose first iteration reads no messages) against toric3d_bp_meta_step from
+    an all-zero buffer: every posterior is the prior plus that step's messages, summed in their order."""
+    n, n3 = 3 * L ** 3, L ** 3
+    s = upload_bits(inp.random_bits(S, n, 0.2, seed=L + S))
+    Sp = 64 * inp.words_for(S)
+    msg = [torch.zeros((7 * n, Sp), dtype=torch.float32, device=dev()) for _ in range(2)]
+    work = workspace(n * Sp * 4)
+    for k in range(iters):
+        t3d.toric3d_bp_meta_step(L, S, s, 0.04, 0.03, msg[k % 2], msg[(k + 1) % 2], work)
+    m = msg[iters % 2]
+    F = m[:4 * n].view(3, L, L, L, 4, Sp)
+    l0 = torch.log(torch.tensor((1 - 0.04) / 0.04, dtype=torch.float64)).float().item()
+    lq = torch.log(torch.tensor((1 - 0.03) / 0.03, dtype=torch.float64)).float().item()
+    axis = {0: 2, 1: 1, 2: 0}                        # lattice axis -> dimension of a [z, y, x, ...] array
+    want = torch.empty((2, n, Sp), dtype=torch.float32, device=dev())
+    for d in range(3):
+        t = torch.full((L, L, L, Sp), l0, dtype=torch.float32, device=dev())
+        for nn in [k for k in range(3) if k != d]:
+            ax = 3 - d - nn
+            lo = 0 if d < ax else 2
+            t = t + F[nn, :, :, :, lo]
+            t = t + torch.roll(F[nn, :, :, :, lo + 1], 1, axis[ax])
+        want[0, d * n3:(d + 1) * n3] = t.reshape(n3, Sp)
+    want[1] = ((lq + m[4 * n:5 * n]) + m[5 * n:6 * n]) + m[6 * n:7 * n]
+    got = torch.empty((2, n, S), dtype=torch.float32, device=dev())
+    e = torch.zeros_like(s)
+    t3d.toric3d_bp_meta(L, S, e, s.clone(), 0.04, 0.03, iters, workspace(t3d.toric3d_bp_meta_workspace_bytes(L, S)), got)
+    assert torch.equal(got, want[:, :, :S])
+    bits = (want[0] < 0)[:, :S].cpu().numpy().astype("uint8")
+    assert (e.cpu().numpy().view("uint64") == inp.pack(bits.T)).all()
