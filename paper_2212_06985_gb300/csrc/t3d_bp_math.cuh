@@ -159,7 +159,6 @@ __device__ __forceinline__ float2 two_atanh2(float2 P, float2 D)
 template <int K>
 __device__ __forceinline__ void check_node2(const float2 (&x)[K], bool syn0, bool syn1, float2 (&out)[K])
 {
-    static_assert(K >= 3, "at least three inputs");
     TD2 v[K], suf[K];
     uint32_t sa0 = syn0 ? 0x80000000u : 0u, sa1 = syn1 ? 0x80000000u : 0u;
 #pragma unroll
@@ -168,13 +167,17 @@ __device__ __forceinline__ void check_node2(const float2 (&x)[K], bool syn0, boo
         sa0 ^= __float_as_uint(x[i].x);
         sa1 ^= __float_as_uint(x[i].y);
     }
-    suf[K - 2] = v[K - 1];
+    if constexpr (K >= 2) suf[K - 2] = v[K - 1];
 #pragma unroll
     for (int i = K - 3; i >= 0; --i) suf[i] = td2_mul(v[i + 1], suf[i + 1]);
     TD2 pre = v[0];
 #pragma unroll
     for (int i = 0; i < K; ++i) {
-        const TD2 o = i == 0 ? suf[0] : (i == K - 1 ? pre : td2_mul(pre, suf[i]));
+        TD2 o;
+        if constexpr (K == 1)
+            o = TD2{f2(1.0f), f2(0.0f)};   // no other input
+        else
+            o = i == 0 ? suf[0] : (i == K - 1 ? pre : td2_mul(pre, suf[i]));
         if (i > 0 && i < K - 1) pre = td2_mul(pre, v[i]);
         const float2 a = two_atanh2(o.t, o.d);
         const float m0 = fminf(a.x, kCheckClamp), m1 = fminf(a.y, kCheckClamp);
