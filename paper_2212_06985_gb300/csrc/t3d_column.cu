@@ -5,9 +5,8 @@
 //
 // Samples are independent, so a word's column of the bit-sliced arrays never needs another
 // column: what separates two applications is a barrier of one block instead of a kernel
-// boundary.  At L <= 16 the syndrome and the flip words (48 bytes per site and word, 196,608
-// bytes at L = 16) fit the 227 KB a block can have; at L <= 14 the error words fit as well
-// (72 bytes), above that they stay in global memory.
+// boundary.  Up to L = 14 the syndrome, the flip and the error words (72 bytes per site and word)
+// fit the 227 KB a block can have.
 //
 // An application is two phases between barriers: every site decides its own three edges from
 // the old syndrome (7 shared reads: the z-neighbour's words are the thread's previous ones)
@@ -21,6 +20,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <type_traits>
 
@@ -55,8 +55,8 @@ struct Rows {
     __device__ __forceinline__ uint64_t& at(int row) const { return p[(int64_t)row * W]; }
 };
 
-// kRun: whole runs (sweeps otherwise); kESmem: the error words are in shared memory as well.
-template <bool kRun, bool kESmem>
+// kRun: whole runs (sweeps otherwise, E gathering the flips for e).
+template <bool kRun>
 __global__ void __launch_bounds__(kColumnThreads, 1)
 k_column(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgram pr)
 {
@@ -65,7 +65,7 @@ k_column(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgr
     const int P = L2 * Wt, N = L3 * Wt;   // a z-plane, the lattice
     uint64_t* const S0 = sm;
     uint64_t* const F0 = sm + 3 * N;
-    uint64_t* const E0 = sm + 6 * N;      // kESmem
+    uint64_t* const E0 = sm + 6 * N;
 
     const int t = threadIdx.x;
     const int zp = t / P, u = t - zp * P, wl = u % Wt, xy = u / Wt;
@@ -107,9 +107,8 @@ k_column(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgr
                                    s0y = S0[i + ym];
                     uint64_t f[3] = {at_least_three(s2, s2y, s1, s1m), at_least_three(s2, s2x, s0, s0m),
                                      at_least_three(s1, s1x, s0, s0y)};
-                    const int site = z * L2 + xy;
                     if (prob) {
-                        const PhiloxSite ps = philox_site(pc, (uint32_t)site);
+                        const PhiloxSite ps = philox_site(pc, (uint32_t)(z * L2 + xy));
                         const U32x4 a = philox_finish(pc, ps, b0), b = philox_finish(pc, ps, b1);
                         f[0] |= exactly_two(s2, s2y, s1, s1m) & ((uint64_t)a.v[0] | ((uint64_t)a.v[1] << 32));
                         f[1] |= exactly_two(s2, s2x, s0, s0m) & ((uint64_t)a.v[2] | ((uint64_t)a.v[3] << 32));
@@ -118,11 +117,7 @@ k_column(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgr
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         F0[k * N + i] = f[k];
-                        if (kESmem) {
-                            if (f[k]) E0[k * N + i] ^= f[k];
-                        } else {
-                            xor_into(&e.at(k * L3 + site), f[k]);
-                        }
+                        if (f[k]) E0[k * N + i] ^= f[k];
                     }
                     s0m = s0;
                     s1m = s1;
@@ -173,7 +168,7 @@ k_column(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgr
 #pragma unroll
                 for (int n = 0; n < 3; ++n) {
                     S0[n * N + i] = s.at(n * L3 + z * L2 + xy);
-                    if (kESmem) E0[n * N + i] = 0;
+                    E0[n * N + i] = 0;
                 }
             }
             __syncthreads();
@@ -191,19 +186,13 @@ k_column(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgr
 #pragma unroll
                 for (int n = 0; n < 3; ++n) {
                     s.at(n * L3 + z * L2 + xy) = S0[n * N + i];
-                    if (kESmem) xor_into(&e.at(n * L3 + z * L2 + xy), E0[n * N + i]);
+                    xor_into(&e.at(n * L3 + z * L2 + xy), E0[n * N + i]);
                 }
             }
         } else {
-            // the error word of edge (k, site z, xy)
-            auto E = [&](int k, int z, int i) -> uint64_t& {
-                if (kESmem) return E0[k * N + i];
-                return e.at(k * L3 + z * L2 + xy);
-            };
-            if (kESmem)
-                for (int z = zb, i = zb * P + u; z < ze; ++z, i += P)
+            for (int z = zb, i = zb * P + u; z < ze; ++z, i += P)
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) E0[k * N + i] = e.at(k * L3 + z * L2 + xy);
+                for (int k = 0; k < 3; ++k) E0[k * N + i] = e.at(k * L3 + z * L2 + xy);
 
             auto noise = [&](uint32_t cycle) {
                 if (pr.thr_p == 0) return;
@@ -215,28 +204,17 @@ k_column(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgr
                         const uint64_t f = all ? ~0ULL
                                                : bernoulli_site(bc, (uint32_t)pr.thr_p,
                                                                 (uint32_t)(k * L3 + z * L2 + xy));
-                        if (f) E(k, z, i) ^= f;
+                        E0[k * N + i] ^= f;
                     }
             };
             auto measure = [&](uint64_t thr, uint32_t cycle) {
                 const bool all = thr >> 32, none = thr == 0;
                 const BernoulliColumn bc = bernoulli_column(pr.seed, kStreamMeas, cycle, group);
-                // row offsets of the neighbours in global memory (sites) and in shared memory
-                const int gx = kESmem ? xp : (x + 1 == L ? 1 - L : 1), gy = kESmem ? yp : (y + 1 == L ? L - L2 : L);
                 for (int z = zb, i = zb * P + u; z < ze; ++z, i += P) {
-                    const int gz = (z + 1 == L ? 1 - L : 1) * (kESmem ? P : L2);
-                    const int site = z * L2 + xy;
-                    uint64_t ex, ey, ez, exy, exz, eyx, eyz, ezx, ezy;
-                    if (kESmem) {
-                        const uint64_t *px = E0 + i, *py = px + N, *pz = py + N;
-                        ex = px[0], exy = px[gy], exz = px[gz];
-                        ey = py[0], eyx = py[gx], eyz = py[gz];
-                        ez = pz[0], ezx = pz[gx], ezy = pz[gy];
-                    } else {
-                        ex = e.at(site), exy = e.at(site + gy), exz = e.at(site + gz);
-                        ey = e.at(L3 + site), eyx = e.at(L3 + site + gx), eyz = e.at(L3 + site + gz);
-                        ez = e.at(2 * L3 + site), ezx = e.at(2 * L3 + site + gx), ezy = e.at(2 * L3 + site + gy);
-                    }
+                    const int zz = (z + 1 == L ? 1 - L : 1) * P, site = z * L2 + xy;
+                    const uint64_t *px = E0 + i, *py = px + N, *pz = py + N;
+                    const uint64_t ex = px[0], exy = px[yp], exz = px[zz], ey = py[0], eyx = py[xp], eyz = py[zz],
+                                   ez = pz[0], ezx = pz[xp], ezy = pz[yp];
                     S0[i] = ey ^ eyz ^ ez ^ ezy;
                     S0[N + i] = ex ^ exz ^ ez ^ ezx;
                     S0[2 * N + i] = ex ^ exy ^ ey ^ eyx;
@@ -265,10 +243,9 @@ k_column(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgr
                 __syncthreads();
                 flip_until_clear(pr.perfect);
             }
-            if (kESmem)
-                for (int z = zb, i = zb * P + u; z < ze; ++z, i += P)
+            for (int z = zb, i = zb * P + u; z < ze; ++z, i += P)
 #pragma unroll
-                    for (int k = 0; k < 3; ++k) e.at(k * L3 + z * L2 + xy) = E0[k * N + i];
+                for (int k = 0; k < 3; ++k) e.at(k * L3 + z * L2 + xy) = E0[k * N + i];
         }
         __syncthreads();   // the next column overwrites the words
     }
@@ -665,9 +642,7 @@ t3d_status launch_slab(const ItemDesc& d, ColumnProgram pr, int kind, cudaStream
     return T3D_OK;
 }
 
-size_t column_bytes(int L, bool e_smem) { return (size_t)L * L * L * (e_smem ? 72 : 48); }
-
-bool e_fits(int L) { return column_bytes(L, true) <= kColumnSmem; }
+size_t column_bytes(int L) { return (size_t)L * L * L * 72; }
 
 // Words per block and z-parts.  A block should have at least two warps, so tiny lattices take
 // several words; a lattice column is split into as many z-parts as keep about kColumnTarget
@@ -683,10 +658,9 @@ struct ColumnShape {
 ColumnShape column_shape(int L, int64_t words)
 {
     ColumnShape c;
-    const bool es = e_fits(L);
     c.wt = 1;
     while (L * L * L * c.wt < 64 && c.wt < words) c.wt *= 2;
-    c.smem = column_bytes(L, es) * c.wt;
+    c.smem = column_bytes(L) * c.wt;
     const int plane = L * L * c.wt;
     const int64_t columns = (words + c.wt - 1) / c.wt;
     const int fit = (int)std::max<size_t>(1, std::min<size_t>(32, kColumnSmem / (c.smem + 1024)));
@@ -706,8 +680,7 @@ t3d_status launch_column(const ItemDesc& item, ColumnProgram pr, int kind, cudaS
     const ColumnShape c = column_shape(d.lat.L, words);
     d.tx = c.wt;
     pr.zt = c.zt;
-    const bool es = e_fits(d.lat.L);
-    auto kernel = es ? k_column<kRun, true> : k_column<kRun, false>;
+    auto kernel = k_column<kRun>;
     T3D_TRY(allow_dynamic_smem((const void*)kernel, c.smem));
     ProfScope prof(kind, st);
     kernel<<<persistent_grid((const void*)kernel, c.threads, kind, (words + c.wt - 1) / c.wt, false, c.smem),
@@ -726,9 +699,23 @@ uint64_t schedule_bits(const char* schedule, int slen)
 
 }  // namespace
 
-bool column_fits(int L) { return column_bytes(L, false) <= kColumnSmem; }
+bool column_fits(int L) { return column_bytes(L) <= kColumnSmem; }
 
-// Whether a schedule of n_apply applications runs on chip.  Above L = 16 the columns are turned
+// Whether a whole run pays on chip.  A column draws its random words on one SM, about
+// 0.0127 L^3 us a cycle, where the noise and measurement kernels spread them over the chip for three
+// launches (about 12 us) a cycle: with fewer columns than SMs, or a last round of columns that
+// leaves SMs idle, the column waits for itself (one FFPFF cycle, columns / step by step with the
+// schedule on chip: L = 14, 160 words 144 / 127 us, 304 words 144 / 162; L = 12, 160 words 92 / 85, 304
+// words 93 / 108).  From four rounds on the launches and the syndrome's way through memory cost more
+// (L = 14, 700 words 344 / 356).
+bool column_run_pays(int L, int64_t words)
+{
+    if (!column_fits(L)) return false;
+    const double rounds = words / 152.0, idle = std::ceil(rounds) - rounds;
+    return rounds >= 4.0 || idle * 0.0127 * L * L * L <= 12.0;
+}
+
+// Whether a schedule of n_apply applications runs on chip.  Above L = 14 the columns are turned
 // first and back afterwards from kTurnWords words on (about 2.2 ms at L = 32, 10^5 samples, five
 // applications' gain: FFPFF 5.6 -> 4.8 ms, PFFPFF x 32 in 33 -> 20 ms); below that a step by
 // step schedule is bound by its launches.
@@ -749,7 +736,7 @@ t3d_status launch_column_sweeps(const ItemDesc& d, const char* schedule, int sle
     pr.sweep0 = sweep0;
     pr.cycle0 = cycle;
     const int kind = pr.sched ? T3D_K_PFLIP : T3D_K_FLIP;
-    return e_fits(d.lat.L) ? launch_column<false>(d, pr, kind, st) : launch_slab(d, pr, kind, st);
+    return column_fits(d.lat.L) ? launch_column<false>(d, pr, kind, st) : launch_slab(d, pr, kind, st);
 }
 
 t3d_status launch_column_until_clear(const ItemDesc& d, int max_sweeps, int32_t* sweeps_done, cudaStream_t st)
@@ -761,7 +748,7 @@ t3d_status launch_column_until_clear(const ItemDesc& d, int max_sweeps, int32_t*
     pr.n_apply = max_sweeps;
     pr.until_clear = 1;
     pr.sweeps_done = sweeps_done;
-    return e_fits(d.lat.L) ? launch_column<false>(d, pr, T3D_K_FLIP, st) : launch_slab(d, pr, T3D_K_FLIP, st);
+    return column_fits(d.lat.L) ? launch_column<false>(d, pr, T3D_K_FLIP, st) : launch_slab(d, pr, T3D_K_FLIP, st);
 }
 
 t3d_status launch_column_run(const ItemDesc& d, int cycles, uint32_t cycle0, uint64_t thr_p, uint64_t thr_q,

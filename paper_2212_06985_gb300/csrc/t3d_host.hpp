@@ -123,7 +123,8 @@ t3d_status launch_logical(ItemTable& tab, cudaStream_t st);
 // Lattices whose syndrome and flip words fit one SM or a cluster of them (t3d_column.cu): a
 // schedule, a flip until clear, or a whole run in one launch per item.  No scratch (ItemDesc::tmp, stop) is used.
 struct ItemDesc;
-bool column_fits(int L);   // whole runs (L <= 16)
+bool column_fits(int L);   // one SM, error words included (L <= 14)
+bool column_run_pays(int L, int64_t words);           // whole runs
 bool sweeps_fit(int L, int64_t words, int n_apply);   // schedules and flip until clear (L <= 32)
 t3d_status launch_column_sweeps(const ItemDesc& d, const char* schedule, int slen, int n_apply, uint32_t sweep0,
                                 uint64_t seed, uint32_t cycle, cudaStream_t st);

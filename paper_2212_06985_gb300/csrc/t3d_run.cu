@@ -346,11 +346,11 @@ t3d_status enqueue_run(const t3d_run_cfg& c, const Plan& pl, cudaStream_t st)
     // flip / p-flip runs of lattices that fit one SM: all cycles and the noiseless round in one
     // launch per item; the other items (`items`) go step by step
     const bool columns = !learned(c) && !c.use_bp;
-    auto stepwise = [&](const ItemDesc& d) { return !columns || !column_fits(d.lat.L); };
+    auto stepwise = [&](const ItemDesc& d) { return !columns || !column_run_pays(d.lat.L, d.W); };
     if (columns) {
         if (c.T > 0 || c.perfect_round)
             for (int i = 0; i < pl.items.n; ++i)
-                if (column_fits(pl.items.it[i].lat.L))
+                if (!stepwise(pl.items.it[i]))
                     T3D_TRY(launch_column_run(pl.items.it[i], c.T, c.cycle0, thr_p, thr_q, c.seed, c.schedule, slen,
                                               c.n_apply, c.perfect_round ? c.perfect_max_sweeps : -1, st));
     }
