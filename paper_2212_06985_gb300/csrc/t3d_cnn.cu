@@ -16,8 +16,8 @@
 // Training: the forward pass with the labels in the third layer's epilogue
 // (BCE gradient, the head's gradients, the ReLU mask), backward data by the
 // same tensor-core convolution with flipped and transposed weights and a
-// masking epilogue, weight and bias gradients by a CUDA-core reduction over
-// sites and samples, Adam.
+// masking epilogue, weight and bias gradients as a tensor-core GEMM over sites
+// and samples, Adam.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -230,8 +230,8 @@ extern "C" t3d_status toric3d_cnn_decode(int L, int64_t n_samples, const uint64_
 extern "C" size_t toric3d_cnn_train_workspace_bytes(int L, int64_t n_samples)
 {
     if (L < 2 || L > 128 || n_samples < 1) return 0;
-    // features, y1, y2, two gradient buffers, two channel-major copies, the ones tile, grads
-    return tc_act_bytes(L, n_samples, 8) + 6 * tc_act_bytes(L, n_samples, kC) + 4096 + round256(kParams * 4) + 256;
+    // features, y1, y2, two gradient buffers, the ones tile, grads
+    return tc_act_bytes(L, n_samples, 8) + 4 * tc_act_bytes(L, n_samples, kC) + 4096 + round256(kParams * 4) + 256;
 }
 
 extern "C" t3d_status toric3d_cnn_train_step(int L, int64_t n_samples, const uint64_t* s_prev,
@@ -258,9 +258,7 @@ extern "C" t3d_status toric3d_cnn_train_step(int L, int64_t n_samples, const uin
     uint8_t* y2 = y1 + ab;
     uint8_t* g3 = y2 + ab;              // dPre3, later dPre1
     uint8_t* g2 = g3 + ab;              // dPre2
-    uint8_t* xt = g2 + ab;              // channel-major copies for the weight gradients
-    uint8_t* dt = xt + ab;
-    uint8_t* ones = dt + ab;
+    uint8_t* ones = g2 + ab;
     float* grads = reinterpret_cast<float*>(ones + 4096);
     if (grads_out) grads = grads_out;
     const int64_t W = words_for(n_samples);
@@ -271,11 +269,11 @@ extern "C" t3d_status toric3d_cnn_train_step(int L, int64_t n_samples, const uin
     T3D_TRY(tc_train_forward(L, n_samples, W, s_prev, s, e_label, b, x0, y1, y2, g3, grads + P_W4, grads + P_B4,
                              loss_out, st));
     // backward: layer 3's weights, the data gradient into layer 2 (gated by y2 > 0), ...
-    T3D_TRY(tc_weight_grad(L, n_samples, kC, kC, y2, g3, xt, dt, ones, grads + P_W3, grads + P_B3, st));
+    T3D_TRY(tc_weight_grad(L, n_samples, kC, kC, y2, g3, ones, grads + P_W3, grads + P_B3, st));
     T3D_TRY(tc_backward_data(L, n_samples, &b->wt[2][0][0][0], g3, y2, g2, st));
-    T3D_TRY(tc_weight_grad(L, n_samples, kC, kC, y1, g2, xt, dt, ones, grads + P_W2, grads + P_B2, st));
+    T3D_TRY(tc_weight_grad(L, n_samples, kC, kC, y1, g2, ones, grads + P_W2, grads + P_B2, st));
     T3D_TRY(tc_backward_data(L, n_samples, &b->wt[1][0][0][0], g2, y1, g3, st));   // dPre1
-    T3D_TRY(tc_weight_grad(L, n_samples, 8, kInC, x0, g3, xt, dt, ones, grads + P_W1, grads + P_B1, st));
+    T3D_TRY(tc_weight_grad(L, n_samples, 8, kInC, x0, g3, ones, grads + P_W1, grads + P_B1, st));
     if (lr > 0.0f) {
         const float b1 = 0.9f, b2 = 0.999f;
         const float c1 = 1.0f - powf(b1, (float)step), c2 = 1.0f - powf(b2, (float)step);

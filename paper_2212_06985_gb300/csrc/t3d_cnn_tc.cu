@@ -41,14 +41,15 @@
 //
 // Shared-memory operand layout ("no swizzle", K-major): core matrices of 8 rows
 // x 16 bytes stored contiguously.  Hidden activations in global memory use the
-// same layout, [sample/8][channel/8][8 samples][8 channels] BF16 per tile, and
-// the tile of (site, 128-sample tile m) starts at byte (m L^3 + site) 4096, so
-// a tile is one contiguous 4 KiB block (K-direction core-matrix stride (LBO)
-// 128 B, M-direction stride (SBO) 256 B).  The first layer's input tile (6 of 8
-// channels used: s_{t-1} then s_t of the three faces) is [sample][8], 2 KiB
-// (SBO 128 B); two x-adjacent sites form one K = 16 operand as its two K chunks
-// (LBO 2 KiB).  Weight blocks: [co/8][ci/8][co%8][ci%8] (512 B, LBO 128 B,
-// SBO 256 B).
+// same layout, [channel/8][128 samples][8 channels] BF16 per tile, and the tile
+// of (site, 128-sample tile m) starts at byte (m L^3 + site) 4096, so a tile is
+// one contiguous 4 KiB block (K-direction core-matrix stride (LBO) 2 KiB,
+// M-direction stride (SBO) 128 B) and a warp of the epilogue writes 512-byte
+// runs.  The first layer's input tile (6 of 8 channels used: s_{t-1} then s_t of
+// the three faces) is [sample][8], 2 KiB (SBO 128 B); two x-adjacent sites form
+// one K = 16 operand as its two K chunks (LBO 2 KiB).  Weight blocks:
+// [co/8][ci/8][co%8][ci%8] (512 B, LBO 128 B, SBO 256 B).  The weight gradients
+// read the same tiles with samples as K (k_wgrad_tc).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -287,6 +288,20 @@ __device__ __forceinline__ void tmem_zero16(uint32_t taddr)
 __device__ __forceinline__ void tmem_wait_st()
 {
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+// One lane of a converged warp (always the same one).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile(
+        "{\n"
+        ".reg .pred q;\n"
+        "elect.sync _|q, 0xffffffff;\n"
+        "selp.u32 %0, 1, 0, q;\n"
+        "}\n"
+        : "=r"(p));
+    return p != 0;
 }
 
 // Arrive on the barrier once every MMA this thread issued so far has completed.
@@ -599,7 +614,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
             uint32_t pseq = 0;
             int64_t qbase = 0;
             bool ok = true;
-            const uint32_t a_lbo = kBitsIn ? 2048u : 128u, a_sbo = kBitsIn ? 128u : 256u;
+            constexpr uint32_t a_lbo = 2048u, a_sbo = 128u;
             const uint64_t bdesc0 = smem_desc(wsm, 128u, 256u);   // + 32 per 512-byte block
             constexpr uint32_t kIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTileM >> 4) << 24);
             for (int64_t u = blockIdx.x; u < a.n_units && ok; u += gridDim.x) {
@@ -720,7 +735,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
                     const int xo = t.x0 + (j & 1), yo = t.y + (j >> 1);
                     if (xo >= L || yo >= L) continue;   // the odd lattice's last column
                     const int64_t site = ((int64_t)zo * L + yo) * L + xo;
-                    const int64_t row_off = tile_off(site, t.m0, a.L3, 4096) + (r >> 3) * 256 + (r & 7) * 16;
+                    const int64_t row_off = tile_off(site, t.m0, a.L3, 4096) + r * 16;
                     float v[16];
 #pragma unroll
                     for (int c = 0; c < 16; ++c) v[c] = __uint_as_float(raw[j][c]);
@@ -734,7 +749,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
                             // the gradient passes where the forward activation (a ReLU output,
                             // so never negative) is non-zero
                             const uint4 m0v = *reinterpret_cast<const uint4*>(a.mask_act + row_off);
-                            const uint4 m1v = *reinterpret_cast<const uint4*>(a.mask_act + row_off + 128);
+                            const uint4 m1v = *reinterpret_cast<const uint4*>(a.mask_act + row_off + 2048);
                             const uint32_t mw[8] = {m0v.x, m0v.y, m0v.z, m0v.w, m1v.x, m1v.y, m1v.z, m1v.w};
 #pragma unroll
                             for (int c = 0; c < kC; c += 2)
@@ -743,7 +758,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
                         }
                         uint8_t* dst = a.out + row_off;
                         *reinterpret_cast<uint4*>(dst) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                        *reinterpret_cast<uint4*>(dst + 128) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                        *reinterpret_cast<uint4*>(dst + 2048) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
                     } else {
                         float y3[kC];
                         float z[3] = {b4[0], b4[1], b4[2]};
@@ -794,7 +809,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
                             }
                             uint8_t* dst = a.out + row_off;
                             *reinterpret_cast<uint4*>(dst) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
-                            *reinterpret_cast<uint4*>(dst + 128) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+                            *reinterpret_cast<uint4*>(dst + 2048) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
                         }
                     }
                 }
@@ -865,174 +880,199 @@ __global__ void k_expand_bits(int L3, int64_t Sp, int64_t W, int64_t words, cons
 // ------------------------------------------------------------------ weight gradients
 // Weight and bias gradients of one convolution as a GEMM over samples:
 //   G[(k, ci)][co] = sum over sites r and samples s of x[r + off_k][s][ci] . d[r][s][co],
-// M = 128 rows (8 offsets x 16 input channels; the first layer 16 x 8), N = 16 output
-// channels, K = 16 samples per MMA.  The reduction runs over samples, so both operands are
-// channel-major copies of the tiles (k_channel_major): a tile of C channels x 128 samples is
-// [C/8][sample/8][8 channels][8 samples] BF16, K-major core matrices with LBO 128 B (the next
-// 8 samples) and SBO 2048 B (the next 8 channels -- also the step to the next tile of an M
-// group, so the 8 (16) neighbour tiles of a group sit at a uniform stride).  The 28th
-// "offset" is a tile of ones: its rows give the bias gradient sum d[r][s][co].  Work item:
-// one (128-sample tile, site); per item the d tile and, per M group, its neighbour tiles are
-// copied into rings of slots, and the group's accumulator in TMEM (16 columns) takes 8 MMAs.
-// The accumulators live for the whole launch and are added to the gradients at the end.
-// Rows beyond offset 27 multiply whatever the slot holds and are never read.
-constexpr int kWgX = 6;                       // group slots, 32 KiB each
-constexpr int kWgD = 4;                       // d-tile slots, 4 KiB each
-constexpr int kWgOffD = kWgX * 32768;
-constexpr int kWgOffBar = kWgOffD + kWgD * 4096;
-constexpr int kWgNumBars = 2 * kWgX + 2 * kWgD + 1;   // x full, x empty, d full, d empty, done
-constexpr int kWgOffMisc = kWgOffBar + kWgNumBars * 8;
-constexpr int kWgSmemBytes = kWgOffMisc + 16 + 1024;
-static_assert(kWgSmemBytes <= 227 * 1024, "shared memory budget");
+// K = 16 samples per MMA.  The reduction runs over samples; both operands are the convolutions'
+// own tiles read with the channels as the contiguous dimension (core matrices of 8 samples x 8
+// channels, LBO 128 B to the next 8 samples, SBO 2048 B to the next 8 channels, which is also the
+// step to the next tile of a run).
+//
+// Work unit: one 128-sample tile x one row (y, z), walked along x.  The 9 tiles around the row at
+// one x, (dy, dz) = -1..1, form a column.  A column meets the d tiles of the three sites
+// x - 1, x, x + 1 as dx = +1, 0, -1 at once: the MMA's M rows are the column's tiles (and a tile of
+// ones, whose rows give the bias gradient sum d[r][s][co]), its N = 48 columns those three d tiles.
+// So every x tile is copied and multiplied once per row, ten tiles a site with d's, where fetching
+// a site's 27 neighbours took 29 tiles; and a site takes 16 MMAs (first layer: 8) where N = 16
+// columns per neighbour took 32 (16).  M is 128: eight 16-channel tiles, then the ninth and the ones
+// in an MMA of their own; the first layer's nine 8-channel tiles and the ones fit one.  Rows past a
+// group's last tile multiply whatever follows in shared memory and are never read.
+//
+// The d tiles sit in a ring of eight slots whose first two are written a second time behind the last,
+// so that any three in a row are contiguous.  The accumulators (48 columns of TMEM per group) live for
+// the whole launch and are added to the gradients at its end.
+//
+// What bounds it: the MMAs (16 a site, 53 cycles each however small N is, 80 us) and the copies to
+// shared memory (42 KB a site, 1.2 GB; about 10 TB/s) alike.  L = 12, 2,048 samples: 113 us for a
+// 16-channel layer, 98 us for the first.  Before, with channel-major copies of x and d written first
+// (350 us a step in all), 27 neighbour tiles fetched per site and N = 16: 490 and 330 us.
+//
+// One elected thread of a converged warp issues the MMAs, and one of each of three producer warps the
+// copies: warp and loop state are then uniform, and addresses and descriptors stay in uniform
+// registers.  From a branch on the lane index every MMA took 94 - 112 cycles to issue and every copy
+// 117 - 190 (164 and 154 us a launch).
+constexpr int kWgProducers = 3;
+constexpr int kWgThreads = kTcThreads + 32 * (kWgProducers - 1);
+
+template <int kCin>
+struct WgShape {
+    static constexpr uint32_t kTileB = kCin * 256;               // one x tile
+    static constexpr uint32_t kColB = 10 * kTileB;               // nine tiles and the ones
+    static constexpr int kCols = kCin == 16 ? 4 : 6;             // column slots
+    static constexpr int kGroups = kCin == 16 ? 2 : 1;           // M groups: tiles 0..7 and 8..9
+    static constexpr int kD = 8;                                 // d slots (and two mirrors), 4 KiB each
+    static constexpr uint32_t kOffD = kCols * kColB;
+    static constexpr uint32_t kOffBar = kOffD + (kD + 2) * 4096;
+    static constexpr int kBars = 2 * kCols + kD + 1;             // column full, empty; d empty; done
+    static constexpr uint32_t kOffMisc = kOffBar + kBars * 8;
+    static constexpr int kSmem = (int)kOffMisc + 16 + 1024;
+    static_assert(kSmem <= 227 * 1024, "shared memory budget");
+    // a group reads 32 KiB from its first tile on
+    static_assert(kOffBar >= (kCols - 1) * kColB + (kGroups - 1) * 8 * kTileB + 32768, "group reads stay inside");
+};
 
 struct WgArgs {
     int L, L3;
-    int64_t n_items;            // 128-sample tiles x L^3 sites
-    const uint8_t* xt;          // channel-major x tiles (kCin channels)
-    const uint8_t* dt;          // channel-major d tiles (16 channels)
+    int64_t n_units;            // 128-sample tiles x L^2 rows
+    const uint8_t* x;           // x tiles (kCin channels)
+    const uint8_t* d;           // d tiles (16 channels)
     const uint8_t* ones;        // one x tile of BF16 ones
     int cin;                    // input channels kept in gw (6 for the first layer)
     float* gw;                  // [co][cin][27], accumulated
     float* gb;                  // [16], accumulated
 };
 
-// Site r + offset k (k = (dz + 1) 9 + (dy + 1) 3 + (dx + 1)), periodic.
-__device__ __forceinline__ int64_t wg_neighbour(int r, int k, int L)
-{
-    const int x = r % L, y = (r / L) % L, z = r / (L * L);
-    const int dx = k % 3 - 1, dy = (k / 3) % 3 - 1, dz = k / 9 - 1;
-    return ((int64_t)wrap(z + dz, L) * L + wrap(y + dy, L)) * L + wrap(x + dx, L);
-}
-
 template <int kCin>
-__global__ void __launch_bounds__(kTcThreads, 1) k_wgrad_tc(const __grid_constant__ WgArgs a)
+__global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constant__ WgArgs a)
 {
-    constexpr uint32_t kTileB = kCin * 256;
-    constexpr int kPer = 128 / kCin;                         // offsets per M group
-    constexpr int kGroups = (kOff + 1 + kPer - 1) / kPer;    // 4, or 2 for the first layer
+    using Sh = WgShape<kCin>;
+    constexpr uint32_t kTileB = Sh::kTileB;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t base = smem_u32(sm);
-    const uint32_t bars = base + kWgOffBar;
-    auto xfull = [&](int i) { return bars + 8u * (uint32_t)i; };
-    auto xempty = [&](int i) { return bars + 8u * (uint32_t)(kWgX + i); };
-    auto dfull = [&](int i) { return bars + 8u * (uint32_t)(2 * kWgX + i); };
-    auto dempty = [&](int i) { return bars + 8u * (uint32_t)(2 * kWgX + kWgD + i); };
-    const uint32_t done_bar = bars + 8u * (uint32_t)(2 * kWgX + 2 * kWgD);
-    uint32_t* misc = reinterpret_cast<uint32_t*>(sm + kWgOffMisc);   // [0] TMEM base, [1] abort, [2] progress
+    const uint32_t bars = base + Sh::kOffBar;
+    // use q of a ring of n goes to slot q % n, its phase parity is (q / n) & 1
+    constexpr uint32_t kNc = Sh::kCols, kNd = Sh::kD;
+    auto col_full = [&](uint32_t q) { return bars + 8u * (q % kNc); };
+    auto col_empty = [&](uint32_t q) { return bars + 8u * (kNc + q % kNc); };
+    auto d_empty = [&](uint32_t q) { return bars + 8u * (2 * kNc + q % kNd); };
+    auto col_at = [&](uint32_t q) { return base + (q % kNc) * Sh::kColB; };
+    auto d_at = [&](uint32_t q) { return base + Sh::kOffD + (q % kNd) * 4096u; };
+    const uint32_t done_bar = bars + 8u * (2 * kNc + kNd);
+    uint32_t* misc = reinterpret_cast<uint32_t*>(sm + Sh::kOffMisc);   // [0] TMEM base, [1] abort, [2] progress
     volatile uint32_t* abort_flag = misc + 1;
     volatile uint32_t* progress = misc + 2;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the shuffle makes the warp index uniform for the compiler
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
         misc[2] = 0;
-        for (int i = 0; i < kWgX; ++i) {
-            mbar_init(xfull(i), 1);
-            mbar_init(xempty(i), 1);
-        }
-        for (int i = 0; i < kWgD; ++i) {
-            mbar_init(dfull(i), 1);
-            mbar_init(dempty(i), 1);
-        }
-        mbar_init(done_bar, 1);
+        for (int i = 0; i < Sh::kBars; ++i) mbar_init(bars + 8u * (uint32_t)i, i < Sh::kCols ? kWgProducers : 1);
         misc[1] = 0;
         fence_mbar_init();
     }
-    if (warp == kIssuerWarp) tmem_alloc(smem_u32(misc), 64);
+    // the ones behind every column's nine tiles
+    for (uint32_t i = threadIdx.x; i < kNc * (kTileB / 16); i += blockDim.x)
+        reinterpret_cast<uint4*>(sm + (i / (kTileB / 16)) * Sh::kColB + 9u * kTileB)[i % (kTileB / 16)] =
+            reinterpret_cast<const uint4*>(a.ones)[i % (kTileB / 16)];
+    fence_proxy_async_smem();
+    if (warp == kIssuerWarp) tmem_alloc(smem_u32(misc), 128);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = misc[0];
-    const int L = a.L;
+    const uint32_t tmem = __shfl_sync(0xffffffffu, misc[0], 0);
+    const int L = a.L, L2 = L * L;
 
-    if (warp == kProducerWarp) {
-        uint32_t xs = 0, ds = 0;
+    if (warp == kProducerWarp || warp > kIssuerWarp) {
+        // producer p copies the tiles 3 p .. 3 p + 2 of a column, the last one the d tiles too
+        const int part = warp == kProducerWarp ? 0 : warp - kIssuerWarp;
+        const bool leader = elect_one();
+        uint32_t cq = 0, dq = 0;   // columns and d tiles copied so far
         bool ok = true;
-        for (int64_t u = blockIdx.x; u < a.n_items && ok; u += gridDim.x) {
-            const int64_t t = u / a.L3;
-            const int r = (int)(u - t * a.L3);
-            {
-                const int g = (int)(ds % kWgD);
-                const uint32_t use = ds / kWgD;
-                int good = 1;
-                if (lane == 0 && use > 0) good = wait_bar(dempty(g), (use - 1) & 1u, abort_flag) ? 1 : 0;
-                if (!__shfl_sync(0xffffffffu, good, 0)) break;
-                if (lane == 0) {
-                    mbar_arrive_expect_tx(dfull(g), 4096u);
-                    bulk_load(base + kWgOffD + (uint32_t)g * 4096u, a.dt + (t * a.L3 + r) * 4096, 4096u, dfull(g));
+        for (int64_t u = blockIdx.x; u < a.n_units && ok; u += gridDim.x) {
+            const int64_t t = u / L2;
+            const int row = (int)(u - t * L2), y = row % L, z = row / L;
+            const uint8_t* xt = a.x + t * a.L3 * (int64_t)kTileB;
+            const uint8_t* dt = a.d + (t * a.L3 + (int64_t)row * L) * 4096;
+            // the row of tile i = 3 part + k: (dy, dz) = (i % 3 - 1, i / 3 - 1) = (k - 1, part - 1)
+            const uint8_t* xrow[3];
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                xrow[k] = xt + ((int64_t)wrap(z + part - 1, L) * L + wrap(y + k - 1, L)) * L * (int64_t)kTileB;
+            for (int c = 0; c < L; ++c) {
+                // d tiles in the order L - 1, 0, 1, .., L - 1, 0: the first column brings three of them
+                const uint32_t nd = part != 2 ? 0 : (c == 0 ? 3 : 1);
+                uint32_t mirrors = 0;
+                for (uint32_t k = dq; k < dq + nd; ++k) mirrors += k % kNd < 2 ? 1u : 0u;
+                bool good = true;
+                if (leader) {
+                    if (cq >= kNc) good = wait_bar(col_empty(cq), ((cq / kNc) - 1) & 1u, abort_flag);
+                    for (uint32_t k = dq; good && k < dq + nd; ++k)
+                        if (k >= kNd) good = wait_bar(d_empty(k), ((k / kNd) - 1) & 1u, abort_flag);
                 }
-                ++ds;
-            }
-            for (int grp = 0; grp < kGroups; ++grp) {
-                const int g = (int)(xs % kWgX);
-                const uint32_t use = xs / kWgX;
-                int good = 1;
-                if (lane == 0 && use > 0) good = wait_bar(xempty(g), (use - 1) & 1u, abort_flag) ? 1 : 0;
-                if (!__shfl_sync(0xffffffffu, good, 0)) {
-                    ok = false;
-                    break;
+                ok = __all_sync(0xffffffffu, good);
+                if (!ok) break;
+                if (leader) mbar_arrive_expect_tx(col_full(cq), 3u * kTileB + (nd + mirrors) * 4096u);
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    if (leader)
+                        bulk_load(col_at(cq) + (uint32_t)(3 * part + k) * kTileB, xrow[k] + (uint32_t)c * kTileB, kTileB,
+                                  col_full(cq));
+                for (uint32_t k = dq; k < dq + nd; ++k) {
+                    const uint8_t* src = dt + (int64_t)wrap(c + 1 - (int)(dq + nd - 1 - k), L) * 4096;
+                    if (leader) bulk_load(d_at(k), src, 4096u, col_full(cq));
+                    if (leader && k % kNd < 2) bulk_load(d_at(k) + kNd * 4096u, src, 4096u, col_full(cq));
                 }
-                const int k0 = grp * kPer;
-                const int n_real = min(kPer, kOff + 1 - k0);     // offsets and the ones tile
-                if (lane == 0) mbar_arrive_expect_tx(xfull(g), (uint32_t)n_real * kTileB);
-                __syncwarp();
-                if (lane < n_real) {
-                    const int k = k0 + lane;
-                    const uint8_t* src = k < kOff ? a.xt + (t * a.L3 + wg_neighbour(r, k, L)) * kTileB : a.ones;
-                    bulk_load(base + (uint32_t)g * 32768u + (uint32_t)lane * kTileB, src, kTileB, xfull(g));
-                }
-                ++xs;
+                ++cq;
+                dq += nd;
             }
         }
         // copies still in flight land before the CTA exits
-        if (lane == 0) {
-            const uint32_t lx = xs < (uint32_t)kWgX ? xs : (uint32_t)kWgX;
-            for (uint32_t g = 0; g < lx; ++g) {
-                const uint32_t q = xs - 1 - ((xs - 1 - g) % kWgX);
-                wait_bar(xfull((int)g), (q / kWgX) & 1u, abort_flag, true);
-            }
-            const uint32_t ld = ds < (uint32_t)kWgD ? ds : (uint32_t)kWgD;
-            for (uint32_t g = 0; g < ld; ++g) {
-                const uint32_t q = ds - 1 - ((ds - 1 - g) % kWgD);
-                wait_bar(dfull((int)g), (q / kWgD) & 1u, abort_flag, true);
-            }
-        }
+        if (leader)
+            for (uint32_t k = cq > kNc ? cq - kNc : 0; k < cq; ++k)
+                wait_bar(col_full(k), (k / kNc) & 1u, abort_flag, true);
         __syncwarp();
     } else if (warp == kIssuerWarp) {
-        if (lane == 0) {
-            constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(16 >> 3) << 17) |
-                                        ((uint32_t)(kTileM >> 4) << 24);
-            uint32_t xs = 0, ds = 0;
-            bool ok = true, first = true;
-            for (int64_t u = blockIdx.x; u < a.n_items && ok; u += gridDim.x) {
-                const int gd = (int)(ds % kWgD);
-                if (!wait_bar(dfull(gd), (ds / kWgD) & 1u, abort_flag)) break;
+        const bool leader = elect_one();
+        // A and B are read with their channels as the contiguous dimension (bits 15 and 16)
+        constexpr uint32_t kIdesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | (1u << 16) |
+                                    ((uint32_t)(48 >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
+        uint32_t cq = 0, dq = 0;   // columns done; the first d tile of the current column's three
+        bool ok = true;
+        for (int64_t u = blockIdx.x; u < a.n_units && ok; u += gridDim.x) {
+            for (int c = 0; c < L; ++c) {
+                bool good = true;
+                if (leader) good = wait_bar(col_full(cq), (cq / kNc) & 1u, abort_flag);
+                ok = __all_sync(0xffffffffu, good);
+                if (!ok) break;
                 tc_fence_after();
-                const uint64_t bdesc = smem_desc(base + kWgOffD + (uint32_t)gd * 4096u, 128u, 2048u);
-                for (int grp = 0; grp < kGroups; ++grp) {
-                    const int g = (int)(xs % kWgX);
-                    if (!wait_bar(xfull(g), (xs / kWgX) & 1u, abort_flag)) {
-                        ok = false;
-                        break;
-                    }
-                    tc_fence_after();
-                    const uint64_t adesc = smem_desc(base + (uint32_t)g * 32768u, 128u, 2048u);
+                const uint64_t bdesc = smem_desc(d_at(dq), 128u, 2048u);
+#pragma unroll
+                for (int grp = 0; grp < Sh::kGroups; ++grp) {
+                    const uint64_t adesc = smem_desc(col_at(cq) + (uint32_t)grp * 8u * kTileB, 128u, 2048u);
 #pragma unroll
                     for (int kk = 0; kk < 8; ++kk) {
                         // 16 samples per step: two core matrices (256 B) further along K
                         const uint64_t step = (uint64_t)((kk * 256) >> 4);
-                        if (first && kk == 0)
-                            mma_bf16_overwrite(tmem + (uint32_t)(grp * 16), adesc + step, bdesc + step, kIdesc);
-                        else
-                            mma_bf16_n(tmem + (uint32_t)(grp * 16), adesc + step, bdesc + step, kIdesc);
+                        if (leader) {
+                            if (kk == 0 && cq == 0)
+                                mma_bf16_overwrite(tmem + (uint32_t)(grp * 48), adesc + step, bdesc + step, kIdesc);
+                            else
+                                mma_bf16_n(tmem + (uint32_t)(grp * 48), adesc + step, bdesc + step, kIdesc);
+                        }
                     }
-                    mma_commit(xempty(g));
-                    ++xs;
                 }
-                first = false;
-                mma_commit(dempty(gd));
-                ++ds;
-                *progress = ds;
+                if (leader) {
+                    mma_commit(col_empty(cq));
+                    mma_commit(d_empty(dq));
+                    if (c == L - 1) {   // the row's last two d tiles serve no further column
+                        mma_commit(d_empty(dq + 1));
+                        mma_commit(d_empty(dq + 2));
+                    }
+                }
+                ++cq;
+                ++dq;
+                if (leader) *progress = cq;
             }
+            dq += 2;
+        }
+        if (leader) {
             mma_commit(done_bar);
             wait_bar(done_bar, 0, abort_flag, true);
         }
@@ -1044,20 +1084,24 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_wgrad_tc(const __grid_constan
         got = __shfl_sync(0xffffffffu, got, 0);
         tc_fence_after();
         if (got && !*abort_flag) {
-            const int row = warp * 32 + lane;
+            const int m = warp * 32 + lane, ci = m % kCin;
 #pragma unroll
-            for (int grp = 0; grp < kGroups; ++grp) {
-                uint32_t v[16];
-                tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(grp * 16), v);
-                tmem_wait_ld();
-                const int k = grp * kPer + row / kCin, ci = row % kCin;
-                if (k < kOff && ci < a.cin) {
+            for (int grp = 0; grp < Sh::kGroups; ++grp) {
+                const int i = grp * 8 + m / kCin;   // the row's tile of the column, (dy, dz) = i
+                const bool mine = kCin == 8 || grp == 1 || i < 8;
 #pragma unroll
-                    for (int co = 0; co < 16; ++co)
-                        atomicAdd(&a.gw[(co * a.cin + ci) * kOff + k], __uint_as_float(v[co]));
-                } else if (k == kOff && ci == 0) {
+                for (int j = 0; j < 3; ++j) {       // the site c - 1 + j: dx = 1 - j
+                    uint32_t v[16];
+                    tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(grp * 48 + j * 16), v);
+                    tmem_wait_ld();
+                    if (mine && i < 9 && ci < a.cin) {
 #pragma unroll
-                    for (int co = 0; co < 16; ++co) atomicAdd(&a.gb[co], __uint_as_float(v[co]));
+                        for (int co = 0; co < 16; ++co)
+                            atomicAdd(&a.gw[(co * a.cin + ci) * kOff + 3 * i + 2 - j], __uint_as_float(v[co]));
+                    } else if (mine && i == 9 && ci == 0 && j == 1) {
+#pragma unroll
+                        for (int co = 0; co < 16; ++co) atomicAdd(&a.gb[co], __uint_as_float(v[co]));
+                    }
                 }
             }
         }
@@ -1066,28 +1110,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_wgrad_tc(const __grid_constan
     __syncthreads();
     if (warp == kIssuerWarp) {
         tc_fence_after();
-        tmem_dealloc(tmem, 64);
-    }
-}
-
-// Channel-major copy of C-channel tiles (k_wgrad_tc's operands): the element (sample m,
-// channel c) of a tile moves from the tile-major place ([m/8][c/8][8][8] for 16 channels,
-// [m][8] for 8) to [c/8][m/8][8 channels][8 samples].  One block per tile.
-template <int kCh>
-__global__ void __launch_bounds__(256) k_channel_major(const uint16_t* __restrict__ src, uint16_t* __restrict__ dst)
-{
-    constexpr int kN = kCh * 128;
-    __shared__ uint16_t tile[kN];
-    const int64_t t = blockIdx.x;
-    for (int i = threadIdx.x; i < kN / 8; i += blockDim.x)
-        reinterpret_cast<uint4*>(tile)[i] = reinterpret_cast<const uint4*>(src + t * kN)[i];
-    __syncthreads();
-    for (int i = threadIdx.x; i < kN; i += blockDim.x) {
-        // destination index i = ((c/8) 16 + m/8) 64 + (c%8) 8 + m%8
-        const int ms = i & 7, cs = (i >> 3) & 7, mg = (i >> 6) & 15, cg = i >> 10;
-        const int m = mg * 8 + ms, c = cg * 8 + cs;
-        const int from = kCh == 16 ? ((m >> 3) * 2 + (c >> 3)) * 64 + (m & 7) * 8 + (c & 7) : m * 8 + c;
-        dst[t * kN + i] = tile[from];
+        tmem_dealloc(tmem, 128);
     }
 }
 
@@ -1161,8 +1184,8 @@ t3d_status tc_prepare()
         T3D_CUDA_CHECK(cudaFuncSetAttribute(k_conv_col<kTcHead, false>, attr, kColSmemBytes));
         T3D_CUDA_CHECK(cudaFuncSetAttribute(k_conv_col<kTcHeadTrain, false>, attr, kColSmemBytes));
         T3D_CUDA_CHECK(cudaFuncSetAttribute(k_conv_col<kTcMask, false>, attr, kColSmemBytes));
-        T3D_CUDA_CHECK(cudaFuncSetAttribute(k_wgrad_tc<8>, attr, kWgSmemBytes));
-        T3D_CUDA_CHECK(cudaFuncSetAttribute(k_wgrad_tc<kC>, attr, kWgSmemBytes));
+        T3D_CUDA_CHECK(cudaFuncSetAttribute(k_wgrad_tc<8>, attr, WgShape<8>::kSmem));
+        T3D_CUDA_CHECK(cudaFuncSetAttribute(k_wgrad_tc<kC>, attr, WgShape<kC>::kSmem));
         configured[dev] = true;
     }
     return T3D_OK;
@@ -1261,7 +1284,7 @@ t3d_status tc_fill_ones(uint8_t* tile, cudaStream_t st)
 }
 
 t3d_status tc_weight_grad(int L, int64_t n_samples, int x_ch, int cin_kept, const uint8_t* x, const uint8_t* d,
-                          uint8_t* xt, uint8_t* dt, const uint8_t* ones, float* gw, float* gb, cudaStream_t st)
+                          const uint8_t* ones, float* gw, float* gb, cudaStream_t st)
 {
     T3D_REQUIRE(x_ch == 8 || x_ch == kC, "weight gradient: %d input channels", x_ch);
     T3D_TRY(tc_prepare());
@@ -1269,31 +1292,22 @@ t3d_status tc_weight_grad(int L, int64_t n_samples, int x_ch, int cin_kept, cons
     T3D_REQUIRE(n_items <= 0x7fffffffLL, "weight gradient: %lld (sample tile, site) pairs exceed one grid",
                 (long long)n_items);
     ProfScope prof(T3D_K_CNN, st);
-    if (x_ch == 8)
-        k_channel_major<8><<<(unsigned)n_items, 256, 0, st>>>(reinterpret_cast<const uint16_t*>(x),
-                                                              reinterpret_cast<uint16_t*>(xt));
-    else
-        k_channel_major<kC><<<(unsigned)n_items, 256, 0, st>>>(reinterpret_cast<const uint16_t*>(x),
-                                                               reinterpret_cast<uint16_t*>(xt));
-    k_channel_major<kC><<<(unsigned)n_items, 256, 0, st>>>(reinterpret_cast<const uint16_t*>(d),
-                                                           reinterpret_cast<uint16_t*>(dt));
-    T3D_LAUNCH_CHECK("channel-major tiles");
     WgArgs a;
     std::memset(&a, 0, sizeof(a));
     a.L = L;
     a.L3 = (int)L3;
-    a.n_items = n_items;
-    a.xt = xt;
-    a.dt = dt;
+    a.n_units = n_items / L;
+    a.x = x;
+    a.d = d;
     a.ones = ones;
     a.cin = cin_kept;
     a.gw = gw;
     a.gb = gb;
-    const int grid = (int)std::min<int64_t>(n_items, sm_count());
+    const int grid = (int)std::min<int64_t>(a.n_units, sm_count());
     if (x_ch == 8)
-        k_wgrad_tc<8><<<grid, kTcThreads, kWgSmemBytes, st>>>(a);
+        k_wgrad_tc<8><<<grid, kWgThreads, WgShape<8>::kSmem, st>>>(a);
     else
-        k_wgrad_tc<kC><<<grid, kTcThreads, kWgSmemBytes, st>>>(a);
+        k_wgrad_tc<kC><<<grid, kWgThreads, WgShape<kC>::kSmem, st>>>(a);
     T3D_LAUNCH_CHECK("tensor-core weight gradient");
     return T3D_OK;
 }
