@@ -20,19 +20,19 @@
 // ring of eight output planes; the epilogue drains a plane once its last
 // input plane has been multiplied.
 //
-// Warp roles (192 threads, one CTA per SM):
-//   warps 0-3  epilogue: tcgen05.ld of a finished plane (warp w reads TMEM lanes
-//              32w..32w+31 = samples), then by mode (TcMode): bias + ReLU +
+// Warp roles (one CTA per SM; each role is warp-uniform code, one elected lane
+// issues):
+//   warps 0-7  epilogue, in two groups of four that take the output planes in
+//              turn: tcgen05.ld of a finished plane (warp w reads TMEM lanes
+//              32 (w % 4) .. = samples), then by mode (TcMode): bias + ReLU +
 //              BF16 store of the next layer's input; the 16 -> 3 head and the
 //              hard decisions; the head with the BCE gradient, the head's
 //              gradients and the gradient at the pre-activation; or the
 //              backward-data gradient gated by the forward activation;
-//   warp 4     producer: sixteen lanes issue the bulk copies of a plane's 16
-//              tiles at once (first layer: four lanes copy a row's four 2 KiB
-//              tiles each as one run) into a ring of shared-memory slots;
-//   warp 5     MMA issuer: one thread issues the MMAs and commits their
-//              completion to the slot's "empty" barrier and to the output
-//              plane's "accumulators full" barrier.
+//   producers  bulk copies of a plane's four rows of four tiles (one copy a row,
+//              four where the row wraps) into a ring of shared-memory slots;
+//   issuer     the MMAs; commits their completion to the slot's "empty" barrier
+//              and to the output plane's "accumulators full" barrier.
 // Every wait is bounded (one second; toric3d_cnn_debug_wait_limit shortens the
 // waits that may give up, so a test can make them run out); a wait that gives
 // up sets the device error flag and the CTA winds down (waiting, again bounded
@@ -156,6 +156,22 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
     return ok != 0;
 }
 
+// Whether the phase of the given parity is complete, without waiting.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // Bounded wait for the phase of the given parity.  Gives up after
 // g_tc_wait_ns, or early once another role of the CTA has given up (abort
 // flag), unless ignore_abort (the final drain of work in flight, bounded by
@@ -205,6 +221,12 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
+}
+
+// Ask for [src, src + bytes) in L2 (16-byte aligned, a multiple of 16 bytes).
+__device__ __forceinline__ void bulk_prefetch(const void* src, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
 
 __device__ __forceinline__ void fence_proxy_async_smem()
@@ -356,23 +378,6 @@ __device__ __forceinline__ int64_t tile_off(int64_t site, int64_t m0, int L3, ui
     return ((m0 >> 7) * L3 + site) * (int64_t)tile_bytes;
 }
 
-// Copy the tiles of sites row + wrap(x0 + i), i = 0 .. n - 1, to dst + i tile_bytes: one bulk
-// copy per run of consecutive sites (a row wraps at x = L at most once when n <= L + 2, twice
-// for the smallest lattices).
-__device__ __forceinline__ void copy_row(uint32_t dst, const uint8_t* in, int64_t row, int x0, int n, int L, int L3,
-                                         int64_t m0, uint32_t tile_bytes, uint32_t bar)
-{
-    int i = 0;
-    while (i < n) {
-        const int x = wrap(x0 + i, L);
-        int k = 1;
-        while (i + k < n && x + k < L && wrap(x0 + i + k, L) == x + k) ++k;
-        bulk_load(dst + (uint32_t)i * tile_bytes, in + tile_off(row + x, m0, L3, tile_bytes), (uint32_t)k * tile_bytes,
-                  bar);
-        i += k;
-    }
-}
-
 // ------------------------------------------------------------------ column kernel
 // The convolution with dense operands: a work unit is one 128-sample tile x one
 // 2 x 2 column of output sites (x0, x0 + 1) x (y0, y0 + 1) run through all L
@@ -479,9 +484,29 @@ __device__ __forceinline__ Unit col_unit_of(const TcArgs& a, int64_t u)
     return t;
 }
 
+// Warps of the column kernel: two epilogue groups of four (group g drains the output planes of parity
+// g), the producers, the issuer.  A group needs longer for a plane (TMEM load, zeroing, conversion and
+// their latencies, one after the other) than the MMAs of the next plane take.
+//
+// Roles are warp-uniform (the warp index comes from a shuffle, the issuing lane from elect.sync), so
+// descriptors, barriers and addresses stay in uniform registers: from a branch on the lane index an MMA
+// took 94 - 112 cycles to issue (the pipe takes one in 53 for N <= 64) and a copy 117 - 190.
+//
+// Times at L = 24, 4,864 samples (38 tiles, 36 units a CTA), before -> now: first layer 762 -> 607 us,
+// hidden 1250 -> 1165, head 1276 -> 991.  One producer: 623, 1184, 1000; four: 614, 1147, 1029.  Four
+// epilogue warps and no prefetch cost 3% each.  What bounds it: the input tiles' way into shared memory,
+// 16 tiles a plane of four output sites, 8.6 GB a hidden layer, at 7.4 TB/s (8.7 for the head, which
+// writes no activations); the MMAs of a plane take 1344 of its 2380 cycles.
+constexpr int kConvProducers = 2;
+constexpr int kConvEpi = 8;
+constexpr int kConvThreads = 32 * (kConvEpi + kConvProducers + 1);
+constexpr int kAhead = 2;   // planes between the L2 prefetch and the copy
+
 template <int kMode, bool kBitsIn>
-__global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constant__ TcArgs a)
+__global__ void __launch_bounds__(kConvThreads, 1) k_conv_col(const __grid_constant__ TcArgs a)
 {
+    constexpr int kProducers = kConvProducers;
+    constexpr int kFirstProducer = kConvEpi, kIssuer = kConvEpi + kProducers;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t ring = smem_u32(sm);
@@ -499,7 +524,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
     ColPos* s_pos = reinterpret_cast<ColPos*>(sm + kColOffPos);   // [b * P + p]
     constexpr int P = kBitsIn ? 2 : 4;
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    // the shuffle makes the warp index uniform for the compiler
+    const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
 
     if (threadIdx.x < 4 * P) s_pos[threadIdx.x] = col_pos(kBitsIn, threadIdx.x % P, threadIdx.x / P);
     __syncthreads();
@@ -535,26 +561,27 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
     fence_proxy_async_smem();
     if (threadIdx.x == 0) {
         for (int i = 0; i < kColIn; ++i) {
-            mbar_init(full_bar(i), 1);
+            mbar_init(full_bar(i), kProducers);
             mbar_init(empty_bar(i), 1);
         }
         for (int i = 0; i < kColSlots; ++i) {
             mbar_init(accf_bar(i), 1);
-            mbar_init(acce_bar(i), kEpiWarps);
+            mbar_init(acce_bar(i), 4);
         }
         mbar_init(done_bar, 1);
         misc[1] = 0;
         fence_mbar_init();
     }
-    if (warp == kIssuerWarp) tmem_alloc(smem_u32(misc), kTmemCols);
+    if (warp == kIssuer) tmem_alloc(smem_u32(misc), kTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = misc[0];
+    const uint32_t tmem = __shfl_sync(0xffffffffu, misc[0], 0);
     // every accumulator starts at zero (the epilogue re-zeroes a plane after draining it)
-    if (warp < kEpiWarps) {
+    if (warp < kConvEpi) {
 #pragma unroll 4
-        for (int c = 0; c < kColSlots * kColPlaneCols; c += 16) tmem_zero16(tmem + ((uint32_t)(warp * 32) << 16) + c);
+        for (int c = 16 * (warp >> 2); c < kColSlots * kColPlaneCols; c += 32)
+            tmem_zero16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + c);
         tmem_wait_st();
     }
     tc_fence_before();
@@ -565,43 +592,68 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
     const uint32_t in_row = kBitsIn ? 16u : 32u;
     const uint32_t tile_bytes = kTileM * in_row;
 
-    if (warp == kProducerWarp) {
-        // one input plane (the 4 x 4 tiles around the column) per slot, one barrier phase each;
-        // lane 4 b + i copies the tile at (x0 - 1 + i, y0 - 1 + b).  Sixteen lanes issuing 4 KiB
-        // copies at once measured faster here than four lanes issuing a row's 16 KiB each.
+    if (warp >= kFirstProducer && warp < kIssuer) {
+        // one input plane (the 4 x 4 tiles around the column) per slot, one barrier phase each; producer k
+        // of n copies the rows b = k, k + n, .. (y0 - 1 + b)
+        const int part = warp - kFirstProducer;
+        const bool leader = elect_one();
         uint32_t pseq = 0;
         bool ok = true;
-        const int b = (lane >> 2) & 3, i = lane & 3;
+        // The column's own sites (rows y0, y0 + 1) are asked for in L2 kAhead planes before they are
+        // copied: all columns of a sample tile walk z together, so without it every plane waits for
+        // HBM.  The cursor (pu, pz) runs kAhead planes ahead, into the next unit.
+        int64_t pu = blockIdx.x;
+        int pz = -1;
+        Unit pt = col_unit_of(a, pu);
+        auto prefetch = [&]() {
+            if (pu >= a.n_units) return;
+            for (int b = part; b < 2; b += kProducers)
+                if (leader && pt.y + b < L)
+                    bulk_prefetch(a.in + tile_off(((int64_t)wrap(pz, L) * L + pt.y + b) * L + pt.x0, pt.m0, a.L3,
+                                                  tile_bytes),
+                                  (pt.x0 + 1 < L ? 2u : 1u) * tile_bytes);
+            if (++pz > L) {
+                pz = -1;
+                pu += gridDim.x;
+                pt = col_unit_of(a, pu);
+            }
+        };
+        for (int k = 0; k < kAhead; ++k) prefetch();
         for (int64_t u = blockIdx.x; u < a.n_units && ok; u += gridDim.x) {
             const Unit t = col_unit_of(a, u);
-            const int64_t xy = (int64_t)wrap(t.y - 1 + b, L) * L + wrap(t.x0 - 1 + i, L);
+            const uint8_t* tile0 = a.in + tile_off(0, t.m0, a.L3, tile_bytes);
+            // the row's tiles are one run of sites unless it wraps
+            const bool run = t.x0 >= 1 && t.x0 + 2 < L;
             for (int zi = -1; zi <= L; ++zi) {
                 const int g = (int)(pseq % kColIn);
                 const uint32_t use = pseq / kColIn;
-                int good = 1;
-                if (lane == 0 && use > 0) good = wait_bar(empty_bar(g), (use - 1) & 1u, abort_flag) ? 1 : 0;
-                if (!__shfl_sync(0xffffffffu, good, 0)) {
-                    ok = false;
-                    break;
+                bool good = true;
+                if (leader && use > 0) good = wait_bar(empty_bar(g), (use - 1) & 1u, abort_flag);
+                ok = __all_sync(0xffffffffu, good);
+                if (!ok) break;
+                if (leader) mbar_arrive_expect_tx(full_bar(g), (16u / kProducers) * tile_bytes);
+#pragma unroll
+                for (int k = 0; k < 4 / kProducers; ++k) {
+                    const int b = part + k * kProducers;
+                    const uint8_t* row = tile0 + (int64_t)((wrap(zi, L) * L + wrap(t.y - 1 + b, L)) * L) * tile_bytes;
+                    const uint32_t dst = ring + (uint32_t)g * kColInBytes + (uint32_t)b * 4u * tile_bytes;
+                    if (run) {
+                        if (leader)
+                            bulk_load(dst, row + (int64_t)(t.x0 - 1) * tile_bytes, 4u * tile_bytes, full_bar(g));
+                    } else {
+#pragma unroll
+                        for (int i = 0; i < 4; ++i)
+                            if (leader)
+                                bulk_load(dst + (uint32_t)i * tile_bytes,
+                                          row + (int64_t)wrap(t.x0 - 1 + i, L) * tile_bytes, tile_bytes, full_bar(g));
+                    }
                 }
-                if (lane == 0) mbar_arrive_expect_tx(full_bar(g), 16u * tile_bytes);
-                __syncwarp();
-                if (kBitsIn) {
-                    // 2 KiB tiles: lane b copies row b's four contiguous tiles (8 KiB) in one run
-                    if (lane < 4)
-                        copy_row(ring + (uint32_t)g * kColInBytes + (uint32_t)lane * 4u * tile_bytes, a.in,
-                                 ((int64_t)wrap(zi, L) * L + wrap(t.y - 1 + lane, L)) * L, t.x0 - 1, 4, L, a.L3, t.m0,
-                                 tile_bytes, full_bar(g));
-                } else if (lane < 16) {
-                    bulk_load(ring + (uint32_t)g * kColInBytes + (uint32_t)lane * tile_bytes,
-                              a.in + tile_off((int64_t)wrap(zi, L) * L * L + xy, t.m0, a.L3, tile_bytes), tile_bytes,
-                              full_bar(g));
-                }
+                prefetch();
                 ++pseq;
             }
         }
         // copies still in flight land before the CTA exits
-        if (lane == 0) {
+        if (leader) {
             const uint32_t last = pseq < (uint32_t)kColIn ? pseq : (uint32_t)kColIn;
             for (uint32_t g = 0; g < last; ++g) {
                 const uint32_t q = pseq - 1 - ((pseq - 1 - g) % kColIn);
@@ -609,87 +661,101 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
             }
         }
         __syncwarp();
-    } else if (warp == kIssuerWarp) {
-        if (lane == 0) {
-            uint32_t pseq = 0;
-            int64_t qbase = 0;
-            bool ok = true;
-            constexpr uint32_t a_lbo = 2048u, a_sbo = 128u;
-            const uint64_t bdesc0 = smem_desc(wsm, 128u, 256u);   // + 32 per 512-byte block
-            constexpr uint32_t kIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTileM >> 4) << 24);
-            for (int64_t u = blockIdx.x; u < a.n_units && ok; u += gridDim.x) {
-                for (int zi = -1; zi <= L && ok; ++zi) {
-                    // output plane zi + 1 is first written by this input plane: its slot must be drained
-                    if (zi + 1 <= L - 1) {
-                        const int64_t q = qbase + zi + 1;
-                        const uint32_t v = (uint32_t)(q >> 3);
-                        if (v > 0 && !wait_bar(acce_bar((int)(q & 7)), (v - 1) & 1u, abort_flag)) {
-                            ok = false;
-                            break;
-                        }
-                        tc_fence_after();
+    } else if (warp == kIssuer) {
+        const bool leader = elect_one();
+        // The tensor pipe takes only a few MMAs ahead, so what this thread does between two planes
+        // idles it: the next plane's barriers are tested (without waiting) before the current
+        // plane's last row is issued, while the pipe still has work.
+        constexpr uint32_t a_lbo = 2048u, a_sbo = 128u;
+        const uint64_t bdesc0 = smem_desc(wsm, 128u, 256u);   // + 32 per 512-byte block
+        const uint64_t adesc_ring = smem_desc(ring, a_lbo, a_sbo);
+        constexpr uint32_t kIdescBase = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTileM >> 4) << 24);
+        constexpr ColTable kTab = make_col_table(kBitsIn);
+        const uint32_t n_planes = (uint32_t)L + 2;   // input planes of a unit, zi = -1 .. L
+        uint32_t pseq = 0, qbase = 0;                // input planes done; output planes of finished units
+        bool ok = true;
+        // barriers of a plane: its copies, and the accumulators of output plane zi + 1, first written by
+        // it, drained (use 0 of a slot needs no wait)
+        auto full_done = [&](uint32_t seq) { return mbar_test(full_bar((int)(seq % kColIn)), (seq / kColIn) & 1u); };
+        auto slot_done = [&](uint32_t q) { return q < 8 || mbar_test(acce_bar((int)(q & 7)), ((q >> 3) - 1) & 1u); };
+        bool ready = false;
+        for (int64_t u = blockIdx.x; u < a.n_units && ok; u += gridDim.x) {
+            for (uint32_t k = 0; k < n_planes; ++k) {   // zi = k - 1; writes output planes k - 2 .. k
+                if (!ready) {
+                    const uint32_t q = qbase + k;
+                    bool good = true;
+                    if (leader) {
+                        good = k >= (uint32_t)L || q < 8 ||
+                               wait_bar(acce_bar((int)(q & 7)), ((q >> 3) - 1) & 1u, abort_flag);
+                        good = good && wait_bar(full_bar((int)(pseq % kColIn)), (pseq / kColIn) & 1u, abort_flag);
                     }
-                    const int t1 = zi - 1 < 0 ? 0 : zi - 1, t2 = zi + 1 > L - 1 ? L - 1 : zi + 1;
-                    const int P1 = t1 - (zi - 1), P2 = t2 - (zi - 1);           // parts 0..2
-                    const int s1 = (int)((qbase + t1) & 7);
-                    const int wrap_at = s1 + (t2 - t1) > 7 ? t1 + (8 - s1) : -1;   // first plane in slot 0
-                    // the window of position (b, p): blocks 4 P1 .. 4 P2 + hi - lo of its sequence
-                    // into TMEM column 64 s1 + 16 lo, N = 16 (4 (P2 - P1) + hi - lo + 1)
-                    const uint64_t bdesc_plane = bdesc0 + (uint64_t)(128 * P1);
-                    const uint32_t idesc_plane = kIdescBase + ((uint32_t)(8 * (P2 - P1)) << 17);
-                    const uint32_t col_plane = tmem + (uint32_t)(s1 * kColPlaneCols);
-                    constexpr ColTable kTab = make_col_table(kBitsIn);
-                    const int g = (int)(pseq % kColIn);
-                    if (!wait_bar(full_bar(g), (pseq / kColIn) & 1u, abort_flag)) {
-                        ok = false;
-                        break;
-                    }
+                    ok = __all_sync(0xffffffffu, good);
+                    if (!ok) break;
+                }
+                tc_fence_after();
+                // parts P1 .. P2 of the windows: output planes k - 2 + P1 .. k - 2 + P2
+                const uint32_t P1 = k >= 2 ? 0u : 2u - k, P2 = k < (uint32_t)L ? 2u : (uint32_t)L + 1 - k;
+                const uint32_t s1 = (qbase + k - 2 + P1) & 7u, n = P2 - P1;
+                // the window of position (b, p): blocks 4 P1 .. 4 P2 + hi - lo of its sequence
+                // into TMEM column 64 s1 + 16 lo, N = 16 (4 (P2 - P1) + hi - lo + 1)
+                const uint64_t bdesc_plane = bdesc0 + (uint64_t)(128 * P1);
+                const uint32_t idesc_plane = kIdescBase + ((8 * n) << 17);
+                const uint32_t col_plane = tmem + s1 * kColPlaneCols;
+                const uint64_t adesc_plane = adesc_ring + (uint64_t)((pseq % kColIn) * (kColInBytes >> 4));
+                auto row_mmas = [&](int b) {
+                    const uint64_t adesc0 = adesc_plane + (uint64_t)((uint32_t)b * ((4u * tile_bytes) >> 4));
+                    if (s1 + n <= 7) {
 #pragma unroll
-                    for (int b = 0; b < 4; ++b) {
-                        const uint64_t adesc0 =
-                            smem_desc(ring + (uint32_t)g * kColInBytes + (uint32_t)b * 4u * tile_bytes, a_lbo, a_sbo);
-                        if (wrap_at < 0) {
-#pragma unroll
-                            for (int p = 0; p < P; ++p) {
-                                const ColPos pos = kTab.pos[b * P + p];
+                        for (int p = 0; p < P; ++p) {
+                            const ColPos pos = kTab.pos[b * P + p];
+                            if (leader)
                                 mma_bf16_n(col_plane + (uint32_t)(pos.lo * kC),
                                            adesc0 + (uint64_t)(p * (kSlotBytes >> 4)),
                                            bdesc_plane + (uint64_t)(32 * pos.base),
                                            idesc_plane + ((uint32_t)(2 * (pos.hi - pos.lo + 1)) << 17));
-                            }
-                        } else {
-                            // the window crosses the ring's end: split at slot 0
-                            const int Pw = wrap_at - (zi - 1);
+                        }
+                    } else {
+                        // the window crosses the ring's end: split at slot 0, part Pw
+                        const int Pw = (int)(P1 + 8 - s1);
 #pragma unroll
-                            for (int p = 0; p < P; ++p) {
-                                const ColPos pos = kTab.pos[b * P + p];
-                                const uint64_t adesc = adesc0 + (uint64_t)(p * (kSlotBytes >> 4));
-                                auto issue = [&](int pa, int ja, int pz, int jz, uint32_t col) {
-                                    // blocks (pa, ja) .. (pz, jz) of the sequence into TMEM column col
-                                    const int b0 = 4 * pa + ja - pos.lo, nb = 4 * (pz - pa) + jz - ja + 1;
+                        for (int p = 0; p < P; ++p) {
+                            const ColPos pos = kTab.pos[b * P + p];
+                            const uint64_t adesc = adesc0 + (uint64_t)(p * (kSlotBytes >> 4));
+                            auto issue = [&](int pa, int ja, int pz, int jz, uint32_t col) {
+                                // blocks (pa, ja) .. (pz, jz) of the sequence into TMEM column col
+                                const int b0 = 4 * pa + ja - pos.lo, nb = 4 * (pz - pa) + jz - ja + 1;
+                                if (leader)
                                     mma_bf16_n(tmem + col, adesc, bdesc0 + (uint64_t)(32 * (pos.base + b0)),
                                                kIdescBase | ((uint32_t)(nb * 2) << 17));
-                                };
-                                issue(P1, pos.lo, Pw - 1, 3, (uint32_t)(s1 * kColPlaneCols + pos.lo * kC));
-                                issue(Pw, 0, P2, pos.hi, 0u);
-                            }
+                            };
+                            issue((int)P1, pos.lo, Pw - 1, 3, s1 * kColPlaneCols + (uint32_t)(pos.lo * kC));
+                            issue(Pw, 0, (int)P2, pos.hi, 0u);
                         }
                     }
-                    mma_commit(empty_bar(g));
-                    ++pseq;
-                    // output plane zi - 1 has received its last contribution
-                    if (zi - 1 >= 0) mma_commit(accf_bar((int)((qbase + zi - 1) & 7)));
-                }
-                qbase += L;
+                };
+#pragma unroll
+                for (int b = 0; b < 3; ++b) row_mmas(b);
+                // the next plane (of this unit or the next): both barriers, if any, already complete?
+                const bool last = k + 1 == n_planes;
+                const uint32_t kn = last ? 0 : k + 1, qn = (last ? qbase + (uint32_t)L : qbase) + kn;
+                ready = __all_sync(0xffffffffu, full_done(pseq + 1) && (kn >= (uint32_t)L || slot_done(qn)));
+                row_mmas(3);
+                if (leader) mma_commit(empty_bar((int)(pseq % kColIn)));
+                ++pseq;
+                // output plane k - 2 has received its last contribution
+                if (leader && k >= 2) mma_commit(accf_bar((int)((qbase + k - 2) & 7u)));
             }
-            // every MMA issued has completed before TMEM is released
+            qbase += (uint32_t)L;
+        }
+        // every MMA issued has completed before TMEM is released
+        if (leader) {
             mma_commit(done_bar);
             wait_bar(done_bar, 0, abort_flag, true);
         }
         __syncwarp();
     } else {
-        // epilogue: warp w owns TMEM lanes (= tile rows = samples) 32w .. 32w + 31
-        const int r = warp * 32 + lane;
+        // epilogue: the warp owns TMEM lanes (= tile rows = samples) 32 quad .. 32 quad + 31
+        const int quad = warp & 3, r = quad * 32 + lane;
         constexpr bool kHead = tc_head(kMode);
         float bias[kC];
 #pragma unroll
@@ -715,6 +781,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
             const bool valid = sample < a.n_samples;
             for (int zo = 0; zo < L; ++zo, ++q) {
                 const int s = (int)(q & 7);
+                if ((s & 1) != warp >> 2) continue;   // the other group's plane
                 int got = 1;
                 if (lane == 0) got = wait_bar(accf_bar(s), (uint32_t)(q >> 3) & 1u, abort_flag) ? 1 : 0;
                 got = __shfl_sync(0xffffffffu, got, 0);
@@ -723,7 +790,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
                     break;
                 }
                 tc_fence_after();
-                const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(s * kColPlaneCols);
+                const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(s * kColPlaneCols);
                 uint32_t raw[4][16];
 #pragma unroll
                 for (int j = 0; j < 4; ++j) tmem_ld16(lane_base + (uint32_t)(j * kC), raw[j]);
@@ -768,8 +835,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
 #pragma unroll
                             for (int d = 0; d < 3; ++d) z[d] = fmaf(y3[c], w4[d * kC + c], z[d]);
                         }
-                        const int64_t wd = (t.m0 + warp * 32) / 64;
-                        const int hw = warp & 1;
+                        const int64_t wd = (t.m0 + quad * 32) / 64;
+                        const int hw = quad & 1;
                         if (kMode == kTcHead) {
 #pragma unroll
                             for (int d = 0; d < 3; ++d) {
@@ -835,7 +902,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_conv_col(const __grid_constan
     }
     tc_fence_before();
     __syncthreads();
-    if (warp == kIssuerWarp) {
+    if (warp == kIssuer) {
         tc_fence_after();
         tmem_dealloc(tmem, kTmemCols);
     }
@@ -1136,7 +1203,7 @@ t3d_status launch_conv_col(const TcArgs& a, cudaStream_t st)
 {
     const int grid = (int)std::min<int64_t>(a.n_units, sm_count());
     ProfScope prof(T3D_K_CNN, st);
-    k_conv_col<kMode, kBitsIn><<<grid, kTcThreads, kColSmemBytes, st>>>(a);
+    k_conv_col<kMode, kBitsIn><<<grid, kConvThreads, kColSmemBytes, st>>>(a);
     T3D_LAUNCH_CHECK("tensor-core convolution");
     return T3D_OK;
 }
