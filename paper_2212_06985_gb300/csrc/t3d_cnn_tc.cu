@@ -351,6 +351,12 @@ __device__ __forceinline__ void tmem_wait_ld()
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 }
 
+// Four floats of shared memory (volatile: loaded where they are used, not kept in registers).
+__device__ __forceinline__ void lds4(uint32_t addr, float (&v)[4])
+{
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(addr));
+}
+
 __device__ __forceinline__ uint32_t pack2(float lo, float hi)
 {
     __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
@@ -410,7 +416,9 @@ constexpr int kColOffBar = kColOffW + kColWBlocks * 512;
 constexpr int kColNumBars = 2 * kColInMax + 2 * kColSlots + 1;   // full, empty, acc_full, acc_empty, done
 constexpr int kColOffMisc = kColOffBar + kColNumBars * 8;
 constexpr int kColOffPos = kColOffMisc + 16;              // ColPos[16]
-constexpr int kColSmemBytes = kColOffPos + 16 * 12 + 1024;
+constexpr int kColOffHead = kColOffPos + 16 * 12 + 8;     // training's head: w4 [3][16], bias [16]
+constexpr int kColSmemBytes = kColOffHead + 4 * kC * 4 + 1024;
+static_assert(kColOffHead % 16 == 0, "16-byte loads");
 static_assert(kColSmemBytes <= 227 * 1024, "shared memory budget");
 static_assert(kColSlots * kColPlaneCols == 512, "TMEM ring");
 
@@ -499,14 +507,19 @@ __device__ __forceinline__ Unit col_unit_of(const TcArgs& a, int64_t u)
 // writes no activations); the MMAs of a plane take 1344 of its 2380 cycles.
 constexpr int kConvProducers = 2;
 constexpr int kConvEpi = 8;
-constexpr int kConvThreads = 32 * (kConvEpi + kConvProducers + 1);
+// Training's head has a heavier epilogue (an exponential, a logarithm, a division and about 300 FMAs a
+// site and sample, 52 running sums a thread) and takes three groups, its weights from shared memory and
+// a plane one site at a time; labels, and the backward pass's gating activations, are requested before
+// the wait for the accumulators.  L = 12, 2,048 samples: head 199 -> 108 us, backward data 88 -> 72.
+__host__ __device__ constexpr int conv_epi(int mode) { return mode == kTcHeadTrain ? 12 : kConvEpi; }
+__host__ __device__ constexpr int conv_threads(int mode) { return 32 * (conv_epi(mode) + kConvProducers + 1); }
 constexpr int kAhead = 2;   // planes between the L2 prefetch and the copy
 
 template <int kMode, bool kBitsIn>
-__global__ void __launch_bounds__(kConvThreads, 1) k_conv_col(const __grid_constant__ TcArgs a)
+__global__ void __launch_bounds__(conv_threads(kMode), 1) k_conv_col(const __grid_constant__ TcArgs a)
 {
     constexpr int kProducers = kConvProducers;
-    constexpr int kFirstProducer = kConvEpi, kIssuer = kConvEpi + kProducers;
+    constexpr int kEpi = conv_epi(kMode), kFirstProducer = kEpi, kIssuer = kEpi + kProducers;
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     const uint32_t ring = smem_u32(sm);
@@ -577,15 +590,18 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_col(const __grid_const
         misc[1] = 0;
         fence_mbar_init();
     }
+    if (kMode == kTcHeadTrain && threadIdx.x < 4 * kC)
+        reinterpret_cast<float*>(sm + kColOffHead)[threadIdx.x] =
+            threadIdx.x < 3 * kC ? a.w4[threadIdx.x] : a.bias[threadIdx.x - 3 * kC];
     if (warp == kIssuer) tmem_alloc(smem_u32(misc), kTmemCols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, misc[0], 0);
     // every accumulator starts at zero (the epilogue re-zeroes a plane after draining it)
-    if (warp < kConvEpi) {
+    if (warp < kEpi) {
 #pragma unroll 4
-        for (int c = 16 * (warp >> 2); c < kColSlots * kColPlaneCols; c += 32)
+        for (int c = 16 * (warp >> 2); c < kColSlots * kColPlaneCols; c += 4 * kEpi)
             tmem_zero16(tmem + ((uint32_t)((warp & 3) * 32) << 16) + c);
         tmem_wait_st();
     }
@@ -762,14 +778,18 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_col(const __grid_const
         // epilogue: the warp owns TMEM lanes (= tile rows = samples) 32 quad .. 32 quad + 31
         const int quad = warp & 3, r = quad * 32 + lane;
         constexpr bool kHead = tc_head(kMode);
+        // training's head keeps its weights in shared memory and takes a plane a site at a time: the sums
+        // need the registers
+        constexpr bool kLean = kMode == kTcHeadTrain;
+        const uint32_t head = smem_u32(sm) + kColOffHead;   // w4 [3][16], bias [16]
         float bias[kC];
 #pragma unroll
-        for (int c = 0; c < kC; ++c) bias[c] = kMode == kTcMask ? 0.0f : a.bias[c];
-        float w4[kHead ? 3 * kC : 1];
+        for (int c = 0; c < kC; ++c) bias[c] = kMode == kTcMask || kLean ? 0.0f : a.bias[c];
+        float w4[kHead && !kLean ? 3 * kC : 1];
         float b4[3] = {0.0f, 0.0f, 0.0f};
         if (kHead) {
 #pragma unroll
-            for (int i = 0; i < 3 * kC; ++i) w4[i] = a.w4[i];
+            for (int i = 0; i < 3 * kC && !kLean; ++i) w4[i] = a.w4[i];
 #pragma unroll
             for (int d = 0; d < 3; ++d) b4[d] = a.b4[d];
         }
@@ -784,9 +804,29 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_col(const __grid_const
             const Unit t = col_unit_of(a, u);
             const int64_t sample = t.m0 + r;
             const bool valid = sample < a.n_samples;
+            const int64_t wd = (t.m0 + quad * 32) / 64;   // the warp's word, its half hw
+            const int hw = quad & 1;
             for (int zo = 0; zo < L; ++zo, ++q) {
                 const int s = (int)(q & 7);
-                if ((s & 1) != warp >> 2) continue;   // the other group's plane
+                if ((int)((uint32_t)q % (kEpi / 4)) != warp >> 2) continue;   // another group's plane
+                // what the epilogue reads of the plane beside the accumulators, requested before the wait
+                uint4 mask[kMode == kTcMask ? 4 : 1][2];
+                uint64_t labels = 0;   // lane 4 d + j: edge d's label word of site j
+                if (kMode == kTcMask) {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int xo = t.x0 + (j & 1), yo = t.y + (j >> 1);
+                        if (xo >= L || yo >= L) continue;
+                        const uint8_t* p = a.mask_act +
+                                           tile_off(((int64_t)zo * L + yo) * L + xo, t.m0, a.L3, 4096) + r * 16;
+                        mask[kMode == kTcMask ? j : 0][0] = *reinterpret_cast<const uint4*>(p);
+                        mask[kMode == kTcMask ? j : 0][1] = *reinterpret_cast<const uint4*>(p + 2048);
+                    }
+                } else if (kMode == kTcHeadTrain) {
+                    const int xo = t.x0 + (lane & 1), yo = t.y + (lane >> 1 & 1);
+                    if (lane < 12 && xo < L && yo < L && wd < a.words)
+                        labels = a.label[((int64_t)(lane >> 2) * a.L3 + ((int64_t)zo * L + yo) * L + xo) * a.W + wd];
+                }
                 int got = 1;
                 if (lane == 0) got = wait_bar(accf_bar(s), (uint32_t)(q >> 3) & 1u, abort_flag) ? 1 : 0;
                 got = __shfl_sync(0xffffffffu, got, 0);
@@ -796,21 +836,28 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_col(const __grid_const
                 }
                 tc_fence_after();
                 const uint32_t lane_base = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(s * kColPlaneCols);
-                uint32_t raw[4][16];
+                uint32_t raw[kLean ? 1 : 4][16];
+                if (!kLean) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) tmem_ld16(lane_base + (uint32_t)(j * kC), raw[j]);
-                tmem_wait_ld();
+                    for (int j = 0; j < 4; ++j) tmem_ld16(lane_base + (uint32_t)(j * kC), raw[kLean ? 0 : j]);
+                    tmem_wait_ld();
 #pragma unroll
-                for (int j = 0; j < 4; ++j) tmem_zero16(lane_base + (uint32_t)(j * kC));
-#pragma unroll
+                    for (int j = 0; j < 4; ++j) tmem_zero16(lane_base + (uint32_t)(j * kC));
+                }
+#pragma unroll (kLean ? 1 : 4)
                 for (int j = 0; j < 4; ++j) {
+                    if (kLean) {
+                        tmem_ld16(lane_base + (uint32_t)(j * kC), raw[0]);
+                        tmem_wait_ld();
+                        tmem_zero16(lane_base + (uint32_t)(j * kC));
+                    }
                     const int xo = t.x0 + (j & 1), yo = t.y + (j >> 1);
                     if (xo >= L || yo >= L) continue;   // the odd lattice's last column
                     const int64_t site = ((int64_t)zo * L + yo) * L + xo;
                     const int64_t row_off = tile_off(site, t.m0, a.L3, 4096) + r * 16;
                     float v[16];
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) v[c] = __uint_as_float(raw[j][c]);
+                    for (int c = 0; c < 16; ++c) v[c] = __uint_as_float(raw[kLean ? 0 : j][c]);
                     if (kMode == kTcRelu || kMode == kTcMask) {
                         uint32_t pk[8];
                         if (kMode == kTcRelu) {
@@ -820,8 +867,7 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_col(const __grid_const
                         } else {
                             // the gradient passes where the forward activation (a ReLU output,
                             // so never negative) is non-zero
-                            const uint4 m0v = *reinterpret_cast<const uint4*>(a.mask_act + row_off);
-                            const uint4 m1v = *reinterpret_cast<const uint4*>(a.mask_act + row_off + 2048);
+                            const uint4 m0v = mask[kMode == kTcMask ? j : 0][0], m1v = mask[kMode == kTcMask ? j : 0][1];
                             const uint32_t mw[8] = {m0v.x, m0v.y, m0v.z, m0v.w, m1v.x, m1v.y, m1v.z, m1v.w};
 #pragma unroll
                             for (int c = 0; c < kC; c += 2)
@@ -835,13 +881,24 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_col(const __grid_const
                         float y3[kC];
                         float z[3] = {b4[0], b4[1], b4[2]};
 #pragma unroll
-                        for (int c = 0; c < kC; ++c) {
-                            y3[c] = fmaxf(v[c] + bias[c], 0.0f);
+                        for (int c4 = 0; c4 < kC; c4 += 4) {
+                            float bw[4][4];   // the three heads' weights and the bias of channels c4 .. c4 + 3
 #pragma unroll
-                            for (int d = 0; d < 3; ++d) z[d] = fmaf(y3[c], w4[d * kC + c], z[d]);
+                            for (int d = 0; d < 4; ++d) {
+                                if (kLean) {
+                                    lds4(head + (uint32_t)(d * kC + c4) * 4u, bw[d]);
+                                } else {
+#pragma unroll
+                                    for (int c = 0; c < 4; ++c) bw[d][c] = d < 3 ? w4[kLean ? 0 : d * kC + c4 + c] : bias[c4 + c];
+                                }
+                            }
+#pragma unroll
+                            for (int c = 0; c < 4; ++c) {
+                                y3[c4 + c] = fmaxf(v[c4 + c] + bw[3][c], 0.0f);
+#pragma unroll
+                                for (int d = 0; d < 3; ++d) z[d] = fmaf(y3[c4 + c], bw[d][c], z[d]);
+                            }
                         }
-                        const int64_t wd = (t.m0 + quad * 32) / 64;
-                        const int hw = quad & 1;
                         if (kMode == kTcHead) {
 #pragma unroll
                             for (int d = 0; d < 3; ++d) {
@@ -856,28 +913,31 @@ __global__ void __launch_bounds__(kConvThreads, 1) k_conv_col(const __grid_const
                             float dz[3];
 #pragma unroll
                             for (int d = 0; d < 3; ++d) {
-                                const uint64_t lw = wd < a.words ? a.label[((int64_t)d * a.L3 + site) * a.W + wd] : 0ull;
+                                const uint64_t lw = __shfl_sync(0xffffffffu, labels, 4 * d + j);
                                 const float yv = (float)((uint32_t)(lw >> (32 * hw + lane)) & 1u);
-                                const float sig = 1.0f / (1.0f + expf(-z[d]));
+                                const float ez = expf(-fabsf(z[d])), sig = (z[d] < 0.0f ? ez : 1.0f) / (1.0f + ez);
                                 dz[d] = valid ? (sig - yv) * a.inv_n : 0.0f;
-                                if (valid) acc[3 * kC + 3] += fmaxf(z[d], 0.0f) - z[d] * yv + log1pf(expf(-fabsf(z[d])));
+                                if (valid) acc[3 * kC + 3] += fmaxf(z[d], 0.0f) - z[d] * yv + log1pf(ez);
                                 acc[3 * kC + d] += dz[d];
                             }
                             uint32_t pk[8];
 #pragma unroll
-                            for (int c = 0; c < kC; c += 2) {
-                                float g2[2];
+                            for (int c4 = 0; c4 < kC; c4 += 4) {
+                                float g4[4], hw4[3][4];
 #pragma unroll
-                                for (int h = 0; h < 2; ++h) {
+                                for (int d = 0; d < 3; ++d) lds4(head + (uint32_t)(d * kC + c4) * 4u, hw4[d]);
+#pragma unroll
+                                for (int h = 0; h < 4; ++h) {
                                     float dy = 0.0f;
 #pragma unroll
                                     for (int d = 0; d < 3; ++d) {
-                                        dy = fmaf(dz[d], w4[d * kC + c + h], dy);
-                                        acc[d * kC + c + h] = fmaf(y3[c + h], dz[d], acc[d * kC + c + h]);
+                                        dy = fmaf(dz[d], hw4[d][h], dy);
+                                        acc[d * kC + c4 + h] = fmaf(y3[c4 + h], dz[d], acc[d * kC + c4 + h]);
                                     }
-                                    g2[h] = y3[c + h] > 0.0f ? dy : 0.0f;
+                                    g4[h] = y3[c4 + h] > 0.0f ? dy : 0.0f;
                                 }
-                                pk[c / 2] = pack2(g2[0], g2[1]);
+                                pk[c4 / 2] = pack2(g4[0], g4[1]);
+                                pk[c4 / 2 + 1] = pack2(g4[2], g4[3]);
                             }
                             uint8_t* dst = a.out + row_off;
                             *reinterpret_cast<uint4*>(dst) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
@@ -1208,7 +1268,7 @@ t3d_status launch_conv_col(const TcArgs& a, cudaStream_t st)
 {
     const int grid = (int)std::min<int64_t>(a.n_units, sm_count());
     ProfScope prof(T3D_K_CNN, st);
-    k_conv_col<kMode, kBitsIn><<<grid, kConvThreads, kColSmemBytes, st>>>(a);
+    k_conv_col<kMode, kBitsIn><<<grid, conv_threads(kMode), kColSmemBytes, st>>>(a);
     T3D_LAUNCH_CHECK("tensor-core convolution");
     return T3D_OK;
 }
