@@ -625,6 +625,146 @@ k_logical(const __grid_constant__ ItemTable tab)
     });
 }
 
+// The readout of few words: a block takes a tile of kWords words and all three axes at once, 256 threads
+// each (thread = line row x word), so a batch that fills the chip at most once waits for one axis' loads
+// and additions instead of three.  A warp's counters are added by shuffles and the warps' in shared
+// memory, up to the highest bit that L^2 has, and an outcome's samples are counted by population counts.
+// Bound by the latency of a line's loads and of the additions.  Per call, before -> now: L = 8, 4,096
+// samples 15 -> 8 us; L = 24, 16,384 121 -> 40; L = 32, 70,000 296 -> 203; L = 48, 20,000 878 -> 467.
+constexpr int kLogThreads = 3 * 256;
+constexpr int kLogWave = 152;   // blocks that fill the chip: one per SM
+
+// c += bit, counters of nb bits
+__device__ __forceinline__ void counter_add_bit(uint64_t (&c)[kCountBits], uint64_t bit, int nb)
+{
+#pragma unroll
+    for (int b = 0; b < kCountBits; ++b) {
+        if (b >= nb) break;
+        uint64_t carry = c[b] & bit;
+        c[b] ^= bit;
+        bit = carry;
+    }
+}
+
+// c += the counters of the lane delta apart (every lane of the warp)
+__device__ __forceinline__ void counter_add_lane(uint64_t (&c)[kCountBits], int delta, int nb)
+{
+    uint64_t carry = 0;
+#pragma unroll
+    for (int b = 0; b < kCountBits; ++b) {
+        if (b >= nb) break;
+        const uint64_t x = c[b], y = __shfl_xor_sync(0xffffffffu, x, delta);
+        c[b] = x ^ y ^ carry;
+        carry = (x & y) | (carry & (x ^ y));
+    }
+}
+
+template <int kWords>
+__global__ void __launch_bounds__(kLogThreads)
+k_logical_axes(const __grid_constant__ ItemTable tab)
+{
+    constexpr int kRows = 256 / kWords;   // line rows of an axis
+    constexpr int kWarps = 8;             // warps of an axis
+    __shared__ uint64_t part[3][kWarps][kCountBits][kWords];
+    __shared__ uint64_t fail[3][kWords];
+    const int dd = threadIdx.x >> 8, lane = threadIdx.x & 31, warp = (threadIdx.x >> 5) & 7;
+    const int tx = threadIdx.x % kWords, ty = (threadIdx.x & 255) / kWords;
+    // block-uniform loop: every thread reaches every barrier
+    for_each_item_block(tab, [&](const ItemDesc& d, int64_t lb) {
+        const Lattice lat = d.lat;
+        const int64_t W = d.W;
+        const int L = lat.L, L2 = lat.L2;
+        const int nb = 32 - __clz(L2);
+        uint64_t cnt[kCountBits];
+#pragma unroll
+        for (int b = 0; b < kCountBits; ++b) cnt[b] = 0;
+        {
+            const int64_t w = lb * kWords + tx;
+            const int u_axis = (dd == 0) ? 1 : 0;
+            const int v_axis = (dd == 2) ? 1 : 2;
+            if (w < W) {
+                // step between consecutive sites of a line along axis dd
+                const int64_t step = (dd == 0 ? 1 : (dd == 1 ? L : L2)) * W;
+                for (int line = ty; line < L2; line += kRows) {
+                    Coord r;
+                    r.x[u_axis] = line % L;
+                    r.x[v_axis] = line / L;
+                    r.x[dd] = 0;
+                    const uint64_t* __restrict__ p = d.e + ((int64_t)dd * lat.L3 + site_index(lat, r)) * W + w;
+                    uint64_t par = 0;
+#pragma unroll 8
+                    for (int t = 0; t < L; ++t) par ^= __ldcs(p + t * step);
+                    counter_add_bit(cnt, par, nb);
+                }
+            }
+        }
+#pragma unroll
+        for (int delta = 16; delta >= kWords; delta >>= 1) counter_add_lane(cnt, delta, nb);
+        if (lane < kWords) {
+#pragma unroll
+            for (int b = 0; b < kCountBits; ++b) part[dd][warp][b][lane] = cnt[b];
+        }
+        __syncthreads();
+        if (warp == 0) {
+            // lane = one of the kWarps partial counts x word; with more than 32 of them a lane takes several
+            constexpr int kLanes = 32 / kWords < kWarps ? 32 / kWords : kWarps;
+            const int lr = lane / kWords;
+#pragma unroll
+            for (int b = 0; b < kCountBits; ++b) cnt[b] = lr < kLanes ? part[dd][lr % kWarps][b][tx] : 0;
+#pragma unroll
+            for (int i = kLanes; i < kWarps; i += kLanes) {
+                uint64_t carry = 0;
+#pragma unroll
+                for (int b = 0; b < kCountBits; ++b) {
+                    const uint64_t x = cnt[b], y = part[dd][i + lr][b][tx];
+                    cnt[b] = x ^ y ^ carry;
+                    carry = (x & y) | (carry & (x ^ y));
+                }
+            }
+#pragma unroll
+            for (int delta = kWords * kLanes / 2; delta >= kWords; delta >>= 1) counter_add_lane(cnt, delta, nb);
+            // samples with count >= ceil(L^2 / 2)
+            const unsigned need = (unsigned)(L2 + 1) / 2;
+            uint64_t gt = 0, eq = ~0ULL;
+#pragma unroll
+            for (int b = kCountBits - 1; b >= 0; --b) {
+                if ((need >> b) & 1u) {
+                    eq &= cnt[b];
+                } else {
+                    gt |= eq & cnt[b];
+                    eq &= ~cnt[b];
+                }
+            }
+            if (lane < kWords) fail[dd][lane] = gt | eq;
+        }
+        __syncthreads();
+        if (d.mask) {
+            for (int i = threadIdx.x; i < 64 * kWords; i += kLogThreads) {
+                const int x = i >> 6, j = i & 63;
+                const int64_t sample = (lb * kWords + x) * 64 + j;
+                if (sample < d.n_samples)
+                    d.mask[sample] = (uint8_t)(((fail[0][x] >> j) & 1ULL) | (((fail[1][x] >> j) & 1ULL) << 1) |
+                                               (((fail[2][x] >> j) & 1ULL) << 2));
+            }
+        }
+        if (d.counts8 && threadIdx.x < 64) {
+            // thread = word x outcome; then the words of a warp
+            const int x = threadIdx.x >> 3, m = threadIdx.x & 7;
+            int n = 0;
+            if (x < kWords) {
+                const int64_t left = d.n_samples - (lb * kWords + x) * 64;
+                uint64_t hit = left >= 64 ? ~0ULL : (left > 0 ? (1ULL << left) - 1 : 0);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) hit &= ((m >> k) & 1) ? fail[k][x] : ~fail[k][x];
+                n = __popcll(hit);
+            }
+            n += __shfl_xor_sync(0xffffffffu, n, 8);
+            n += __shfl_xor_sync(0xffffffffu, n, 16);
+            if (lane < 8 && n) atomicAdd(&d.counts8[m], (unsigned long long)n);
+        }
+    });
+}
+
 // Fallback gate: flag every word in which some sample's syndrome has more
 // than max_weight unsatisfied checks.  Two passes.  k_gate_count: block
 // (32, 8) over a 32-word tile and one of Y face ranges (blockIdx.y);
@@ -1024,16 +1164,26 @@ t3d_status launch_flip_until_clear(ItemTable& all, int max_sweeps, int32_t* swee
 
 t3d_status launch_logical(ItemTable& tab, cudaStream_t st)
 {
+    // One block per SM of k_logical_axes with the widest tiles that still make a wave's worth of blocks
+    // (L = 16, 20,000 samples: 32, 21 and 25 us with two, four and eight words; L = 16, 70,000: 65, 43
+    // and 33); more words than one wave of eight go to k_logical, whose blocks share an SM (L = 32,
+    // 100,000 samples: 320 us against 390).
+    int64_t words = 0;
+    for (int i = 0; i < tab.n; ++i) words += tab.it[i].W;
+    const bool serial = words > 8 * kLogWave;
+    const int tile = serial ? kLogWords : (words > 4 * kLogWave ? 8 : (words > 2 * kLogWave ? 4 : 2));
     for (int i = 0; i < tab.n; ++i) {
         ItemDesc& d = tab.it[i];
-        d.blocks = (d.W + kLogWords - 1) / kLogWords;
+        d.blocks = (d.W + tile - 1) / tile;
         if (d.counts8) T3D_CUDA_CHECK(cudaMemsetAsync(d.counts8, 0, 8 * sizeof(int64_t), st));
     }
     finish_table(tab);
     ProfScope prof(T3D_K_LOGICAL, st);
-    k_logical<<<persistent_grid((const void*)k_logical, kLogWords * kLogSplit, T3D_K_LOGICAL, tab.prefix[tab.n],
-                                has_live(tab)),
-                kLogWords * kLogSplit, 0, st>>>(tab);
+    const auto kernel = serial ? k_logical
+                               : (tile == 8 ? k_logical_axes<8> : (tile == 4 ? k_logical_axes<4> : k_logical_axes<2>));
+    const int threads = serial ? kLogWords * kLogSplit : kLogThreads;
+    kernel<<<persistent_grid((const void*)kernel, threads, T3D_K_LOGICAL, tab.prefix[tab.n], has_live(tab)), threads, 0,
+             st>>>(tab);
     T3D_LAUNCH_CHECK("logical");
     return T3D_OK;
 }
