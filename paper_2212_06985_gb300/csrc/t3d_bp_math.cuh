@@ -138,7 +138,7 @@ __device__ __forceinline__ TD2 td2_of(float2 x)
     h = __ffma2_rn(a, h, f2(-0.5f));
     h = __ffma2_rn(a, h, f2(1.0f));
     const float2 ah = __fmul2_rn(a, h);
-    const float2 ome = __fadd2_rn(f2(1.0f), make_float2(-E.x, -E.y));
+    const float2 ome = __ffma2_rn(E, f2(-1.0f), f2(1.0f));
     const float2 om = make_float2(a.x < 0.1f ? ah.x : ome.x, a.y < 0.1f ? ah.y : ome.y);
     return TD2{__fmul2_rn(om, r), __fmul2_rn(__fadd2_rn(E, E), r)};
 }
@@ -160,13 +160,19 @@ template <int K>
 __device__ __forceinline__ void check_node2(const float2 (&x)[K], bool syn0, bool syn1, float2 (&out)[K])
 {
     TD2 v[K], suf[K];
-    uint32_t sa0 = syn0 ? 0x80000000u : 0u, sa1 = syn1 ? 0x80000000u : 0u;
+    // the inputs' sign bits, packed (input i at bit K - 1 - i): the inputs themselves need not stay in
+    // registers, which for K = 7 spilled.  (The toric code's four inputs fit either way, and t3d_bp.cu
+    // keeps them: with packed signs its iteration takes 2.7% longer.)
+    uint32_t sg0 = 0, sg1 = 0;
 #pragma unroll
     for (int i = 0; i < K; ++i) {
         v[i] = td2_of(x[i]);
-        sa0 ^= __float_as_uint(x[i].x);
-        sa1 ^= __float_as_uint(x[i].y);
+        sg0 = __funnelshift_l(__float_as_uint(x[i].x), sg0, 1);
+        sg1 = __funnelshift_l(__float_as_uint(x[i].y), sg1, 1);
     }
+    // an output's sign: the parity of the other inputs' and the syndrome
+    const uint32_t all0 = ((uint32_t)__popc(sg0) + (syn0 ? 1u : 0u)) << 31;
+    const uint32_t all1 = ((uint32_t)__popc(sg1) + (syn1 ? 1u : 0u)) << 31;
     if constexpr (K >= 2) suf[K - 2] = v[K - 1];
 #pragma unroll
     for (int i = K - 3; i >= 0; --i) suf[i] = td2_mul(v[i + 1], suf[i + 1]);
@@ -181,8 +187,8 @@ __device__ __forceinline__ void check_node2(const float2 (&x)[K], bool syn0, boo
         if (i > 0 && i < K - 1) pre = td2_mul(pre, v[i]);
         const float2 a = two_atanh2(o.t, o.d);
         const float m0 = fminf(a.x, kCheckClamp), m1 = fminf(a.y, kCheckClamp);
-        const uint32_t g0 = (sa0 ^ __float_as_uint(x[i].x)) & 0x80000000u;
-        const uint32_t g1 = (sa1 ^ __float_as_uint(x[i].y)) & 0x80000000u;
+        const uint32_t g0 = (all0 ^ (sg0 << (32 - K + i))) & 0x80000000u;
+        const uint32_t g1 = (all1 ^ (sg1 << (32 - K + i))) & 0x80000000u;
         out[i] = make_float2(__uint_as_float(__float_as_uint(m0) | g0), __uint_as_float(__float_as_uint(m1) | g1));
     }
 }

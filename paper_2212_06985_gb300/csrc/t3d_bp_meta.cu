@@ -67,12 +67,13 @@ struct Args {
 // Each message is read from HBM once and written once, 56 bytes per edge and sample; the earlier
 // three kernels (edge totals, faces, cubes) wrote and read the totals as well and read the face
 // and cube messages twice, 104 bytes.  kFirst: every message in is zero and nothing is read.
-// A block takes four words of one site (1 KB runs of a row).  Bound by the latency of those loads at
-// 20 warps per SM (96 registers; DRAM at 61% of its peak, issue 55%).  At L = 18, 1,536 samples
-// one iteration takes 0.29 ms against 0.37 for the three kernels, 12 iterations with the decision
-// 4.88 -> 3.49 ms (four sites and one word per block 3.70, 256 threads 3.81, six blocks per SM 4.00).
+// A block takes four words of one site (1 KB runs of a row).  Bound by the latency of those loads, so by
+// the warps in flight: 28 per SM (72 registers) since the check nodes pack their inputs' signs.  At
+// L = 18, 1,536 samples 12 iterations with the decision took 4.88 ms with the three kernels, 3.57 at 20
+// warps (DRAM at 61% of its peak, issue 55%), 3.49 at 24 and 3.43 now (four sites and one word per block
+// 3.70 against 3.49 of that time, 256 threads 3.81).
 template <bool kFirst>
-__global__ void __launch_bounds__(kThreads, 5) k_iteration(const __grid_constant__ Args a)
+__global__ void __launch_bounds__(kThreads, 7) k_iteration(const __grid_constant__ Args a)
 {
     const Lattice lat = a.lat;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -100,7 +101,7 @@ __global__ void __launch_bounds__(kThreads, 5) k_iteration(const __grid_constant
     // message of face (n, q) to its edge j
     auto F = [&](int n, int q, int j) { return row(a.in.F, (n * L3 + q) * 4 + j); };
     auto add = [](float2 u, float2 v) { return __fadd2_rn(u, v); };
-    auto sub = [](float2 u, float2 v) { return __fadd2_rn(u, make_float2(-v.x, -v.y)); };
+    auto sub = [](float2 u, float2 v) { return __ffma2_rn(v, make_float2(-1.0f, -1.0f), u); };
     const float2 l0 = make_float2(a.l0, a.l0), lq = make_float2(a.lq, a.lq);
     auto sum4 = [&](float2 m0, float2 m1, float2 m2, float2 m3) { return add(add(add(add(l0, m0), m1), m2), m3); };
     auto word = [&](int f) { return a.s[(int64_t)f * a.W + w]; };

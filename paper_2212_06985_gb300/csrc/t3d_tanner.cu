@@ -276,9 +276,11 @@ __global__ void __launch_bounds__(kThreads, 3) k_tg_checks(const BpArgs a)
 // is only kIterWords words wide at a time.  kFirst: every message in is zero and nothing is read.
 // Bound by issue (64%) and by L2, which keeps half of the repeated reads: 2,000 samples of the
 // hypergraph product with 200 classical bits (210,000 Tanner edges), 20 iterations with the
-// decision 23.4 -> 20.7 ms, 80 bits 3.92 -> 3.37, 300 samples of 120 bits 1.63 -> 1.44 (a few
-// spilled registers included; 24 warps per SM without any 21.7 / 3.30 / 1.45, and with the index
-// lists followed in the kernel instead of k_tg_lists 25.2 / 3.69 / 1.62).
+// decision 23.4 -> 20.7 ms, 80 bits 3.92 -> 3.37, 300 samples of 120 bits 1.63 -> 1.44 (24 warps per SM
+// 21.7 / 3.30 / 1.45, and with the index lists followed in the kernel instead of k_tg_lists
+// 25.2 / 3.69 / 1.62); with the check nodes' signs packed 16 bytes of registers spill at 32 warps
+// instead of 272, the first of these with its noise, gate and readout 21.0 -> 19.9 ms (56 registers and
+// 36 warps: 20.2).
 constexpr int kIterChecks = 1, kIterWords = 2, kIterThreads = 32 * kIterChecks * kIterWords;
 constexpr int kIterCheckDeg = 8, kIterVarDeg = 4;
 
@@ -311,7 +313,7 @@ __device__ __forceinline__ void check_word(const BpArgs& a, int32_t t0, float pr
                 if (e[j] >= 0) T = sum;
                 if (e[j] == t0 + k) own = m[j];
             }
-            T = __fadd2_rn(T, make_float2(-own.x, -own.y));
+            T = __ffma2_rn(own, make_float2(-1.0f, -1.0f), T);
         }
         x[k] = T;
     }
