@@ -14,9 +14,10 @@
 // shared reads, again the z-neighbour's kept in registers).  Each edge is decided once, where
 // the one-pass kernel for larger lattices decides nine edges per site.
 //
-// Thread (xy, word) of z-part zp walks the sites z0 <= z < z1 of one lattice column, so its x
-// and y neighbour offsets are fixed for the whole kernel, and a column of random words shares
-// the generator's first rounds (PhiloxColumn).
+// Up to L = 10 a thread has one site and keeps its words in registers (k_column_one).  Above, thread
+// (xy, word) of z-part zp walks the sites z0 <= z < z1 of one lattice column, so its x and y neighbour
+// offsets are fixed for the whole kernel, and a column of random words shares the generator's first
+// rounds (PhiloxColumn).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -246,6 +247,163 @@ k_column(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgr
             for (int z = zb, i = zb * P + u; z < ze; ++z, i += P)
 #pragma unroll
                 for (int k = 0; k < 3; ++k) e.at(k * L3 + z * L2 + xy) = E0[k * N + i];
+        }
+        __syncthreads();   // the next column overwrites the words
+    }
+}
+
+// k_column for lattices with at most one site per thread (L <= 10): the site's syndrome, errors and flips
+// stay in the thread's registers, and shared memory holds only what neighbours read.  A few columns are a
+// chain of dependent applications, whose length halves without the loops and the words' way through
+// shared memory; many are bound by the ALUs, which have less to do.  T = 4 cycles with the readout, z-parts
+// of several sites -> this: L = 4, 10,000 samples, 32 flips a cycle 100 -> 61 us; FFPFF at L = 6, 300,000
+// 822 -> 619 us; L = 8, 10^6 4.41 -> 4.24 ms; L = 10, 300,000 3.72 -> 3.52 ms.
+template <bool kRun>
+__global__ void __launch_bounds__(kColumnThreads, 1)
+k_column_one(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgram pr)
+{
+    extern __shared__ uint64_t sm[];
+    const int L = d.lat.L, L2 = d.lat.L2, L3 = d.lat.L3, Wt = d.tx;
+    const int P = L2 * Wt, N = L3 * Wt;   // a z-plane, the lattice
+    uint64_t* const S0 = sm;
+    uint64_t* const F0 = sm + 3 * N;
+    uint64_t* const E0 = sm + 6 * N;
+
+    const int i = threadIdx.x;            // the site's place: word fastest, then x, y, z
+    const int z = i / P, u = i - z * P, wl = u % Wt, xy = u / Wt;
+    const int y = xy / L, x = xy - y * L, site = z * L2 + xy;
+    const int xm = i + (x == 0 ? L - 1 : -1) * Wt, xp = i + (x + 1 == L ? 1 - L : 1) * Wt;
+    const int ym = i + (y == 0 ? L - 1 : -1) * L * Wt, yp = i + (y + 1 == L ? 1 - L : 1) * L * Wt;
+    const int zm = i + (z == 0 ? L - 1 : -1) * P, zp = i + (z + 1 == L ? 1 - L : 1) * P;
+
+    const int64_t words = d.nw ? d.nw : d.W;
+    const int64_t have = d.live ? min(words, *d.live - d.w0) : words;
+    for (int64_t w0 = (int64_t)blockIdx.x * Wt; w0 < have; w0 += (int64_t)gridDim.x * Wt) {
+        const int64_t w = w0 + wl;
+        const bool on = i < N && w < have;
+        const uint64_t group = on ? word_group(d, w) : 0;
+        const Rows eg{d.e + w, d.W}, sg{d.s + w, d.W};
+        uint64_t s[3] = {0, 0, 0}, e[3] = {0, 0, 0};   // the site's faces and edges
+
+        // one application; returns whether this thread's faces keep an unsatisfied check
+        auto apply = [&](bool prob, uint32_t cycle, uint32_t sweep) -> uint64_t {
+            uint64_t f[3] = {0, 0, 0};
+            if (on) {
+                const uint64_t s2y = S0[2 * N + ym], s2x = S0[2 * N + xm], s1x = S0[N + xm], s0y = S0[ym],
+                               s0z = S0[zm], s1z = S0[N + zm];
+                f[0] = at_least_three(s[2], s2y, s[1], s1z);
+                f[1] = at_least_three(s[2], s2x, s[0], s0z);
+                f[2] = at_least_three(s[1], s1x, s[0], s0y);
+                if (prob) {
+                    const PhiloxColumn pc = philox_column(pr.seed, kStreamCoin, cycle, sweep, group);
+                    const PhiloxSite ps = philox_site(pc, (uint32_t)site);
+                    const U32x4 a = philox_finish(pc, ps, philox_block(pc, 0));
+                    const U32x4 b = philox_finish(pc, ps, philox_block(pc, 1));
+                    f[0] |= exactly_two(s[2], s2y, s[1], s1z) & ((uint64_t)a.v[0] | ((uint64_t)a.v[1] << 32));
+                    f[1] |= exactly_two(s[2], s2x, s[0], s0z) & ((uint64_t)a.v[2] | ((uint64_t)a.v[3] << 32));
+                    f[2] |= exactly_two(s[1], s1x, s[0], s0y) & ((uint64_t)b.v[0] | ((uint64_t)b.v[1] << 32));
+                }
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    F0[k * N + i] = f[k];
+                    e[k] ^= f[k];
+                }
+            }
+            __syncthreads();
+            if (on) {
+                s[0] ^= f[1] ^ F0[N + zp] ^ f[2] ^ F0[2 * N + yp];
+                s[1] ^= f[0] ^ F0[zp] ^ f[2] ^ F0[2 * N + xp];
+                s[2] ^= f[0] ^ F0[yp] ^ f[1] ^ F0[N + xp];
+#pragma unroll
+                for (int k = 0; k < 3; ++k) S0[k * N + i] = s[k];
+            }
+            return s[0] | s[1] | s[2];
+        };
+
+        // up to `most` flip applications, stopping once the column is clear: the applications that ran
+        auto flip_until_clear = [&](int most) -> int {
+            uint64_t nz = s[0] | s[1] | s[2];
+            int k = 0;
+            while (k < most && __syncthreads_or(nz != 0)) {
+                nz = apply(false, 0, 0);
+                ++k;
+            }
+            return k;
+        };
+
+        auto schedule = [&](uint32_t cycle, uint32_t sweep0) {
+            for (int k = 0, letter = 0; k < pr.n_apply; ++k) {
+                __syncthreads();
+                apply((pr.sched >> letter) & 1, cycle, sweep0 + (uint32_t)k);
+                if (++letter == pr.slen) letter = 0;
+            }
+        };
+
+        if (!kRun) {
+            if (on) {
+#pragma unroll
+                for (int n = 0; n < 3; ++n) S0[n * N + i] = s[n] = sg.at(n * L3 + site);
+            }
+            if (pr.until_clear) {
+                const int k = flip_until_clear(pr.n_apply);
+                if (pr.sweeps_done && threadIdx.x == 0) atomicMax(pr.sweeps_done, k);
+            } else {
+                schedule(pr.cycle0, pr.sweep0);
+            }
+            if (on) {
+#pragma unroll
+                for (int n = 0; n < 3; ++n) {
+                    sg.at(n * L3 + site) = s[n];
+                    xor_into(&eg.at(n * L3 + site), e[n]);
+                }
+            }
+        } else {
+            // the syndrome of e, measured with error rate thr / 2^32
+            auto measure = [&](uint64_t thr, uint32_t cycle) {
+                __syncthreads();   // the last measurement's reads are done
+                if (on) {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) E0[k * N + i] = e[k];
+                }
+                __syncthreads();
+                if (on) {
+                    s[0] = e[1] ^ E0[N + zp] ^ e[2] ^ E0[2 * N + yp];
+                    s[1] = e[0] ^ E0[zp] ^ e[2] ^ E0[2 * N + xp];
+                    s[2] = e[0] ^ E0[yp] ^ e[1] ^ E0[N + xp];
+                    if (thr != 0) {
+                        const BernoulliColumn bc = bernoulli_column(pr.seed, kStreamMeas, cycle, group);
+#pragma unroll
+                        for (int n = 0; n < 3; ++n)
+                            s[n] ^= thr >> 32 ? ~0ULL : bernoulli_site(bc, (uint32_t)thr, (uint32_t)(n * L3 + site));
+                    }
+#pragma unroll
+                    for (int n = 0; n < 3; ++n) S0[n * N + i] = s[n];
+                }
+            };
+            if (on) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) e[k] = eg.at(k * L3 + site);
+            }
+            for (int c = 1; c <= pr.cycles; ++c) {
+                const uint32_t cycle = pr.cycle0 + (uint32_t)c;
+                if (pr.thr_p != 0 && on) {
+                    const BernoulliColumn bc = bernoulli_column(pr.seed, kStreamQubit, cycle, group);
+#pragma unroll
+                    for (int k = 0; k < 3; ++k)
+                        e[k] ^= pr.thr_p >> 32 ? ~0ULL
+                                               : bernoulli_site(bc, (uint32_t)pr.thr_p, (uint32_t)(k * L3 + site));
+                }
+                measure(pr.thr_q, cycle);
+                schedule(cycle, 0);
+            }
+            if (pr.perfect >= 0) {
+                measure(0, 0);
+                flip_until_clear(pr.perfect);
+            }
+            if (on) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) eg.at(k * L3 + site) = e[k];
+            }
         }
         __syncthreads();   // the next column overwrites the words
     }
@@ -645,9 +803,9 @@ t3d_status launch_slab(const ItemDesc& d, ColumnProgram pr, int kind, cudaStream
 size_t column_bytes(int L) { return (size_t)L * L * L * 72; }
 
 // Words per block and z-parts.  A block should have at least two warps, so tiny lattices take
-// several words; a lattice column is split into as many z-parts as keep about kColumnTarget
-// threads resident on an SM (all the blocks that fit its shared memory together), or, when
-// there are fewer columns than that, into one part per site.
+// several words.  A lattice that fits a block with a thread per site takes one (k_column_one); a larger
+// lattice's columns are split into as many z-parts as keep about kColumnTarget threads resident on an SM
+// (all the blocks that fit its shared memory together).
 constexpr int kColumnTarget = 1024;
 
 struct ColumnShape {
@@ -665,9 +823,9 @@ ColumnShape column_shape(int L, int64_t words)
     const int64_t columns = (words + c.wt - 1) / c.wt;
     const int fit = (int)std::max<size_t>(1, std::min<size_t>(32, kColumnSmem / (c.smem + 1024)));
     const int per_sm = (int)std::min<int64_t>(fit, std::max<int64_t>(1, (columns + 151) / 152));
-    c.zt = 1;
-    for (int z = 2; z <= L; ++z)
-        if (plane * z <= kColumnThreads && plane * z * per_sm <= kColumnTarget) c.zt = z;
+    c.zt = plane * L <= kColumnThreads ? L : 1;
+    for (int z = 2; z < L; ++z)
+        if (c.zt < L && plane * z <= kColumnThreads && plane * z * per_sm <= kColumnTarget) c.zt = z;
     c.threads = (plane * c.zt + 31) / 32 * 32;
     return c;
 }
@@ -680,7 +838,7 @@ t3d_status launch_column(const ItemDesc& item, ColumnProgram pr, int kind, cudaS
     const ColumnShape c = column_shape(d.lat.L, words);
     d.tx = c.wt;
     pr.zt = c.zt;
-    auto kernel = k_column<kRun>;
+    auto kernel = c.zt == d.lat.L ? k_column_one<kRun> : k_column<kRun>;
     T3D_TRY(allow_dynamic_smem((const void*)kernel, c.smem));
     ProfScope prof(kind, st);
     kernel<<<persistent_grid((const void*)kernel, c.threads, kind, (words + c.wt - 1) / c.wt, false, c.smem),

@@ -68,3 +68,23 @@ def test_sweeps_and_until_clear_match_oracle(L, S):
     clear = zeros_words(n, S)
     t3d.toric3d_flip_until_clear(L, e, clear, 6, work, done)
     assert int(done.item()) == 0 and not clear.any()
+
+
+@pytest.mark.parametrize("L,S,T,schedule,n_apply", [(3, 129, 3, "F", 0), (6, 64 * 700 + 9, 2, "FP", 3),
+                                                    (8, 64 * 400, 2, "FFPFF", 5), (10, 64 * 310 + 5, 2, "PF", 2),
+                                                    (11, 64 * 3 + 1, 2, "PF", 2)])
+def test_runs_with_a_thread_per_site_match_oracle(L, S, T, schedule, n_apply):
+    # L = 10 is the largest lattice with a thread per site, L = 11 the first without; more columns than
+    # blocks resident at once; n_apply = 0: measurements follow each other directly
+    n = 3 * L ** 3
+    kw = dict(schedule=schedule, n_apply=n_apply, perfect_round=True, perfect_max_sweeps=3)
+    start = inp.random_bits(S, n, 0.02, seed=L)
+    cfg = t3d.make_run_cfg(L, T, 0.03, 0.03, 78, S, sample0=64, cycle0=1, use_graph=False, **kw)
+    e, mask = upload_bits(start), torch.zeros(S, dtype=torch.uint8, device=dev())
+    t3d.toric3d_run_cycles(cfg, e, workspace(t3d.toric3d_run_workspace_bytes(cfg)), mask)
+    got_e, got_mask = download_bits(e, S), mask.cpu().numpy()
+    for a in {0, (S - 1) // 64 * 64}:   # the first words and the last
+        k = min(S - a, 100)
+        want_mask, want_e = oracle.run_batch(oracle.make_cfg(L, T, 0.03, 0.03, 78, cycle0=1, **kw), 64 + a, k,
+                                             start[a:a + k])
+        assert np.array_equal(got_e[a:a + k], want_e) and np.array_equal(got_mask[a:a + k], want_mask)
