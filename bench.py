@@ -39,13 +39,15 @@ VALUE_IS = "BP+p-flip; learned_pflip.value = learned+p-flip, learned_pflip.vs_bp
 
 # DRAM bytes (read + write) per edge-sample of the dominant kernel from one
 # ncu capture of the current k_bp_step (L = 32, 1024 samples; traffic grows in
-# proportion to the samples a launch covers, so it scales to full launches).
+# proportion to the samples a launch covers, so it scales to full launches); the
+# first launch of a chunk does the first two iterations and reads only syndrome words.
 # Set to None when the kernel changes until it is captured again.
-BP_STEP_TRAFFIC = {"first_iteration": 15.69, "full_iteration": 31.90}
-# The same for k_flip_tiled inside the FFPFF cycle at p = q = 4% (L = 32, 8192 samples, the
-# four flip applications of one cycle: 322.4 MB of DRAM traffic each on average, per
-# qubit-sample 0.400 B against the dense 0.5 B: e is touched only where a word has a flipped
-# lane, so the figure depends on the noise rates).  None when the kernel changes.
+BP_STEP_TRAFFIC = {"first_two_iterations": 15.67, "full_iteration": 31.93}
+# The same for k_flip_tiled (schedules taken step by step: lattices above L = 32, short schedules)
+# inside the FFPFF cycle at p = q = 4% (L = 32, 8192 samples, the four flip applications of one
+# cycle: 322.4 MB of DRAM traffic each on average, per qubit-sample 0.400 B against the dense
+# 0.5 B: e is touched only where a word has a flipped lane, so the figure depends on the noise
+# rates).  None when the kernel changes.
 FLIP_TRAFFIC_P = 0.04
 FLIP_TRAFFIC = 322.4e6 / (98304 * 8192)
 UNIT = "qubit-cycles/s"
@@ -339,10 +341,12 @@ SWEEP_BYTES = {"noise": 0.25, "syndrome": 0.25, "flip": 0.5, "pflip": 0.875}
 # Warp instructions per 64-sample word of each qubit (noise), check (syndrome)
 # or site (the decision pass of one p-flip application) at p = q = 4%, from one
 # ncu capture of the current kernels (smsp__inst_executed.sum / (units x words),
-# L = 32, 8192 samples: 157.0 M, 189.7 M and 51.8 M instructions).  The Philox
-# arithmetic binds these kernels on the instruction issue rate.
+# L = 32, 8192 samples: 105.3 M, 118.7 M and 51.8 M instructions).  The Philox
+# arithmetic binds these kernels on the integer pipe.
 SWEEP_INST_P = 0.04
-SWEEP_INST = {"noise": 157.0e6 / (98304 * 128), "syndrome": 189.7e6 / (98304 * 128), "pflip": 51.8e6 / (32768 * 128)}
+SWEEP_INST = {"noise": 105.3e6 / (98304 * 128), "syndrome": 118.7e6 / (98304 * 128), "pflip": 51.8e6 / (32768 * 128)}
+# A schedule run on chip reads s and e and writes both once, whatever its length.
+SCHEDULE_BYTES = 0.5
 # The p-flip syndrome pass reads the flip words and updates s in place (0.375 B).
 PFLIP_APPLY_BYTES = 0.375
 
@@ -355,17 +359,26 @@ def sweep_roofline(prof, w, qubits, S, steps, ms, hbm_peak, peak_source, clk):
     n_p = sum(1 for k in range(w.n_apply) if w.schedule[k % len(w.schedule)] == "P")
     per_step = {"noise": 1, "syndrome": 1, "flip": w.n_apply - n_p, "pflip": n_p}
     kinds = {k: prof[k] for k in SWEEP_BYTES if prof[k][1]}
+    unit_bytes = SWEEP_BYTES
+    sweep_launches = prof["flip"][1] + prof["pflip"][1]
+    if sweep_launches < (per_step["flip"] + 2 * n_p) * steps:
+        # fewer launches than steps: the whole schedule ran on chip (all of it under one kind)
+        per_step = {"noise": 1, "syndrome": 1, "schedule": 1}
+        unit_bytes = {"noise": SWEEP_BYTES["noise"], "syndrome": SWEEP_BYTES["syndrome"], "schedule": SCHEDULE_BYTES}
+        kinds = {k: prof[k] for k in ("noise", "syndrome") if prof[k][1]}
+        kinds["schedule"] = (prof["flip"][0] + prof["pflip"][0], sweep_launches)
     dom = max(kinds, key=lambda k: kinds[k][0])
     d_ms, d_launches = kinds[dom]
     apps = per_step[dom] * steps                      # applications (a p-flip one is two launches)
     t_app = d_ms / apps / 1e3
     words = (S + 63) // 64
-    cycle_bytes = sum(SWEEP_BYTES[k] * per_step[k] for k in SWEEP_BYTES) * qubits * S * steps
+    cycle_bytes = sum(unit_bytes[k] * per_step[k] for k in unit_bytes) * qubits * S * steps
     out = {"kernel": {"noise": "k_noise", "syndrome": "k_syndrome", "flip": "k_flip_tiled",
-                      "pflip": "k_pflip_decide + k_pflip_apply"}[dom],
+                      "pflip": "k_pflip_decide + k_pflip_apply",
+                      "schedule": "k_slab + k_to_columns + k_from_columns (or k_column)"}[dom],
            "launches": d_launches, "avg_launch_ms": d_ms / d_launches, "ms_per_application": 1e3 * t_app,
            "share_of_step": d_ms / ms, "cycle_hbm_frac": cycle_bytes / (ms / 1e3) / 1e9 / hbm_peak,
-           "kernels_hbm_frac": {k: SWEEP_BYTES[k] * qubits * S * steps * per_step[k] / (v[0] / 1e3) / 1e9 / hbm_peak
+           "kernels_hbm_frac": {k: unit_bytes[k] * qubits * S * steps * per_step[k] / (v[0] / 1e3) / 1e9 / hbm_peak
                                 for k, v in kinds.items()},
            "traffic": None, "peak_source": peak_source}
     if (dom == "flip" and FLIP_TRAFFIC and abs(w.p - FLIP_TRAFFIC_P) < 1e-12 and abs(w.q - FLIP_TRAFFIC_P) < 1e-12):
@@ -380,10 +393,15 @@ def sweep_roofline(prof, w, qubits, S, steps, ms, hbm_peak, peak_source, clk):
         b_noise = max(SWEEP_BYTES["noise"] * qubits * S / hbm, SWEEP_INST["noise"] * units["noise"] * words / issue_peak)
         b_syn = max(SWEEP_BYTES["syndrome"] * qubits * S / hbm,
                     SWEEP_INST["syndrome"] * units["syndrome"] * words / issue_peak)
-        b_flip = SWEEP_BYTES["flip"] * qubits * S / hbm
-        b_pflip = (max((SWEEP_BYTES["pflip"] - PFLIP_APPLY_BYTES) * qubits * S / hbm,
-                       SWEEP_INST["pflip"] * units["pflip"] * words / issue_peak) + PFLIP_APPLY_BYTES * qubits * S / hbm)
-        bound_s = b_noise + b_syn + per_step["flip"] * b_flip + per_step["pflip"] * b_pflip
+        i_pflip = SWEEP_INST["pflip"] * units["pflip"] * words / issue_peak
+        if "schedule" in per_step:
+            b_sched = max(SCHEDULE_BYTES * qubits * S / hbm, n_p * i_pflip)
+        else:
+            b_flip = SWEEP_BYTES["flip"] * qubits * S / hbm
+            b_pflip = (max((SWEEP_BYTES["pflip"] - PFLIP_APPLY_BYTES) * qubits * S / hbm, i_pflip) +
+                       PFLIP_APPLY_BYTES * qubits * S / hbm)
+            b_sched = per_step["flip"] * b_flip + per_step["pflip"] * b_pflip
+        bound_s = b_noise + b_syn + b_sched
         out["cycle_bound_ms"] = 1e3 * bound_s
         out["cycle_roofline_frac"] = bound_s / (ms / 1e3 / steps)
         out["cycle_roofline"] = ("sum over the cycle's kernels of max(algorithmic bytes / HBM peak, warp "
@@ -394,7 +412,7 @@ def sweep_roofline(prof, w, qubits, S, steps, ms, hbm_peak, peak_source, clk):
         out.update(bound="alu", achieved=achieved, peak=peak, unit="Ginst/s", frac=achieved / peak,
                    peak_derivation=f"152 SMs x 4 schedulers x 1 warp instruction/clock x {sm_mhz:.0f} MHz")
     else:
-        alg = SWEEP_BYTES[dom] * qubits * S
+        alg = unit_bytes[dom] * qubits * S
         achieved = alg / t_app / 1e9
         out.update(bound="hbm", achieved=achieved, peak=hbm_peak, unit="GB/s", frac=achieved / hbm_peak,
                    algorithmic_bytes_per_application=alg)
@@ -487,15 +505,15 @@ def cuda_arm(args):
     peak_source = "MEASURED_PEAKS.json hbm_gbs (measured)" if peaks else "fallback 6.8 TB/s"
     if kw["use_bp"]:
         # dominant kernel: BP iteration (algorithmic bytes per edge-sample: 16 B read + 16 B
-        # written; the first iteration of each chunk reads nothing)
+        # written; the first two iterations of each chunk are one launch that reads no messages)
         bp_ms, bp_launches = prof["bp_step"]
         rounds = math.ceil(S / chunk)
-        alg_bytes = qubits * S * args.steps * (32.0 * (w.bp_iters - 1) + 16.0)
+        alg_bytes = qubits * S * args.steps * (32.0 * max(w.bp_iters - 2, 0) + 16.0)
         achieved = alg_bytes / (bp_ms / 1e3) / 1e9 if bp_ms > 0 else 0.0
         traffic = None
         if BP_STEP_TRAFFIC and bp_launches:
-            traffic = qubits * S * args.steps * (BP_STEP_TRAFFIC["first_iteration"] +
-                                                 BP_STEP_TRAFFIC["full_iteration"] * (w.bp_iters - 1)) / bp_launches
+            traffic = qubits * S * args.steps * (BP_STEP_TRAFFIC["first_two_iterations"] +
+                                                 BP_STEP_TRAFFIC["full_iteration"] * max(w.bp_iters - 2, 0)) / bp_launches
         roofline = {"kernel": "k_bp_step", "bound": "hbm", "achieved": achieved, "peak": hbm_peak, "unit": "GB/s",
                     "frac": achieved / hbm_peak, "traffic": traffic, "peak_source": peak_source,
                     "launches": bp_launches, "avg_launch_ms": bp_ms / max(bp_launches, 1),
