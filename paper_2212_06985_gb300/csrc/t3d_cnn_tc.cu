@@ -193,29 +193,6 @@ __device__ bool wait_bar(uint32_t bar, uint32_t parity, volatile uint32_t* abort
     }
 }
 
-// Wait for phase 0 of a barrier that completes only at the end of a long launch: gives up
-// (error flag, abort) once *progress has not changed for g_tc_wait_ns.
-__device__ bool wait_bar_progress(uint32_t bar, volatile uint32_t* progress, volatile uint32_t* abort_flag)
-{
-    uint64_t t0 = global_ns();
-    uint32_t last = *progress;
-    for (;;) {
-        for (int i = 0; i < 32; ++i)
-            if (mbar_try_wait(bar, 0)) return true;
-        if (*abort_flag) return false;
-        const uint32_t now_p = *progress;
-        const uint64_t now = global_ns();
-        if (now_p != last) {
-            last = now_p;
-            t0 = now;
-        } else if (now - t0 > *(volatile unsigned long long*)&g_tc_wait_ns) {
-            *abort_flag = 1;
-            atomicOr(&g_tc_error, 1u);
-            return false;
-        }
-    }
-}
-
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar)
 {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
@@ -1017,24 +994,30 @@ __global__ void k_expand_bits(int L3, int64_t Sp, int64_t W, int64_t words, cons
 // channels, LBO 128 B to the next 8 samples, SBO 2048 B to the next 8 channels, which is also the
 // step to the next tile of a run).
 //
-// Work unit: one 128-sample tile x one row (y, z), walked along x.  The 9 tiles around the row at
-// one x, (dy, dz) = -1..1, form a column.  A column meets the d tiles of the three sites
-// x - 1, x, x + 1 as dx = +1, 0, -1 at once: the MMA's M rows are the column's tiles (and a tile of
-// ones, whose rows give the bias gradient sum d[r][s][co]), its N = 48 columns those three d tiles.
-// So every x tile is copied and multiplied once per row, ten tiles a site with d's, where fetching
-// a site's 27 neighbours took 29 tiles; and a site takes 16 MMAs (first layer: 8) where N = 16
-// columns per neighbour took 32 (16).  M is 128: eight 16-channel tiles, then the ninth and the ones
-// in an MMA of their own; the first layer's nine 8-channel tiles and the ones fit one.  Rows past a
-// group's last tile multiply whatever follows in shared memory and are never read.
+// Work unit: one 128-sample tile x two rows (y, z), (y + 1, z), walked along x.  The 12 tiles around
+// the rows at one x, (dy, dz) = -1..2 x -1..1 with dy fastest, form a column.  A column meets the d tiles
+// of a row's three sites x - 1, x, x + 1 as dx = +1, 0, -1 at once: the MMA's M rows are the column's
+// tiles (and a tile of ones, whose rows give the bias gradient sum d[r][s][co]), its N = 48 columns those
+// three d tiles.  The second row takes the same column from one tile further on, so that dy counts from
+// it, into the same accumulators (of every four tiles three are read); the ones are there twice.  So an x
+// tile is copied once per two rows: seven tiles a site with the d's, where fetching a site's 27
+// neighbours took 29; and a site takes 16 MMAs (first layer: 8) where N = 16 columns per neighbour took
+// 32 (16).  M is 128: eight 16-channel tiles, then the other four and the ones in an MMA of their own;
+// the first layer's twelve 8-channel tiles and the ones fit one.  Rows past a group's last tile multiply
+// whatever follows in shared memory and are never read.
 //
-// The d tiles sit in a ring of eight slots whose first two are written a second time behind the last,
-// so that any three in a row are contiguous.  The accumulators (48 columns of TMEM per group) live for
-// the whole launch and are added to the gradients at its end.
+// (Both rows' d tiles in one MMA of N = 96, the two rows' sums apart, is faster still, 77 and 55 us.  But
+// the tensor cores' sums over half the terms differ from the whole ones by 3e-5.)
 //
-// What bounds it: the MMAs (16 a site, 53 cycles each however small N is, 80 us) and the copies to
-// shared memory (42 KB a site, 1.2 GB; about 10 TB/s) alike.  L = 12, 2,048 samples: 113 us for a
-// 16-channel layer, 98 us for the first.  Before, with channel-major copies of x and d written first
-// (350 us a step in all), 27 neighbour tiles fetched per site and N = 16: 490 and 330 us.
+// The d tiles of each row sit in a ring of slots whose first two are written a second time behind the
+// last, so that any three in a row are contiguous.  The accumulators (48 columns of TMEM per group) live
+// for the whole launch; at its end they go through shared memory, so that they are added to the gradients
+// in runs (every lane adding its own: about 10 us more).
+//
+// What bounds it: the MMAs (53 cycles each however small N is, 80 us) and the copies to shared memory (29
+// KB a site, first layer 17) alike.  L = 12, 2,048 samples: 103 us for a 16-channel layer, 65 us for the
+// first; a row at a time (42 KB a site) 113 and 98.  Before, with channel-major copies of x and d written
+// first (350 us a step in all), 27 neighbour tiles fetched per site and N = 16: 490 and 330 us.
 //
 // One elected thread of a converged warp issues the MMAs, and one of each of three producer warps the
 // copies: warp and loop state are then uniform, and addresses and descriptors stay in uniform
@@ -1046,23 +1029,23 @@ constexpr int kWgThreads = kTcThreads + 32 * (kWgProducers - 1);
 template <int kCin>
 struct WgShape {
     static constexpr uint32_t kTileB = kCin * 256;               // one x tile
-    static constexpr uint32_t kColB = 10 * kTileB;               // nine tiles and the ones
-    static constexpr int kCols = kCin == 16 ? 4 : 6;             // column slots
-    static constexpr int kGroups = kCin == 16 ? 2 : 1;           // M groups: tiles 0..7 and 8..9
-    static constexpr int kD = 8;                                 // d slots (and two mirrors), 4 KiB each
+    static constexpr uint32_t kColB = 14 * kTileB;               // twelve tiles and the ones twice
+    static constexpr int kCols = kCin == 16 ? 3 : 5;             // column slots
+    static constexpr int kGroups = kCin == 16 ? 2 : 1;           // M groups: tiles 0..7 and 8..12
+    static constexpr int kD = 5;                                 // a row's d slots (and two mirrors), 4 KiB each
     static constexpr uint32_t kOffD = kCols * kColB;
-    static constexpr uint32_t kOffBar = kOffD + (kD + 2) * 4096;
+    static constexpr uint32_t kOffBar = kOffD + 2 * (kD + 2) * 4096;
     static constexpr int kBars = 2 * kCols + kD + 1;             // column full, empty; d empty; done
     static constexpr uint32_t kOffMisc = kOffBar + kBars * 8;
     static constexpr int kSmem = (int)kOffMisc + 16 + 1024;
     static_assert(kSmem <= 227 * 1024, "shared memory budget");
     // a group reads 32 KiB from its first tile on
-    static_assert(kOffBar >= (kCols - 1) * kColB + (kGroups - 1) * 8 * kTileB + 32768, "group reads stay inside");
+    static_assert(kOffBar >= (kCols - 1) * kColB + ((kGroups - 1) * 8 + 1) * kTileB + 32768, "group reads stay inside");
 };
 
 struct WgArgs {
     int L, L3;
-    int64_t n_units;            // 128-sample tiles x L^2 rows
+    int64_t n_units;            // 128-sample tiles x L planes x ceil(L / 2) pairs of rows
     const uint8_t* x;           // x tiles (kCin channels)
     const uint8_t* d;           // d tiles (16 channels)
     const uint8_t* ones;        // one x tile of BF16 ones
@@ -1086,46 +1069,47 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
     auto col_empty = [&](uint32_t q) { return bars + 8u * (kNc + q % kNc); };
     auto d_empty = [&](uint32_t q) { return bars + 8u * (2 * kNc + q % kNd); };
     auto col_at = [&](uint32_t q) { return base + (q % kNc) * Sh::kColB; };
-    auto d_at = [&](uint32_t q) { return base + Sh::kOffD + (q % kNd) * 4096u; };
+    auto d_at = [&](uint32_t q, int r) { return base + Sh::kOffD + ((uint32_t)r * (kNd + 2) + q % kNd) * 4096u; };
     const uint32_t done_bar = bars + 8u * (2 * kNc + kNd);
-    uint32_t* misc = reinterpret_cast<uint32_t*>(sm + Sh::kOffMisc);   // [0] TMEM base, [1] abort, [2] progress
+    uint32_t* misc = reinterpret_cast<uint32_t*>(sm + Sh::kOffMisc);   // [0] TMEM base, [1] abort
     volatile uint32_t* abort_flag = misc + 1;
-    volatile uint32_t* progress = misc + 2;
     // the shuffle makes the warp index uniform for the compiler
     const int warp = __shfl_sync(0xffffffffu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        misc[2] = 0;
         for (int i = 0; i < Sh::kBars; ++i) mbar_init(bars + 8u * (uint32_t)i, i < Sh::kCols ? kWgProducers : 1);
         misc[1] = 0;
         fence_mbar_init();
     }
-    // the ones behind every column's nine tiles
-    for (uint32_t i = threadIdx.x; i < kNc * (kTileB / 16); i += blockDim.x)
-        reinterpret_cast<uint4*>(sm + (i / (kTileB / 16)) * Sh::kColB + 9u * kTileB)[i % (kTileB / 16)] =
-            reinterpret_cast<const uint4*>(a.ones)[i % (kTileB / 16)];
+    // the ones behind every column's twelve tiles
+    constexpr uint32_t kOnes = kTileB / 16;
+    for (uint32_t i = threadIdx.x; i < kNc * 2 * kOnes; i += blockDim.x)
+        reinterpret_cast<uint4*>(sm + (i / (2 * kOnes)) * Sh::kColB + 12u * kTileB)[i % (2 * kOnes)] =
+            reinterpret_cast<const uint4*>(a.ones)[i % kOnes];
     fence_proxy_async_smem();
     if (warp == kIssuerWarp) tmem_alloc(smem_u32(misc), 128);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, misc[0], 0);
-    const int L = a.L, L2 = L * L;
+    bool finished = true;   // the issuer's: every MMA has completed
+    const int L = a.L, pairs = (L + 1) / 2, per_tile = pairs * L;
 
     if (warp == kProducerWarp || warp > kIssuerWarp) {
-        // producer p copies the tiles 3 p .. 3 p + 2 of a column, the last one the d tiles too
+        // producer p copies the tiles 4 p .. 4 p + 3 of a column, the last one the d tiles too
         const int part = warp == kProducerWarp ? 0 : warp - kIssuerWarp;
         const bool leader = elect_one();
         uint32_t cq = 0, dq = 0;   // columns and d tiles copied so far
         bool ok = true;
         for (int64_t u = blockIdx.x; u < a.n_units && ok; u += gridDim.x) {
-            const int64_t t = u / L2;
-            const int row = (int)(u - t * L2), y = row % L, z = row / L;
+            const int64_t t = u / per_tile;
+            const int row = (int)(u - t * per_tile), y = 2 * (row % pairs), z = row / pairs;
             const uint8_t* xt = a.x + t * a.L3 * (int64_t)kTileB;
-            const uint8_t* dt = a.d + (t * a.L3 + (int64_t)row * L) * 4096;
-            // the row of tile i = 3 part + k: (dy, dz) = (i % 3 - 1, i / 3 - 1) = (k - 1, part - 1)
-            const uint8_t* xrow[3];
+            const uint8_t* dt = a.d + (t * a.L3 + ((int64_t)z * L + y) * L) * 4096;
+            const uint32_t rows = y + 1 < L ? 2 : 1;   // the odd lattice's last row is alone
+            // the row of tile i = 4 part + k: (dy, dz) = (i % 4 - 1, i / 4 - 1) = (k - 1, part - 1)
+            const uint8_t* xrow[4];
 #pragma unroll
-            for (int k = 0; k < 3; ++k)
+            for (int k = 0; k < 4; ++k)
                 xrow[k] = xt + ((int64_t)wrap(z + part - 1, L) * L + wrap(y + k - 1, L)) * L * (int64_t)kTileB;
             for (int c = 0; c < L; ++c) {
                 // d tiles in the order L - 1, 0, 1, .., L - 1, 0: the first column brings three of them
@@ -1140,16 +1124,18 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
                 }
                 ok = __all_sync(0xffffffffu, good);
                 if (!ok) break;
-                if (leader) mbar_arrive_expect_tx(col_full(cq), 3u * kTileB + (nd + mirrors) * 4096u);
+                if (leader) mbar_arrive_expect_tx(col_full(cq), 4u * kTileB + (nd + mirrors) * rows * 4096u);
 #pragma unroll
-                for (int k = 0; k < 3; ++k)
+                for (int k = 0; k < 4; ++k)
                     if (leader)
-                        bulk_load(col_at(cq) + (uint32_t)(3 * part + k) * kTileB, xrow[k] + (uint32_t)c * kTileB, kTileB,
+                        bulk_load(col_at(cq) + (uint32_t)(4 * part + k) * kTileB, xrow[k] + (uint32_t)c * kTileB, kTileB,
                                   col_full(cq));
                 for (uint32_t k = dq; k < dq + nd; ++k) {
                     const uint8_t* src = dt + (int64_t)wrap(c + 1 - (int)(dq + nd - 1 - k), L) * 4096;
-                    if (leader) bulk_load(d_at(k), src, 4096u, col_full(cq));
-                    if (leader && k % kNd < 2) bulk_load(d_at(k) + kNd * 4096u, src, 4096u, col_full(cq));
+                    for (uint32_t r = 0; r < rows; ++r, src += (int64_t)L * 4096) {
+                        if (leader) bulk_load(d_at(k, (int)r), src, 4096u, col_full(cq));
+                        if (leader && k % kNd < 2) bulk_load(d_at(k, (int)r) + kNd * 4096u, src, 4096u, col_full(cq));
+                    }
                 }
                 ++cq;
                 dq += nd;
@@ -1168,25 +1154,30 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
         uint32_t cq = 0, dq = 0;   // columns done; the first d tile of the current column's three
         bool ok = true;
         for (int64_t u = blockIdx.x; u < a.n_units && ok; u += gridDim.x) {
+            const bool alone = L % 2 != 0 && u % pairs == pairs - 1;   // the odd lattice's last row
             for (int c = 0; c < L; ++c) {
                 bool good = true;
                 if (leader) good = wait_bar(col_full(cq), (cq / kNc) & 1u, abort_flag);
                 ok = __all_sync(0xffffffffu, good);
                 if (!ok) break;
                 tc_fence_after();
-                const uint64_t bdesc = smem_desc(d_at(dq), 128u, 2048u);
 #pragma unroll
-                for (int grp = 0; grp < Sh::kGroups; ++grp) {
-                    const uint64_t adesc = smem_desc(col_at(cq) + (uint32_t)grp * 8u * kTileB, 128u, 2048u);
+                for (int r = 0; r < 2; ++r) {
+                    if (r == 1 && alone) break;
+                    const uint64_t bdesc = smem_desc(d_at(dq, r), 128u, 2048u);
 #pragma unroll
-                    for (int kk = 0; kk < 8; ++kk) {
-                        // 16 samples per step: two core matrices (256 B) further along K
-                        const uint64_t step = (uint64_t)((kk * 256) >> 4);
-                        if (leader) {
-                            if (kk == 0 && cq == 0)
-                                mma_bf16_overwrite(tmem + (uint32_t)(grp * 48), adesc + step, bdesc + step, kIdesc);
-                            else
-                                mma_bf16_n(tmem + (uint32_t)(grp * 48), adesc + step, bdesc + step, kIdesc);
+                    for (int grp = 0; grp < Sh::kGroups; ++grp) {
+                        const uint64_t adesc = smem_desc(col_at(cq) + (uint32_t)(grp * 8 + r) * kTileB, 128u, 2048u);
+#pragma unroll
+                        for (int kk = 0; kk < 8; ++kk) {
+                            // 16 samples per step: two core matrices (256 B) further along K
+                            const uint64_t step = (uint64_t)((kk * 256) >> 4);
+                            if (leader) {
+                                if (r == 0 && kk == 0 && cq == 0)
+                                    mma_bf16_overwrite(tmem + (uint32_t)(grp * 48), adesc + step, bdesc + step, kIdesc);
+                                else
+                                    mma_bf16_n(tmem + (uint32_t)(grp * 48), adesc + step, bdesc + step, kIdesc);
+                            }
                         }
                     }
                 }
@@ -1200,43 +1191,46 @@ __global__ void __launch_bounds__(kWgThreads, 1) k_wgrad_tc(const __grid_constan
                 }
                 ++cq;
                 ++dq;
-                if (leader) *progress = cq;
             }
             dq += 2;
         }
         if (leader) {
             mma_commit(done_bar);
-            wait_bar(done_bar, 0, abort_flag, true);
+            finished = wait_bar(done_bar, 0, abort_flag, true);
         }
         __syncwarp();
-    } else if (warp < kEpiWarps) {
-        // every MMA has completed: add the accumulators to the gradients; TMEM lane = M row
-        int got = 1;
-        if (lane == 0) got = wait_bar_progress(done_bar, progress, abort_flag) ? 1 : 0;
-        got = __shfl_sync(0xffffffffu, got, 0);
-        tc_fence_after();
-        if (got && !*abort_flag) {
-            const int m = warp * 32 + lane, ci = m % kCin;
+    }
+    // every MMA and copy has completed (or the launch gave up): the sums go to shared memory in the
+    // gradients' layout, and from there to the gradients in runs
+    tc_fence_before();
+    const bool good = __syncthreads_and(finished && !*abort_flag);
+    tc_fence_after();
+    if (good) {
+        float* g = reinterpret_cast<float*>(sm);   // [co][cin][27], then [16] of the bias
+        const int n_w = kC * a.cin * kOff;
+        if (warp < kEpiWarps) {
+            const int m = warp * 32 + lane, ci = m % kCin;   // TMEM lane = M row
 #pragma unroll
             for (int grp = 0; grp < Sh::kGroups; ++grp) {
-                const int i = grp * 8 + m / kCin;   // the row's tile of the column, (dy, dz) = i
-                const bool mine = kCin == 8 || grp == 1 || i < 8;
+                const int i = grp * 8 + m / kCin;            // the tile from the row's first, (dy, dz) = (i % 4, i / 4) - 1
 #pragma unroll
-                for (int j = 0; j < 3; ++j) {       // the site c - 1 + j: dx = 1 - j
+                for (int j = 0; j < 3; ++j) {                // the site c - 1 + j: dx = 1 - j
                     uint32_t v[16];
                     tmem_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(grp * 48 + j * 16), v);
                     tmem_wait_ld();
-                    if (mine && i < 9 && ci < a.cin) {
+                    if (i < 12 && (i & 3) < 3 && ci < a.cin) {
 #pragma unroll
                         for (int co = 0; co < 16; ++co)
-                            atomicAdd(&a.gw[(co * a.cin + ci) * kOff + 3 * i + 2 - j], __uint_as_float(v[co]));
-                    } else if (mine && i == 9 && ci == 0 && j == 1) {
+                            g[(co * a.cin + ci) * kOff + 3 * (3 * (i >> 2) + (i & 3)) + 2 - j] = __uint_as_float(v[co]);
+                    } else if (i == 12 && ci == 0 && j == 1) {
 #pragma unroll
-                        for (int co = 0; co < 16; ++co) atomicAdd(&a.gb[co], __uint_as_float(v[co]));
+                        for (int co = 0; co < 16; ++co) g[n_w + co] = __uint_as_float(v[co]);
                     }
                 }
             }
         }
+        __syncthreads();
+        for (int i = threadIdx.x; i < n_w + kC; i += blockDim.x) atomicAdd(i < n_w ? a.gw + i : a.gb + (i - n_w), g[i]);
     }
     tc_fence_before();
     __syncthreads();
@@ -1428,7 +1422,7 @@ t3d_status tc_weight_grad(int L, int64_t n_samples, int x_ch, int cin_kept, cons
     std::memset(&a, 0, sizeof(a));
     a.L = L;
     a.L3 = (int)L3;
-    a.n_units = n_items / L;
+    a.n_units = n_items / (L * L) * ((L + 1) / 2);
     a.x = x;
     a.d = d;
     a.ones = ones;
