@@ -309,6 +309,12 @@ __device__ __forceinline__ uint64_t bernoulli_site(const BernoulliColumn& bc, ui
 #pragma unroll
     for (int blk = 0; blk < 3; ++blk) {
         const U32x4 o = philox_finish(bc.col, ps, bc.blk[blk]);
+        // both bits 0, as in the first blocks of small rates (P < 1/4, < 1/16): one three-input operation a
+        // half (L = 32, 10^5 samples at 4%: a cycle's noise and measurement 3.83 -> 3.55 ms)
+        if (((thr >> (30 - 2 * blk)) & 3u) == 0) {
+            eq &= ~((uint64_t)(o.v[0] | o.v[2]) | ((uint64_t)(o.v[1] | o.v[3]) << 32));
+            continue;
+        }
 #pragma unroll
         for (int i = 0; i < 2; ++i) {
             const uint64_t w = (uint64_t)o.v[2 * i] | ((uint64_t)o.v[2 * i + 1] << 32);
