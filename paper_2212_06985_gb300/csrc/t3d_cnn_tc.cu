@@ -470,18 +470,19 @@ __device__ __forceinline__ Unit col_unit_of(const TcArgs& a, int64_t u)
 }
 
 // Warps of the column kernel: two epilogue groups of four (group g drains the output planes of parity
-// g), the producers, the issuer.  A group needs longer for a plane (TMEM load, zeroing, conversion and
-// their latencies, one after the other) than the MMAs of the next plane take.
+// g), the producers, the issuer.
 //
 // Roles are warp-uniform (the warp index comes from a shuffle, the issuing lane from elect.sync), so
 // descriptors, barriers and addresses stay in uniform registers: from a branch on the lane index an MMA
 // took 94 - 112 cycles to issue (the pipe takes one in 53 for N <= 64) and a copy 117 - 190.
 //
-// Times at L = 24, 4,864 samples (38 tiles, 36 units a CTA), before -> now: first layer 762 -> 607 us,
-// hidden 1250 -> 1165, head 1276 -> 991.  One producer: 623, 1184, 1000; four: 614, 1147, 1029.  Four
-// epilogue warps and no prefetch cost 3% each.  What bounds it: the input tiles' way into shared memory,
-// 16 tiles a plane of four output sites, 8.6 GB a hidden layer, at 7.4 TB/s (8.7 for the head, which
-// writes no activations); the MMAs of a plane take 1344 of its 2380 cycles.
+// Times at L = 24, 4,864 samples (38 tiles, 36 units a CTA), lane-indexed roles -> now: first layer 762 ->
+// 591 us, hidden 1250 -> 1130, head 1276 -> 952.  Without the prefetch 600, 1154, 961, and a decode of L =
+// 12, 2,048 samples 200 us against 190.  One epilogue group is 1% faster there (581, 1125, 946) and 3%
+// slower at L = 12, where planes are drained in bursts.  One producer instead of two 2% slower, four 4%
+// slower in the head.  What bounds it: the input tiles' way into shared memory, 16 tiles a plane of four
+// output sites, 8.6 GB a hidden layer, at 7.6 TB/s (9.0 for the head, which writes no activations); the
+// MMAs of a plane take 1344 of its 2300 cycles.
 constexpr int kConvProducers = 2;
 constexpr int kConvEpi = 8;
 // Training's head has a heavier epilogue (an exponential, a logarithm, a division and about 300 FMAs a
