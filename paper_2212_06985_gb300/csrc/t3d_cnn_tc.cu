@@ -479,7 +479,7 @@ __device__ __forceinline__ Unit col_unit_of(const TcArgs& a, int64_t u)
 // Times at L = 24, 4,864 samples (38 tiles, 36 units a CTA), lane-indexed roles -> now: first layer 762 ->
 // 591 us, hidden 1250 -> 1130, head 1276 -> 952.  Without the prefetch 600, 1154, 961, and a decode of L =
 // 12, 2,048 samples 200 us against 190.  One epilogue group is 1% faster there (581, 1125, 946) and 3%
-// slower at L = 12, where planes are drained in bursts.  One producer instead of two 2% slower, four 4%
+// slower at L = 12 (195 us against 190).  One producer instead of two 2% slower, four 4%
 // slower in the head.  What bounds it: the input tiles' way into shared memory, 16 tiles a plane of four
 // output sites, 8.6 GB a hidden layer, at 7.6 TB/s (9.0 for the head, which writes no activations); the
 // MMAs of a plane take 1344 of its 2300 cycles.
