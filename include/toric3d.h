@@ -492,7 +492,9 @@ t3d_status toric3d_cnn_train_step(int L, int64_t n_samples, const uint64_t* s_pr
  * paper's multi-size threshold plots, Fig. 2, 6, 7).  Up to 8 independent
  * ensembles, each with its own L, sample range and state, advance through the
  * same cycles with the decoder settings of `cfg` (its L, n_samples and sample0
- * are ignored); every step is one launch over all ensembles.  e,
+ * are ignored).  A step is one launch over all ensembles, except that an
+ * ensemble whose schedule (or, without BP and up to L = 14, whose whole run)
+ * is estimated to be faster on chip has launches of its own for it.  e,
  * mask and counts8 of each item are as for toric3d_run_cycles.  BP chunks are
  * sized per item so the workspace holds one chunk of every item (rounds are
  * added until it does).

@@ -428,15 +428,6 @@ k_flip_tiled(const __grid_constant__ ItemTable tab)
     });
 }
 
-// Words per tile row of k_flip_tiled: L x Wt <= max_threads, Wt a power of two <= 32
-// and no wider than the batch.
-int tiled_words(int L, int64_t nw, int max_threads)
-{
-    int wt = 32;
-    while (wt > 1 && (L * wt > max_threads || wt / 2 >= nw)) wt /= 2;
-    return wt;
-}
-
 // p-flip in two passes, so that each (site, word) draws one Philox block.
 // The first pass is bound by the Philox arithmetic; at 40 registers six blocks
 // per SM keep the integer pipes busier (2.45 -> 2.27 ms per application at
@@ -1070,6 +1061,16 @@ bool layout_vec(const void* bits, int64_t n_bits) { return n_bits % 4 == 0 && al
 }  // namespace
 
 // ----------------------------------------------------------------- launchers
+// Words per tile row of k_flip_tiled: L x Wt threads at most, Wt a power of two <= 32
+// and no wider than the batch.
+int flip_tile_words(int L, int64_t words, bool wide)
+{
+    const int max_threads = wide ? kFlipThreads : kFlipThreadsSmall;
+    int wt = 32;
+    while (wt > 1 && (L * wt > max_threads || wt / 2 >= words)) wt /= 2;
+    return wt;
+}
+
 t3d_status launch_noise(ItemTable& tab, uint64_t thr, uint64_t seed, uint32_t cycle, cudaStream_t st)
 {
     if (thr == 0) return T3D_OK;
@@ -1109,12 +1110,13 @@ t3d_status launch_sweeps(ItemTable& all, const char* schedule, int slen, int n_a
                          uint64_t seed, uint32_t cycle, cudaStream_t st)
 {
     if (n_apply <= 0) return T3D_OK;
-    // lattices that fit one SM or a cluster run the whole schedule in one launch
-    auto on_chip = [&](const ItemDesc& d) { return !d.stop && sweeps_fit(d.lat.L, d.nw ? d.nw : d.W, n_apply); };
+    // the items whose schedule is faster on chip, each in a launch of its own; the others share the rest
+    // (a flip until clear has chosen already)
+    bool chip[kMaxItems] = {};
+    if (all.n > 0 && !all.it[0].stop) route_sweeps(all, schedule, slen, n_apply, false, chip);
     for (int i = 0; i < all.n; ++i)
-        if (on_chip(all.it[i]))
-            T3D_TRY(launch_column_sweeps(all.it[i], schedule, slen, n_apply, sweep0, seed, cycle, st));
-    ItemTable tab = select_items(all, [&](const ItemDesc& d) { return !on_chip(d); });
+        if (chip[i]) T3D_TRY(launch_column_sweeps(all.it[i], schedule, slen, n_apply, sweep0, seed, cycle, st));
+    ItemTable tab = select_items(all, [&](const ItemDesc& d) { return !chip[&d - all.it]; });
     if (tab.n == 0) return T3D_OK;
     for (int i = 0; i < tab.n; ++i) {
         ItemDesc& d = tab.it[i];
@@ -1139,7 +1141,7 @@ t3d_status launch_sweeps(ItemTable& all, const char* schedule, int slen, int n_a
         ItemDesc& d = tt.it[i];
         const int64_t nw = d.nw ? d.nw : d.W;
         tiled = tiled && d.lat.L * (wide ? 16 : 8) <= max_threads;
-        d.tx = tiled_words(d.lat.L, nw, max_threads);
+        d.tx = flip_tile_words(d.lat.L, nw, wide);
         d.blocks = (int64_t)d.lat.L * ((nw + d.tx - 1) / d.tx);
         d.live_wpu = d.tx;
         d.live_bpu = d.lat.L;   // one z-plane per block, word tiles outermost
@@ -1195,12 +1197,12 @@ t3d_status launch_flip_until_clear(ItemTable& all, int max_sweeps, int32_t* swee
         if (sweeps_done) T3D_CUDA_CHECK(cudaMemsetAsync(sweeps_done, 0, sizeof(int32_t), st));
         return T3D_OK;
     }
-    auto on_chip = [&](const ItemDesc& d) { return sweeps_fit(d.lat.L, d.nw ? d.nw : d.W, max_sweeps); };
+    bool chip[kMaxItems] = {};
+    route_sweeps(all, "F", 1, max_sweeps, true, chip);
     for (int i = 0; i < all.n; ++i)
-        if (on_chip(all.it[i]))
-            T3D_TRY(launch_column_until_clear(all.it[i], max_sweeps, i == 0 ? sweeps_done : nullptr, st));
-    if (all.n > 0 && on_chip(all.it[0])) sweeps_done = nullptr;
-    ItemTable tab = select_items(all, [&](const ItemDesc& d) { return !on_chip(d); });
+        if (chip[i]) T3D_TRY(launch_column_until_clear(all.it[i], max_sweeps, i == 0 ? sweeps_done : nullptr, st));
+    if (chip[0]) sweeps_done = nullptr;
+    ItemTable tab = select_items(all, [&](const ItemDesc& d) { return !chip[&d - all.it]; });
     if (tab.n == 0) return T3D_OK;
     for (int i = 0; i < tab.n; ++i) {
         T3D_REQUIRE(tab.it[i].stop != nullptr, "flip until clear: item %d has no flag words", i);

@@ -463,7 +463,7 @@ struct ColumnView {
 // words read or written per site and application) and, in p-flip, the ALU (the coins).  Measured
 // at L = 32, 10^5 samples, one application of a longer schedule: flip 0.43 ms against 0.83 as a
 // kernel of its own, p-flip 0.83 against 1.46; the columns' way in and out costs 2.2 ms once (see
-// sweeps_fit).  Keeping the syndrome in registers too (17 words, but 96 registers of state that
+// route_schedule).  Keeping the syndrome in registers too (17 words, but 96 registers of state that
 // spill) measured the same, row pairs with shared y-neighbours and prefetched planes slower.
 // Keeps the compiler from computing what follows from v outside the loop over applications: the
 // unrolled sites' shared-memory addresses, kept in registers across it, would push the state
@@ -710,6 +710,8 @@ __global__ void __launch_bounds__(256) k_from_columns(int64_t R, int64_t W, cons
 // that can be resident with about 200 KB each (cudaOccupancyMaxActiveClusters on GB300) and the
 // share of them that a split of L planes into unequal slabs leaves waiting.  A thread takes at
 // most four planes of its row pair (96 registers of state).  cluster 0: none fits.
+constexpr int kResident[kMaxCluster + 1] = {0, 152, 152, 138, 144, 140, 138, 105, 120};   // blocks by cluster size
+
 struct SlabShape {
     int cluster, zt, z, threads;
     size_t smem;
@@ -717,7 +719,6 @@ struct SlabShape {
 
 SlabShape slab_shape(int L)
 {
-    constexpr int resident[kMaxCluster + 1] = {0, 152, 152, 138, 144, 140, 138, 105, 120};
     SlabShape best{0, 0, 0, 0, 0};
     double busy = 0.0;
     const int per = (L + 1) / 2 * L;
@@ -725,7 +726,7 @@ SlabShape slab_shape(int L)
         const int most = (L + c - 1) / c;
         const size_t smem = (size_t)48 * L * L * most;
         if (smem + 1024 > kColumnSmem) continue;
-        const double b = resident[c] * (double)L / (c * most);
+        const double b = kResident[c] * (double)L / (c * most);
         if (b <= busy) continue;
         // planes per thread: 4 with up to 512 threads, 3 with up to 640, 2 with up to 896
         for (int z = std::min(4, most); z >= 1; --z) {
@@ -855,31 +856,227 @@ uint64_t schedule_bits(const char* schedule, int slen)
     return b;
 }
 
-}  // namespace
+// ------------------------------------------------------------------ which form runs
+// A schedule runs on chip (one launch per lattice, its columns in and out once, an application between
+// two barriers) or step by step (one launch per application over all lattices of a batch, every word
+// through L2 or HBM).  Which is faster depends on the lattice, the words, the letters and what else is in
+// the batch, so both are estimated, in microseconds.  The constants are fitted to both forms' times at L = 3
+// .. 32, 1 .. 1,563 words and the schedules F, FF, 8 F, P, 5 P and FFPFF (1,440 sizes; rms of the estimates 10%
+// on chip, 7% step by step).  The form they choose takes 0.3% longer than the faster of the two on
+// average, where step by step always takes 35% longer and on chip up to L = 14, below 64 words or from five
+// applications on 13%.  Examples, step by
+// step / on chip: FFPFF at L = 8, 1,563 words 87 / 50; L = 25, 1,563 words 2,605 / 3,573; L = 32, 1,563 words 5,459 /
+// 5,166, 16 words 189 / 96; P alone at L = 16, 16 words 6 / 35; F alone at L = 28, 48 words 48 / 80.
+constexpr double kSms = 152.0;
+constexpr int64_t kClearTypical = 8;  // flip until clear: applications that do some work
+constexpr double kSkipUs = 2.0;       // ... and what a skipped one costs as a launch
+constexpr double kClearUs = 7.0;      // ... and its flags
 
-bool column_fits(int L) { return column_bytes(L) <= kColumnSmem; }
+struct Letters {
+    int64_t flips, pflips;
+};
 
-// Whether a whole run pays on chip.  A column draws its random words on one SM, about
-// 0.0127 L^3 us a cycle, where the noise and measurement kernels spread them over the chip for three
-// launches (about 12 us) a cycle: with fewer columns than SMs, or a last round of columns that
-// leaves SMs idle, the column waits for itself (one FFPFF cycle, columns / step by step with the
-// schedule on chip: L = 14, 160 words 144 / 127 us, 304 words 144 / 162; L = 12, 160 words 92 / 85, 304
-// words 93 / 108).  From four rounds on the launches and the syndrome's way through memory cost more
-// (L = 14, 700 words 344 / 356).
-bool column_run_pays(int L, int64_t words)
+// The work of a single on-chip launch: rounds of columns and ns-weighted sites per round.
+struct ChipShape {
+    double rounds, ksites;   // columns (clusters' words) one SM takes in turn; thousands of sites of a block
+    double io, flip, pflip;  // us per thousand sites: columns in and out, one application of each kind
+    double each;             // us per application beside that (the cluster's barriers)
+};
+
+bool chip_shape(int L, int64_t words, ChipShape& c)
 {
-    if (!column_fits(L)) return false;
-    const double rounds = words / 152.0, idle = std::ceil(rounds) - rounds;
-    return rounds >= 4.0 || idle * 0.0127 * L * L * L <= 12.0;
+    if (column_bytes(L) <= kColumnSmem) {
+        const int wt = column_shape(L, words).wt;
+        c.rounds = std::ceil(std::ceil((double)words / wt) / kSms);
+        c.ksites = 1e-3 * L * L * L * wt;
+        c.each = 0.0;
+        if (L * L * L <= kColumnThreads) {   // k_column_one
+            c.io = 5.0; c.flip = 0.82; c.pflip = 2.05;
+        } else {                             // k_column
+            c.io = 4.6; c.flip = 1.23; c.pflip = 2.5;
+        }
+    } else {
+        const SlabShape s = slab_shape(L);
+        if (s.cluster == 0) return false;
+        c.rounds = std::ceil((double)words / (kResident[s.cluster] / s.cluster));
+        c.ksites = 1e-3 * L * L * ((L + s.cluster - 1) / s.cluster);
+        c.io = 5.3; c.flip = 0.67; c.pflip = 1.95;
+        c.each = 1.5;
+    }
+    // a row's words share 32-byte sectors, which the column of every word fetches for itself
+    c.io *= std::min(1.0, 0.2 * (double)words);
+    return true;
 }
 
-// Whether a schedule of n_apply applications runs on chip.  Above L = 14 the columns are turned
-// first and back afterwards from kTurnWords words on (about 2.2 ms at L = 32, 10^5 samples, five
-// applications' gain: FFPFF 5.6 -> 4.8 ms, PFFPFF x 32 in 33 -> 20 ms); below that a step by
-// step schedule is bound by its launches.
-bool sweeps_fit(int L, int64_t words, int n_apply)
+constexpr double kLaunchUs = 2.8;
+
+double chip_us(const ChipShape& c, const Letters& n)
 {
-    return column_fits(L) || (slab_shape(L).cluster > 0 && (words < kTurnWords || n_apply >= 5));
+    const double flip = std::max(0.2, c.rounds * (c.each + c.flip * c.ksites)),
+                 pflip = std::max(0.3, c.rounds * (c.each + c.pflip * c.ksites));
+    return kLaunchUs + c.rounds * c.io * c.ksites + n.flips * flip + n.pflips * pflip;
+}
+
+// Whole runs on chip: a column draws a cycle's noise and measurement on one SM, 12 ns a site (at least
+// 3.5 us a cycle), where the noise and measurement kernels spread them over the chip.
+double chip_run_us(const ChipShape& c, int cycles, const Letters& n, int perfect)
+{
+    const Letters all{cycles * n.flips + std::min<int64_t>(std::max(perfect, 0), kClearTypical), cycles * n.pflips};
+    return chip_us(c, all) + cycles * std::max(3.5, 12.0 * c.rounds * c.ksites) +
+           (perfect >= 0 ? 2.5 * c.rounds * c.ksites : 0.0);
+}
+
+int64_t item_words(const ItemDesc& d)
+{
+    // compacted words: the device knows how many there are, usually few
+    return d.live ? std::min<int64_t>(d.W, 16) : (d.nw ? d.nw : d.W);
+}
+
+// The step by step form over the items i of tab with !skip[i]: an application's launch takes a
+// latency that grows with L (the flip's walk along y) beside the blocks' work; an odd number of flips
+// leaves the syndrome in the scratch array and is copied back row by row.
+double steps_us(const ItemTable& tab, const bool* skip, const Letters& n, bool until_clear)
+{
+    int items = 0, maxL = 0;
+    bool wide = true;
+    for (int i = 0; i < tab.n; ++i)
+        if (!skip[i]) {
+            ++items;
+            maxL = std::max(maxL, tab.it[i].lat.L);
+            wide = wide && tab.it[i].lat.L >= 32;
+        }
+    if (items == 0) return 0.0;
+    double work = 0.0, longest = 0.0, blocks = 0.0, waves = 0.0, msites = 0.0, copies = 0.0;
+    for (int i = 0; i < tab.n; ++i) {
+        if (skip[i]) continue;
+        const int L = tab.it[i].lat.L;
+        const int64_t words = item_words(tab.it[i]);
+        const double m = 1e-6 * L * L * L * (double)words;
+        const int wt = flip_tile_words(L, words, wide);
+        const double us = 2.5e-3 * L * L * wt, b = L * std::ceil((double)words / wt);
+        longest = std::max(longest, us);
+        work += us * b / kSms;
+        waves += us * std::ceil(b / kSms);
+        blocks += b;
+        msites += m;
+        // below 65,536 rows the copy takes a time per row
+        copies += 1.1 + (L < 28 ? std::max(1.6e-3 * L * L * L, 24.0 * m) : std::max(0.55e-3 * L * L * L, 13.0 * m));
+    }
+    const double turns = items == 1 ? waves : (blocks <= kSms ? longest : work + 0.5 * longest);
+    const double flip = std::hypot(1.7 + 0.54 * maxL, turns);
+    // up to 1.5 million sites x words p-flip's arrays stay in L2
+    const double pflip = 3.7 + (msites < 1.5 ? 20.0 : 26.0 + 0.5 * std::max(0, maxL - 24)) * msites;
+    double us = 0.8 + n.pflips * pflip + (n.flips & 1 ? copies : 0.0);
+    if (until_clear) {
+        const int64_t run = std::min(n.flips, kClearTypical);
+        us += run * flip + (double)(n.flips - run) * kSkipUs + items * kClearUs;
+    } else {
+        us += n.flips * flip;
+    }
+    return us;
+}
+
+// The fastest of: all items step by step, every item that fits on chip, or those whose time on chip is
+// below what they add to the shared launches.  chip[i] says which; returns the estimate.
+double route_schedule(const ItemTable& tab, const bool* skip, const Letters& n, bool until_clear, bool* chip)
+{
+    const Letters work{until_clear ? std::min(n.flips, kClearTypical) : n.flips, n.pflips};
+    double on[kMaxItems];
+    bool fits[kMaxItems], none[kMaxItems], all[kMaxItems], some[kMaxItems];
+    double us_all = 0.0;
+    for (int i = 0; i < tab.n; ++i) {
+        ChipShape c;
+        fits[i] = !skip[i] && chip_shape(tab.it[i].lat.L, item_words(tab.it[i]), c);
+        on[i] = fits[i] ? chip_us(c, work) : 0.0;
+        none[i] = skip[i];
+        all[i] = skip[i] || fits[i];
+        us_all += on[i];
+    }
+    const double us_none = steps_us(tab, none, n, until_clear);
+    us_all += steps_us(tab, all, n, until_clear);
+    double us_some = 0.0;
+    for (int i = 0; i < tab.n; ++i) some[i] = none[i];
+    for (int i = 0; i < tab.n; ++i) {
+        if (!fits[i]) continue;
+        none[i] = true;   // without this item
+        const bool pays = on[i] < us_none - steps_us(tab, none, n, until_clear);
+        none[i] = skip[i];
+        some[i] = pays;
+        us_some += pays ? on[i] : 0.0;
+    }
+    us_some += steps_us(tab, some, n, until_clear);
+    const bool* best = us_all <= us_none && us_all <= us_some ? all : (us_some < us_none ? some : none);
+    for (int i = 0; i < tab.n; ++i) chip[i] = fits[i] && best[i];
+    return std::min(us_all, std::min(us_none, us_some));
+}
+
+// A run's cycles step by step, its schedules in whichever form is faster.
+double step_run_us(const ItemTable& tab, const bool* skip, int cycles, const Letters& n, int perfect)
+{
+    double msites = 0.0;
+    int items = 0;
+    for (int i = 0; i < tab.n; ++i)
+        if (!skip[i]) {
+            const double L = tab.it[i].lat.L;
+            msites += 1e-6 * L * L * L * (double)tab.it[i].W;
+            ++items;
+        }
+    if (items == 0) return 0.0;
+    bool chip[kMaxItems];
+    double us = cycles * (5.5 + 75.0 * msites);
+    if (n.flips + n.pflips > 0) us += cycles * route_schedule(tab, skip, n, false, chip);
+    if (perfect >= 0) us += 3.0 + 20.0 * msites;
+    if (perfect > 0) us += route_schedule(tab, skip, Letters{perfect, 0}, true, chip);
+    return us;
+}
+
+Letters letters_of(const char* schedule, int slen, int n_apply)
+{
+    Letters n{0, 0};
+    for (int k = 0; k < slen; ++k) {
+        const int times = n_apply / slen + (k < n_apply % slen ? 1 : 0);
+        (schedule[k] == 'P' ? n.pflips : n.flips) += times;
+    }
+    return n;
+}
+
+}  // namespace
+
+void route_sweeps(const ItemTable& tab, const char* schedule, int slen, int n_apply, bool until_clear, bool* chip)
+{
+    const bool skip[kMaxItems] = {};
+    route_schedule(tab, skip, letters_of(schedule, slen, n_apply), until_clear, chip);
+}
+
+void route_run(const ItemTable& tab, int cycles, const char* schedule, int slen, int n_apply, int perfect, bool* whole)
+{
+    const Letters n = letters_of(schedule, slen, n_apply);
+    double on[kMaxItems];
+    bool fits[kMaxItems], some[kMaxItems];
+    const bool none[kMaxItems] = {};
+    double us_all = 0.0;
+    for (int i = 0; i < tab.n; ++i) {
+        const int L = tab.it[i].lat.L;
+        ChipShape c;
+        fits[i] = column_bytes(L) <= kColumnSmem && chip_shape(L, tab.it[i].W, c);
+        on[i] = fits[i] ? chip_run_us(c, cycles, n, perfect) : 0.0;
+        us_all += on[i];
+    }
+    const double us_none = step_run_us(tab, none, cycles, n, perfect);
+    us_all += step_run_us(tab, fits, cycles, n, perfect);
+    double us_some = 0.0;
+    bool without[kMaxItems] = {};
+    for (int i = 0; i < tab.n; ++i) {
+        some[i] = false;
+        if (!fits[i]) continue;
+        without[i] = true;
+        some[i] = on[i] < us_none - step_run_us(tab, without, cycles, n, perfect);
+        without[i] = false;
+        us_some += some[i] ? on[i] : 0.0;
+    }
+    us_some += step_run_us(tab, some, cycles, n, perfect);
+    const bool* best = us_all <= us_none && us_all <= us_some ? fits : (us_some < us_none ? some : none);
+    for (int i = 0; i < tab.n; ++i) whole[i] = best[i];
 }
 
 t3d_status launch_column_sweeps(const ItemDesc& d, const char* schedule, int slen, int n_apply, uint32_t sweep0,
@@ -894,7 +1091,7 @@ t3d_status launch_column_sweeps(const ItemDesc& d, const char* schedule, int sle
     pr.sweep0 = sweep0;
     pr.cycle0 = cycle;
     const int kind = pr.sched ? T3D_K_PFLIP : T3D_K_FLIP;
-    return column_fits(d.lat.L) ? launch_column<false>(d, pr, kind, st) : launch_slab(d, pr, kind, st);
+    return column_bytes(d.lat.L) <= kColumnSmem ? launch_column<false>(d, pr, kind, st) : launch_slab(d, pr, kind, st);
 }
 
 t3d_status launch_column_until_clear(const ItemDesc& d, int max_sweeps, int32_t* sweeps_done, cudaStream_t st)
@@ -906,7 +1103,7 @@ t3d_status launch_column_until_clear(const ItemDesc& d, int max_sweeps, int32_t*
     pr.n_apply = max_sweeps;
     pr.until_clear = 1;
     pr.sweeps_done = sweeps_done;
-    return column_fits(d.lat.L) ? launch_column<false>(d, pr, T3D_K_FLIP, st) : launch_slab(d, pr, T3D_K_FLIP, st);
+    return column_bytes(d.lat.L) <= kColumnSmem ? launch_column<false>(d, pr, T3D_K_FLIP, st) : launch_slab(d, pr, T3D_K_FLIP, st);
 }
 
 t3d_status launch_column_run(const ItemDesc& d, int cycles, uint32_t cycle0, uint64_t thr_p, uint64_t thr_q,

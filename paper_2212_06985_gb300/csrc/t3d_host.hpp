@@ -120,12 +120,17 @@ t3d_status launch_flip_until_clear(ItemTable& tab, int max_sweeps, int32_t* swee
 t3d_status launch_sweeps(ItemTable& tab, const char* schedule, int slen, int n_apply,
                          uint32_t sweep0, uint64_t seed, uint32_t cycle, cudaStream_t st);
 t3d_status launch_logical(ItemTable& tab, cudaStream_t st);
-// Lattices whose syndrome and flip words fit one SM or a cluster of them (t3d_column.cu): a
-// schedule, a flip until clear, or a whole run in one launch per item.  No scratch (ItemDesc::tmp, stop) is used.
+// Lattices whose syndrome and flip words fit one SM or a cluster of them (L <= 32, t3d_column.cu): a
+// schedule, a flip until clear, or (L <= 14) a whole run on chip, in launches of the item's own.  From L = 15 and
+// 64 words on, without live words or a word range, the item's tmp is overwritten and its s array holds flips
+// meanwhile (launch_slab); ItemDesc::stop is not used.
 struct ItemDesc;
-bool column_fits(int L);   // one SM, error words included (L <= 14)
-bool column_run_pays(int L, int64_t words);           // whole runs
-bool sweeps_fit(int L, int64_t words, int n_apply);   // schedules and flip until clear (L <= 32)
+// chip[i]: whether item i's schedule (until_clear: up to n_apply flips) is faster on chip than in the batch's
+// shared launches; whole[i]: the same for a whole run (perfect: the noiseless round's most applications, -1 none).
+void route_sweeps(const ItemTable& tab, const char* schedule, int slen, int n_apply, bool until_clear, bool* chip);
+void route_run(const ItemTable& tab, int cycles, const char* schedule, int slen, int n_apply, int perfect, bool* whole);
+// Words of a tile row of the step by step flip; wide: every lattice of the launch has L >= 32.
+int flip_tile_words(int L, int64_t words, bool wide);
 t3d_status launch_column_sweeps(const ItemDesc& d, const char* schedule, int slen, int n_apply, uint32_t sweep0,
                                 uint64_t seed, uint32_t cycle, cudaStream_t st);
 t3d_status launch_column_until_clear(const ItemDesc& d, int max_sweeps, int32_t* sweeps_done, cudaStream_t st);

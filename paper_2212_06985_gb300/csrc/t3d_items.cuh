@@ -1,8 +1,9 @@
 // Work items for persistent multi-lattice launches.
 //
 // A batch holds up to kMaxItems independent ensembles, each with its own
-// lattice size L, sample count and buffers.  Every kernel of a run is launched
-// once per step for the whole batch: the item table travels by value in the
+// lattice size L, sample count and buffers.  A kernel of a run is launched
+// once per step for the whole batch (schedules and runs kept on chip, an item at a
+// time: t3d_column.cu): the item table travels by value in the
 // kernel parameters, each item needs `blocks` thread blocks of work, and a
 // persistent grid (a multiple of the SM count) walks the concatenated block
 // ranges with a grid-stride loop, so uneven lattices share one launch and no

@@ -1,8 +1,10 @@
 // Whole Monte Carlo runs: T code cycles of noise, noisy measurement and
 // decoding (Sec. 3.1 Fig. 2, Sec. 3.2 schedules, Sec. 4.2 p-BP), an optional
 // noiseless final round, and the logical readout.  A run covers a batch of up
-// to eight ensembles of different lattice sizes; every step is one persistent
-// launch over all of them (t3d_items.cuh).  The whole T-cycle sequence can be
+// to eight ensembles of different lattice sizes; a step is one launch over all
+// of them (t3d_items.cuh), except that lattices up to L = 14 may run whole and
+// lattices up to L = 32 their schedules on chip, a launch each, where that is
+// estimated to be faster (t3d_column.cu).  The whole T-cycle sequence can be
 // captured into a CUDA graph, instantiated once per distinct run and replayed.
 #include <cuda_runtime.h>
 
@@ -343,18 +345,17 @@ t3d_status enqueue_run(const t3d_run_cfg& c, const Plan& pl, cudaStream_t st)
     const uint64_t thr_p = prob_threshold(c.p), thr_q = prob_threshold(c.q);
     const int slen = (int)strnlen(c.schedule, sizeof(c.schedule));
     ItemTable tab;
-    // flip / p-flip runs of lattices that fit one SM: all cycles and the noiseless round in one
-    // launch per item; the other items (`items`) go step by step
-    const bool columns = !learned(c) && !c.use_bp;
-    auto stepwise = [&](const ItemDesc& d) { return !columns || !column_run_pays(d.lat.L, d.W); };
-    if (columns) {
-        if (c.T > 0 || c.perfect_round)
-            for (int i = 0; i < pl.items.n; ++i)
-                if (!stepwise(pl.items.it[i]))
-                    T3D_TRY(launch_column_run(pl.items.it[i], c.T, c.cycle0, thr_p, thr_q, c.seed, c.schedule, slen,
-                                              c.n_apply, c.perfect_round ? c.perfect_max_sweeps : -1, st));
-    }
-    const ItemTable items = select_items(pl.items, stepwise);
+    // flip / p-flip runs of lattices that fit one SM, where that is faster: all cycles and the noiseless
+    // round in one launch per item; the other items (`items`) go step by step
+    const int perfect = c.perfect_round ? c.perfect_max_sweeps : -1;
+    bool whole[kMaxItems] = {};
+    if (!learned(c) && !c.use_bp && (c.T > 0 || c.perfect_round))
+        route_run(pl.items, c.T, c.schedule, slen, c.n_apply, perfect, whole);
+    for (int i = 0; i < pl.items.n; ++i)
+        if (whole[i])
+            T3D_TRY(launch_column_run(pl.items.it[i], c.T, c.cycle0, thr_p, thr_q, c.seed, c.schedule, slen, c.n_apply,
+                                      perfect, st));
+    const ItemTable items = select_items(pl.items, [&](const ItemDesc& d) { return !whole[&d - pl.items.it]; });
     for (int t = 1; t <= c.T && items.n > 0; ++t) {
         const uint32_t cycle = c.cycle0 + (uint32_t)t;
         if (learned(c)) {
@@ -390,7 +391,7 @@ t3d_status enqueue_run(const t3d_run_cfg& c, const Plan& pl, cudaStream_t st)
             // perfect_max_sweeps applications)
             ItemTable flagged = pl.items;
             for (int i = 0; i < flagged.n; ++i) flagged.it[i].stop = pl.stop[i];
-            tab = select_items(flagged, stepwise);
+            tab = select_items(flagged, [&](const ItemDesc& d) { return !whole[&d - flagged.it]; });
             T3D_TRY(launch_flip_until_clear(tab, c.perfect_max_sweeps, nullptr, st));
         }
     }
