@@ -458,9 +458,10 @@ t3d_status toric3d_run_cycles(const t3d_run_cfg* cfg, uint64_t* e, void* work, s
  * toric3d_cnn_train_step: one Adam step (lr > 0) of mean binary cross-entropy
  * between the logits and the labels e_label (bit-sliced, the error before
  * decoding) on this batch; params, adam_m, adam_v (device FP32) are updated in
- * place and blob re-prepared; grads_out (nullable, FP32 [param_count])
- * receives the gradient; loss_out (device float) the summed loss.  lr = 0
- * computes gradient and loss only.  work: toric3d_cnn_train_workspace_bytes.
+ * place and blob, here only 4-byte aligned, re-prepared; grads_out (nullable,
+ * FP32 [param_count]) receives the gradient; loss_out (device float) the summed
+ * loss.  lr = 0 computes gradient and loss only.  work:
+ * toric3d_cnn_train_workspace_bytes.
  */
 int toric3d_cnn_param_count(void);
 size_t toric3d_cnn_blob_bytes(void);

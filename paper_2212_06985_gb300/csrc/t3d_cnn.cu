@@ -247,6 +247,7 @@ extern "C" t3d_status toric3d_cnn_train_step(int L, int64_t n_samples, const uin
     T3D_TRY(check_words(s, "s"));
     T3D_TRY(check_words(e_label, "e_label"));
     T3D_REQUIRE(params && adam_m && adam_v && blob && loss_out, "params, adam state, blob and loss_out are required");
+    T3D_REQUIRE(aligned(blob, 4), "blob must be 4-byte aligned");
     T3D_REQUIRE(step >= 1, "Adam step counts from 1");
     T3D_REQUIRE(work != nullptr && aligned(work, 256), "work must be 256-byte aligned");
     T3D_REQUIRE(work_bytes >= toric3d_cnn_train_workspace_bytes(L, n_samples), "workspace too small");

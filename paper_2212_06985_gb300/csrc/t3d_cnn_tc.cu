@@ -526,6 +526,8 @@ __global__ void __launch_bounds__(conv_threads(kMode), 1) k_conv_col(const __gri
     // channels, 16 bytes each.  (Element by element with the search inside a launch took 30 us longer: a
     // decode of L = 12, 2,048 samples 281 us, now 192.)
     int* s_k = reinterpret_cast<int*>(sm);   // [block][chunk]
+    // training takes weights that are only 4-byte aligned
+    const bool wide_w = (reinterpret_cast<uintptr_t>(a.w) & 15) == 0;
     {
         const ColPos last = s_pos[4 * P - 1];
         const int n_blocks = last.base + (4 - last.lo) + 4 + (last.hi + 1);
@@ -550,7 +552,15 @@ __global__ void __launch_bounds__(conv_threads(kMode), 1) k_conv_col(const __gri
             const int blk = i >> 5, c = (i >> 3) & 1, co = (i >> 1 & 8) | (i & 7);   // in the order of the layout
             const int k = s_k[2 * blk + c];
             uint4 w = make_uint4(0u, 0u, 0u, 0u);
-            if (k >= 0) w = __ldg(reinterpret_cast<const uint4*>(a.w + k + co * kC));
+            if (k >= 0) {
+                const __nv_bfloat16* row = a.w + k + co * kC;
+                if (wide_w) {
+                    w = __ldg(reinterpret_cast<const uint4*>(row));
+                } else {
+                    const uint32_t* r = reinterpret_cast<const uint32_t*>(row);
+                    w = make_uint4(__ldg(r), __ldg(r + 1), __ldg(r + 2), __ldg(r + 3));
+                }
+            }
             reinterpret_cast<uint4*>(sm + kColOffW)[i] = w;
         }
     }
