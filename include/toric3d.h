@@ -206,8 +206,9 @@ size_t toric3d_bp_workspace_bytes(int L, int64_t chunk_samples);
  * Local BP decoder (Sec. 4.1): `iters` flooding iterations from the priors,
  * then the hard decision applied to e and s.  Samples are processed in chunks
  * of whole 64-sample words, as large as the workspace allows (at least one
- * word must fit; see toric3d_bp_workspace_bytes).  llr_out as for
- * toric3d_bp_decide; it needs a workspace for the whole batch.
+ * word must fit; see toric3d_bp_workspace_bytes).  work: 32-byte aligned device
+ * scratch.  llr_out as for toric3d_bp_decide; it needs a workspace for the whole
+ * batch.
  */
 t3d_status toric3d_bp(int L, int64_t n_samples, uint64_t* e, uint64_t* s, double p,
                       double q_meas, int iters, void* work, size_t work_bytes, float* llr_out,

@@ -719,7 +719,9 @@ extern "C" t3d_status toric3d_bp(int L, int64_t n_samples, uint64_t* e, uint64_t
     T3D_TRY(check_words(e, "e"));
     T3D_TRY(check_words(s, "s"));
     T3D_REQUIRE(iters >= 0, "iters must be >= 0");
-    T3D_REQUIRE(work != nullptr && aligned(work, 16), "work must be a 16-byte aligned device pointer");
+    // the syndrome copy behind the message buffers (whole multiples of 32 bytes) moves in 32-byte records; two
+    // 16-byte accesses each would take any 16-byte address, but an iteration 0.4 to 1% longer at L = 14 .. 24
+    T3D_REQUIRE(work != nullptr && aligned(work, 32), "work must be a 32-byte aligned device pointer");
     int64_t chunk = (int64_t)(work_bytes / bp_bytes_per_word(L));
     const int64_t G = words_for(n_samples);
     T3D_REQUIRE(chunk >= 1, "workspace too small: %zu bytes, need at least %zu", work_bytes,
