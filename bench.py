@@ -43,7 +43,7 @@ VALUE_IS = "BP+p-flip; learned_pflip.value = learned+p-flip, learned_pflip.vs_bp
 # first launch of a chunk does the first two iterations and reads only syndrome words.
 # Set to None when the kernel changes until it is captured again.
 BP_STEP_TRAFFIC = {"first_two_iterations": 15.67, "full_iteration": 31.93}
-# The same for k_flip_tiled (schedules taken step by step: lattices above L = 32, short schedules)
+# The same for k_flip_tiled (schedules taken step by step: lattices above L = 32, and where that is faster)
 # inside the FFPFF cycle at p = q = 4% (L = 32, 8192 samples, the four flip applications of one
 # cycle: 322.4 MB of DRAM traffic each on average, per qubit-sample 0.400 B against the dense
 # 0.5 B: e is touched only where a word has a flipped lane, so the figure depends on the noise
@@ -361,15 +361,17 @@ def sweep_roofline(prof, w, qubits, S, steps, ms, hbm_peak, peak_source, clk):
     kinds = {k: prof[k] for k in SWEEP_BYTES if prof[k][1]}
     unit_bytes = SWEEP_BYTES
     sweep_launches = prof["flip"][1] + prof["pflip"][1]
-    if sweep_launches < (per_step["flip"] + 2 * n_p) * steps:
-        # fewer launches than steps: the whole schedule ran on chip (all of it under one kind)
+    # a p-flip application is recorded as one launch (its two passes together); fewer records than applications, or
+    # none of one of the schedule's letters: the whole schedule ran on chip, under one kind
+    letters = {"flip": per_step["flip"], "pflip": n_p}
+    if sweep_launches < w.n_apply * steps or any(letters[k] and not prof[k][1] for k in letters):
         per_step = {"noise": 1, "syndrome": 1, "schedule": 1}
         unit_bytes = {"noise": SWEEP_BYTES["noise"], "syndrome": SWEEP_BYTES["syndrome"], "schedule": SCHEDULE_BYTES}
         kinds = {k: prof[k] for k in ("noise", "syndrome") if prof[k][1]}
         kinds["schedule"] = (prof["flip"][0] + prof["pflip"][0], sweep_launches)
     dom = max(kinds, key=lambda k: kinds[k][0])
     d_ms, d_launches = kinds[dom]
-    apps = per_step[dom] * steps                      # applications (a p-flip one is two launches)
+    apps = per_step[dom] * steps                      # applications
     t_app = d_ms / apps / 1e3
     words = (S + 63) // 64
     cycle_bytes = sum(unit_bytes[k] * per_step[k] for k in unit_bytes) * qubits * S * steps
