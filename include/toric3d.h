@@ -251,8 +251,8 @@ t3d_status toric3d_bp_meta(int L, int64_t n_samples, uint64_t* e, uint64_t* s, d
  * along the face's normal (upper face) -> that variable.  msg_out gets every
  * check -> variable message computed from msg_in (all zero: the first
  * iteration); the buffers must not overlap; toric3d_bp_meta_message_bytes
- * gives their size and work (16-byte aligned device scratch for the edge
- * totals) needs a seventh of it.
+ * gives their size and work (16-byte aligned device scratch, checked but not
+ * used) needs a seventh of it.
  */
 size_t toric3d_bp_meta_message_bytes(int L, int64_t n_samples);
 t3d_status toric3d_bp_meta_step(int L, int64_t n_samples, const uint64_t* s, double p, double q,
@@ -540,8 +540,11 @@ t3d_status toric3d_autotune_batch(const t3d_run_cfg* cfg, const t3d_batch_item* 
  * kernel the library enqueues outside a stream capture is bracketed by a pair
  * of CUDA events on its own stream.  toric3d_profile_read() waits for the
  * recorded events and returns, for one kernel kind, the summed device time in
- * milliseconds and the number of launches; toric3d_profile_reset() forgets
- * them.  Host-side state is global to the process; do not toggle it while
+ * milliseconds and the number of launches (records: a p-flip application's two
+ * passes are one); toric3d_profile_reset() forgets them.  On chip a schedule
+ * counts as T3D_K_PFLIP if it has a 'P' and as T3D_K_FLIP otherwise, one record or
+ * (L >= 15, 64 words or more) three, and a whole run, noise and measurement
+ * included, as one of T3D_K_FLIP.  Host-side state is global to the process; do not toggle it while
  * another thread is enqueuing toric3d work.
  */
 typedef enum {

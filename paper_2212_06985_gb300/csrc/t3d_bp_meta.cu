@@ -268,7 +268,9 @@ Args make_args(const Lattice& lat, int64_t S, int64_t W, const uint64_t* s, doub
 size_t floats_per_sample(int L)
 {
     const size_t n = 3ull * L * L * L;
-    return n /* T */ + 2 * 7 * n /* F, Fm, Cl, Ch x2 */;
+    // two sets of messages, and a plane that nothing reads (the edge totals of a three-kernel iteration): the
+    // size that callers ask for, and the smaller ones refused, stay as they were
+    return n + 2 * 7 * n /* F, Fm, Cl, Ch x2 */;
 }
 
 }  // namespace

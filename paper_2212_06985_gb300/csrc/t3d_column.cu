@@ -414,8 +414,8 @@ k_column_one(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnP
 // of a thread-block cluster, each keeping its slab's syndrome and flip words in shared memory.
 // The two phases of an application read one word per (x, y) column from the neighbouring block
 // (distributed shared memory): the syndrome below the slab, the flips above it; a cluster barrier
-// separates them.  The flips that reach e are gathered in registers, kK sites a thread, and XORed
-// into e once at the end.
+// separates them.  The flips that reach e are gathered in registers, up to 2 kZ sites a thread,
+// and XORed into e once at the end.
 __device__ __forceinline__ void cluster_barrier()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -458,13 +458,6 @@ struct ColumnView {
     __device__ __forceinline__ uint64_t& at(int64_t r, int64_t w) const { return p[r * row + w * word]; }
 };
 
-// Thread (x, j) of z-part zp owns the sites of rows j and j + ceil(L / 2), z0 <= z < z1 (at most
-// kZ planes); the z-neighbours are words it has just read.  Bound by the shared-memory pipe (23
-// words read or written per site and application) and, in p-flip, the ALU (the coins).  Measured
-// at L = 32, 10^5 samples, one application of a longer schedule: flip 0.43 ms against 0.83 as a
-// kernel of its own, p-flip 0.83 against 1.46; the columns' way in and out costs 2.2 ms once (see
-// route_schedule).  Keeping the syndrome in registers too (17 words, but 96 registers of state that
-// spill) measured the same, row pairs with shared y-neighbours and prefetched planes slower.
 // Keeps the compiler from computing what follows from v outside the loop over applications: the
 // unrolled sites' shared-memory addresses, kept in registers across it, would push the state
 // itself into local memory.
@@ -474,6 +467,13 @@ __device__ __forceinline__ int here(int v)
     return v;
 }
 
+// Thread (x, j) of z-part zp owns the sites of rows j and j + ceil(L / 2), z0 <= z < z1 (at most
+// kZ planes); the z-neighbours are words it has just read.  Bound by the shared-memory pipe (23
+// words read or written per site and application) and, in p-flip, the ALU (the coins).  Measured
+// at L = 32, 10^5 samples, one application of a longer schedule: flip 0.43 ms against 0.83 as a
+// kernel of its own, p-flip 0.83 against 1.46; the columns' way in and out costs 2.2 ms once (see
+// route_schedule).  Keeping the syndrome in registers too (17 words, but 96 registers of state, which
+// spill) measured the same, row pairs with shared y-neighbours and prefetched planes slower.
 template <int kZ, int kT>
 __global__ void __launch_bounds__(kT, 1)
 k_slab(const __grid_constant__ ItemDesc d, const __grid_constant__ ColumnProgram pr, int C, const ColumnView sv,
@@ -706,12 +706,13 @@ __global__ void __launch_bounds__(256) k_from_columns(int64_t R, int64_t W, cons
         if (r0 + ty + i < R && w0 + tx < W) out[(r0 + ty + i) * W + w0 + tx] = was[i / 8] ^ tile[tx][ty + i];
 }
 
+// Resident blocks by cluster size.
+constexpr int kResident[kMaxCluster + 1] = {0, 152, 152, 138, 144, 140, 138, 105, 120};
+
 // Blocks of a cluster for lattice size L: the choice with the most busy SMs, counting the blocks
 // that can be resident with about 200 KB each (cudaOccupancyMaxActiveClusters on GB300) and the
 // share of them that a split of L planes into unequal slabs leaves waiting.  A thread takes at
-// most four planes of its row pair (96 registers of state).  cluster 0: none fits.
-constexpr int kResident[kMaxCluster + 1] = {0, 152, 152, 138, 144, 140, 138, 105, 120};   // blocks by cluster size
-
+// most four planes of its row pair (24 words of flips, 48 registers).  cluster 0: none fits.
 struct SlabShape {
     int cluster, zt, z, threads;
     size_t smem;
