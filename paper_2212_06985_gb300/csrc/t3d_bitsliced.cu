@@ -166,6 +166,31 @@ k_syndrome(const __grid_constant__ ItemTable tab, uint64_t thr, uint64_t seed, u
     });
 }
 
+// The same with a face a thread, for launches that leave SMs idle: a thread's time is then a launch's, and three
+// draws one after the other took 4.1 - 4.4 us where one takes 2.6 (L = 8, 1,000 samples).
+__global__ void __launch_bounds__(kThreads)
+k_syndrome_faces(const __grid_constant__ ItemTable tab, uint64_t thr, uint64_t seed, uint32_t cycle)
+{
+    for_each_item_block(tab, [&](const ItemDesc& d, int64_t lb) {
+        const Lattice lat = d.lat;
+        int f;
+        int64_t w;
+        if (!tile_site_word(d, lb, 3 * lat.L3, f, w)) return;
+        const int n = (f >= lat.L3) + (f >= 2 * lat.L3), site = f - n * lat.L3;
+        const int64_t W = d.W;
+        const Coord r = site_coord(lat, site);
+        const int L = lat.L;
+        const int dx = r.x[0] + 1 == L ? 1 - L : 1, dy = r.x[1] + 1 == L ? L - lat.L2 : L,
+                  dz = r.x[2] + 1 == L ? lat.L2 - lat.L3 : lat.L2;
+        const int a = n == 0 ? 1 : 0, b = n == 2 ? 1 : 2;   // the face's axes
+        const int da = a == 0 ? dx : dy, db = b == 1 ? dy : dz;
+        const uint64_t* __restrict__ pa = d.e + ((int64_t)a * lat.L3 + site) * W + w;
+        const uint64_t* __restrict__ pb = d.e + ((int64_t)b * lat.L3 + site) * W + w;
+        const uint64_t s = pa[0] ^ pa[db * W] ^ pb[0] ^ pb[da * W];
+        d.s[(int64_t)f * W + w] = s ^ bernoulli_word(thr, seed, kStreamMeas, (uint64_t)f, cycle, 0, d.group0 + w);
+    });
+}
+
 // Periodic neighbour offsets of a site: step[a] and the +1 / -1 moves along
 // each axis expressed as index deltas.
 struct Moves {
@@ -1092,16 +1117,32 @@ t3d_status launch_noise(ItemTable& tab, uint64_t thr, uint64_t seed, uint32_t cy
 t3d_status launch_syndrome(ItemTable& tab, uint64_t thr, uint64_t seed, uint32_t cycle, cudaStream_t st)
 {
     const int per = sites_per_thread(tab, 1);
+    int64_t blocks = 0;   // with a site a thread
     for (int i = 0; i < tab.n; ++i) {
         ItemDesc& d = tab.it[i];
         const int64_t nw = d.nw ? d.nw : d.W;
         d.tx = row_words(nw);
+        blocks += tile_blocks(d.lat.L3, nw, d.tx);
         T3D_TRY(tile_blocks_checked(d, d.lat.L3, nw, d.tx, &d.blocks, per));
     }
+    // a face a thread up to about 1.5 blocks of sites an SM (before / after, one site a thread: 32 blocks 4.4 / 2.6
+    // us, 160 5.4 / 4.6, 216 5.4 / 5.1; from 256 blocks on 5.6 / 5.9)
+    const bool faces = blocks < 240;
+    if (faces)
+        for (int i = 0; i < tab.n; ++i) {
+            ItemDesc& d = tab.it[i];
+            d.blocks = tile_blocks(3LL * d.lat.L3, d.nw ? d.nw : d.W, d.tx);
+        }
     finish_table(tab);
     ProfScope prof(T3D_K_SYNDROME, st);
-    k_syndrome<<<persistent_grid((const void*)k_syndrome, kThreads, T3D_K_SYNDROME, tab.prefix[tab.n], has_live(tab)),
-                 kThreads, 0, st>>>(tab, thr, seed, cycle, per);
+    if (faces)
+        k_syndrome_faces<<<persistent_grid((const void*)k_syndrome_faces, kThreads, T3D_K_SYNDROME, tab.prefix[tab.n],
+                                           has_live(tab)),
+                           kThreads, 0, st>>>(tab, thr, seed, cycle);
+    else
+        k_syndrome<<<persistent_grid((const void*)k_syndrome, kThreads, T3D_K_SYNDROME, tab.prefix[tab.n],
+                                     has_live(tab)),
+                     kThreads, 0, st>>>(tab, thr, seed, cycle, per);
     T3D_LAUNCH_CHECK("syndrome");
     return T3D_OK;
 }
