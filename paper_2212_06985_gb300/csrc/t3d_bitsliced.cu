@@ -1018,6 +1018,8 @@ k_unpack(int64_t n_bits, int64_t n_samples, int64_t W, const uint64_t* __restric
 {
     __shared__ __align__(16) uint64_t tile[kLayoutWords * kLayoutPitch];
     const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5, tw = blockDim.x >> 5;
+    // this block's share of a word's samples, in eighths
+    const int g0 = 8 * blockIdx.y / gridDim.y, g1 = 8 * (blockIdx.y + 1) / gridDim.y;
     for (int64_t b = blockIdx.x; b < tiles; b += gridDim.x) {
         const int64_t wt = b / col_tiles, c0 = (b - wt * col_tiles) * kLayoutCols;
         for (int i = threadIdx.x; i < kLayoutCols * tw; i += blockDim.x) {
@@ -1037,6 +1039,7 @@ k_unpack(int64_t n_bits, int64_t n_samples, int64_t W, const uint64_t* __restric
         uint8_t* __restrict__ p = bits + s0 * n_bits + c0 + layout_col<kVec>(lane, 0);
 #pragma unroll
         for (int g = 0; g < 8; ++g) {
+            if (g < g0 || g >= g1) continue;
             // byte g of the four columns' words side by side: bit j of each byte is sample 8 g + j
             const uint32_t pair = (uint32_t)((g & 3) | ((4 + (g & 3)) << 4));
             uint32_t h[4];
@@ -1061,6 +1064,20 @@ k_unpack(int64_t n_bits, int64_t n_samples, int64_t W, const uint64_t* __restric
     }
 }
 
+// Unpacking a few bytes, a thread each: nothing waits for shared memory or for another sample's store.
+// Up to so many bytes, and while all samples share one word (whose rows are then read once) somewhat more.
+constexpr int64_t kUnpackBytes = 400000, kUnpackWordBytes = 1000000;
+
+__global__ void __launch_bounds__(kThreads)
+k_unpack_bytes(int64_t n_bits, int64_t n_samples, int64_t W, const uint64_t* __restrict__ words,
+               uint8_t* __restrict__ bits)
+{
+    const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    if (i >= n_bits * n_samples) return;
+    const int64_t sample = i / n_bits, c = i - sample * n_bits;
+    bits[i] = (uint8_t)((words[c * W + (sample >> 6)] >> (sample & 63)) & 1ULL);
+}
+
 // Grid of the layout kernels: words per block (a warp each), column tiles, tiles in all.
 struct LayoutGrid {
     int threads;
@@ -1078,6 +1095,17 @@ LayoutGrid layout_grid(int64_t n_bits, int64_t W)
     g.tiles = g.col_tiles * ((W + tw - 1) / tw);
     g.blocks = (unsigned)std::min<int64_t>(g.tiles, 0x7fffffffLL);
     return g;
+}
+
+// Unpacking writes a word's 64 samples one after the other, 3.6 - 5.9 us however few the words are.  Where
+// the tiles leave SMs idle they are split over up to eight blocks by samples (L = 6, 1,024 samples 5.9 ->
+// 3.8 us), and a few bytes go a thread each (L = 4, 256 samples 3.8 us, 3.1 split by samples, 1.8 so; L = 4, 2,048
+// samples, 393 KB, 3.3 so and 3.6 split; L = 6, 1,024 samples, 663 KB, 4.6 and 3.8; one word of L = 14 2.6 and 3.6).
+unsigned unpack_parts(const LayoutGrid& g)
+{
+    unsigned parts = 8;
+    while (parts > 1 && g.tiles * parts > 152) parts /= 2;
+    return parts;
 }
 
 // Four bytes of a row at a time: every sample's row starts 4-byte aligned.
@@ -1600,12 +1628,16 @@ extern "C" t3d_status toric3d_unpack(int64_t n_bits, int64_t n_samples, const ui
     T3D_TRY(check_words(words, "words"));
     int64_t W = words_for(n_samples);
     const LayoutGrid g = layout_grid(n_bits, W);
+    const dim3 grid(g.blocks, unpack_parts(g));
     cudaStream_t st = as_stream(stream);
     ProfScope prof(T3D_K_LAYOUT, st);
-    if (layout_vec(bits, n_bits))
-        k_unpack<true><<<g.blocks, g.threads, 0, st>>>(n_bits, n_samples, W, words, bits, g.col_tiles, g.tiles);
+    if (n_bits <= (W == 1 ? kUnpackWordBytes : kUnpackBytes) / n_samples)
+        k_unpack_bytes<<<(unsigned)((n_bits * n_samples + kThreads - 1) / kThreads), kThreads, 0, st>>>(n_bits, n_samples, W,
+                                                                                                    words, bits);
+    else if (layout_vec(bits, n_bits))
+        k_unpack<true><<<grid, g.threads, 0, st>>>(n_bits, n_samples, W, words, bits, g.col_tiles, g.tiles);
     else
-        k_unpack<false><<<g.blocks, g.threads, 0, st>>>(n_bits, n_samples, W, words, bits, g.col_tiles, g.tiles);
+        k_unpack<false><<<grid, g.threads, 0, st>>>(n_bits, n_samples, W, words, bits, g.col_tiles, g.tiles);
     T3D_LAUNCH_CHECK("unpack");
     return T3D_OK;
 }
