@@ -370,16 +370,19 @@ __global__ void __launch_bounds__(kIterThreads, 16) k_tg_iteration(const BpArgs 
 }
 
 // Posterior decision of variable v for 32 samples per ballot: T_v = prior_v + the messages into v
-// (a.in nullptr: every message is zero), d = [T_v < 0] into the decision words (as e's layout),
-// e ^= d; optional posteriors.
+// (a.in nullptr: every message is zero), or with kTotals as k_tg_totals left it; d = [T_v < 0] into the decision
+// words (as e's layout), e ^= d; optional posteriors.  The graphs of k_tg_iteration, with at most four messages,
+// sum them here; for the others (up to 32 messages behind an index each) the totals pass with its four
+// samples a thread is faster: 12,000 variables of degree 6, 2,000 samples, one iteration 650 us against 751.
+template <bool kTotals>
 __global__ void __launch_bounds__(kThreads) k_tg_decide_bp(const BpArgs a, int64_t n_valid, uint64_t* __restrict__ e,
                                                             uint64_t* __restrict__ d, int64_t dW,
                                                             float* __restrict__ llr, int64_t llr_stride)
 {
     const int64_t smp = (int64_t)blockIdx.y * kThreads + threadIdx.x, v = blockIdx.x;
     if (smp >= a.S) return;   // S is a multiple of 64: whole warps
-    float l = a.prior[v];
-    if (a.in)
+    float l = kTotals ? a.T[v * a.S + smp] : a.prior[v];
+    if (!kTotals && a.in)
         for (int32_t k = a.g.vptr[v]; k < a.g.vptr[v + 1]; ++k) l += __ldcs(&a.in[(int64_t)a.g.vedge[k] * a.S + smp]);
     const bool valid = smp < n_valid;
     const uint32_t bits = __ballot_sync(0xffffffffu, valid && l < 0.0f);
@@ -717,7 +720,13 @@ extern "C" t3d_status toric3d_tanner_bp(const t3d_tanner* g, int64_t n_samples, 
             T3D_TRY(launch_bp_iteration(a, one, one && it == 0 ? nullptr : M[it & 1], M[(it + 1) & 1], st));
         a.in = iters ? M[iters & 1] : nullptr;
         ProfScope prof(T3D_K_BP_DECIDE, st);
-        k_tg_decide_bp<<<dim3((unsigned)g->n_vars, (unsigned)((S + kThreads - 1) / kThreads)), kThreads, 0, st>>>(
+        const bool totals = !one && iters > 0;
+        if (totals) {
+            k_tg_totals<<<dim3((unsigned)g->n_vars, quad_blocks(S)), quad_threads(S), 0, st>>>(a);
+            T3D_LAUNCH_CHECK("Tanner BP posteriors");
+        }
+        auto decide = totals ? k_tg_decide_bp<true> : k_tg_decide_bp<false>;
+        decide<<<dim3((unsigned)g->n_vars, (unsigned)((S + kThreads - 1) / kThreads)), kThreads, 0, st>>>(
             a, std::min<int64_t>(S, n_samples - 64 * w0), e + w0, d, cw, llr_out, n_samples);
         T3D_LAUNCH_CHECK("Tanner BP decisions");
         k_tg_apply<<<bs_grid(g->n_checks, cw), bs_block(cw), 0, st>>>(gv, cw, s + w0, W, d, cw);
