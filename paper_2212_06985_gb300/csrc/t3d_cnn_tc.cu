@@ -526,8 +526,6 @@ __global__ void __launch_bounds__(conv_threads(kMode), 1) k_conv_col(const __gri
     // channels, 16 bytes each.  (Element by element with the search inside a launch took 30 us longer: a
     // decode of L = 12, 2,048 samples 281 us, now 192.)
     int* s_k = reinterpret_cast<int*>(sm);   // [block][chunk]
-    // training takes weights that are only 4-byte aligned
-    const bool wide_w = (reinterpret_cast<uintptr_t>(a.w) & 15) == 0;
     {
         const ColPos last = s_pos[4 * P - 1];
         const int n_blocks = last.base + (4 - last.lo) + 4 + (last.hi + 1);
@@ -547,21 +545,23 @@ __global__ void __launch_bounds__(conv_threads(kMode), 1) k_conv_col(const __gri
             s_k[i] = in_reach ? ((dz + 1) * 9 + (dy + 1) * 3 + (dx + 1)) * kC * kC + (kBitsIn ? 0 : c * 8) : -1;
         }
         __syncthreads();
+        auto windows = [&](auto&& row_of) {
 #pragma unroll 4
-        for (int i = threadIdx.x; i < n_blocks * 32; i += blockDim.x) {
-            const int blk = i >> 5, c = (i >> 3) & 1, co = (i >> 1 & 8) | (i & 7);   // in the order of the layout
-            const int k = s_k[2 * blk + c];
-            uint4 w = make_uint4(0u, 0u, 0u, 0u);
-            if (k >= 0) {
-                const __nv_bfloat16* row = a.w + k + co * kC;
-                if (wide_w) {
-                    w = __ldg(reinterpret_cast<const uint4*>(row));
-                } else {
-                    const uint32_t* r = reinterpret_cast<const uint32_t*>(row);
-                    w = make_uint4(__ldg(r), __ldg(r + 1), __ldg(r + 2), __ldg(r + 3));
-                }
+            for (int i = threadIdx.x; i < n_blocks * 32; i += blockDim.x) {
+                const int blk = i >> 5, c = (i >> 3) & 1, co = (i >> 1 & 8) | (i & 7);   // in the order of the layout
+                const int k = s_k[2 * blk + c];
+                uint4 w = make_uint4(0u, 0u, 0u, 0u);
+                if (k >= 0) w = row_of(a.w + k + co * kC);
+                reinterpret_cast<uint4*>(sm + kColOffW)[i] = w;
             }
-            reinterpret_cast<uint4*>(sm + kColOffW)[i] = w;
+        };
+        if ((reinterpret_cast<uintptr_t>(a.w) & 15) == 0) {
+            windows([](const __nv_bfloat16* p) { return __ldg(reinterpret_cast<const uint4*>(p)); });
+        } else {   // training takes weights that are only 4-byte aligned
+            windows([](const __nv_bfloat16* p) {
+                const uint32_t* r = reinterpret_cast<const uint32_t*>(p);
+                return make_uint4(__ldg(r), __ldg(r + 1), __ldg(r + 2), __ldg(r + 3));
+            });
         }
     }
     fence_proxy_async_smem();
