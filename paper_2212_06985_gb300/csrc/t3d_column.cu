@@ -863,12 +863,13 @@ uint64_t schedule_bits(const char* schedule, int slen)
 // through L2 or HBM).  Which is faster depends on the lattice, the words, the letters and what else is in
 // the batch, so both are estimated, in microseconds.  The constants are fitted to both forms' times at L = 3
 // .. 32, 1 .. 1,563 words and the schedules F, FF, 8 F, P, 5 P and FFPFF (1,440 sizes; rms of the estimates 10%
-// on chip, 7% step by step).  The form they choose takes 0.3% longer than the faster of the two on
+// on chip, 7% step by step).  The form they choose takes 0.25% longer than the faster of the two on
 // average, where step by step always takes 35% longer and on chip up to L = 14, below 64 words or from five
 // applications on 13%.  Examples, step by
 // step / on chip: FFPFF at L = 8, 1,563 words 87 / 50; L = 25, 1,563 words 2,605 / 3,573; L = 32, 1,563 words 5,459 /
 // 5,166, 16 words 189 / 96; P alone at L = 16, 16 words 6 / 35; F alone at L = 28, 48 words 48 / 80.
 constexpr double kSms = 152.0;
+constexpr double kL2Msites = 1.5;     // millions of sites x words whose arrays stay in L2
 constexpr int64_t kClearTypical = 8;  // flip until clear: applications that do some work
 constexpr double kSkipUs = 2.0;       // ... and what a skipped one costs as a launch
 constexpr double kClearUs = 7.0;      // ... and its flags
@@ -894,15 +895,17 @@ bool chip_shape(int L, int64_t words, ChipShape& c)
         if (L * L * L <= kColumnThreads) {   // k_column_one
             c.io = 5.0; c.flip = 0.82; c.pflip = 2.05;
         } else {                             // k_column
-            c.io = 4.6; c.flip = 1.23; c.pflip = 2.5;
+            c.io = c.rounds > 1.0 ? 4.6 : 6.0; c.flip = 1.23; c.pflip = 2.5;
         }
     } else {
         const SlabShape s = slab_shape(L);
         if (s.cluster == 0) return false;
         c.rounds = std::ceil((double)words / (kResident[s.cluster] / s.cluster));
         c.ksites = 1e-3 * L * L * ((L + s.cluster - 1) / s.cluster);
-        c.io = 5.3; c.flip = 0.67; c.pflip = 1.95;
-        c.each = 1.5;
+        // turned columns are cheap while their four arrays stay in L2
+        c.io = words < kTurnWords ? 5.0 : (kL2Msites > 1e-6 * L * L * L * (double)words ? 4.4 : 5.6);
+        c.flip = 0.8; c.pflip = 1.9;
+        c.each = 1.0;
     }
     // a row's words share 32-byte sectors, which the column of every word fetches for itself
     c.io *= std::min(1.0, 0.2 * (double)words);
@@ -965,8 +968,7 @@ double steps_us(const ItemTable& tab, const bool* skip, const Letters& n, bool u
     }
     const double turns = items == 1 ? waves : (blocks <= kSms ? longest : work + 0.5 * longest);
     const double flip = std::hypot(1.7 + 0.54 * maxL, turns);
-    // up to 1.5 million sites x words p-flip's arrays stay in L2
-    const double pflip = 3.7 + (msites < 1.5 ? 20.0 : 26.0 + 0.5 * std::max(0, maxL - 24)) * msites;
+    const double pflip = 3.7 + (msites < kL2Msites ? 20.0 : 26.0 + 0.5 * std::max(0, maxL - 24)) * msites;
     double us = 0.8 + n.pflips * pflip + (n.flips & 1 ? copies : 0.0);
     if (until_clear) {
         const int64_t run = std::min(n.flips, kClearTypical);
