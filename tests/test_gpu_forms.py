@@ -68,7 +68,7 @@ def test_turned_columns_match_oracle(L, W):
     assert sum(check_schedule(L, W, schedule, 7, pflip(L, schedule, 7))) == 3
 
 
-@pytest.mark.parametrize("L,W", [(15, 64), (17, 66), (23, 67), (31, 66)])
+@pytest.mark.parametrize("L,W", [(15, 64), (17, 66), (23, 67), (26, 66), (31, 66)])   # clusters of 1, 2, 4, 7, 8
 @pytest.mark.parametrize("p,most", [(0.002, 40), (0.05, 11)])   # clears early (L = 31 keeps a stuck pair); does not
 def test_until_clear_with_turned_columns_matches_oracle(L, W, p, most):
     e, s = noisy(L, W, p, 0.0)
